@@ -27,6 +27,12 @@ constexpr int kRsSlices = 32;        // slices per chunk of the row-staged kerne
 // infeasibility direction; FP32 iterations therefore test rays at
 // max(infeas_tol, kFp32RayTol).
 constexpr double kFp32RayTol = 1e-6;
+constexpr int kGroup = 4;        // slices per aligned group of one width
+constexpr int kRunBits = 26;     // bits of a column index in the second word of a column run
+// low bits of SellView::soff, one value per group of slices
+constexpr int kRunsNone = 0;     // explicit column indices
+constexpr int kRunsTwo = 1;      // every k-column is one or two runs
+constexpr int kRunsOne = 2;      // every k-column is one run
 constexpr int kTraceCheckCols = 12;  // values recorded per KKT check in the trace
 
 // Sliced ELL with 32-row slices over the internal (length-sorted) row order.
@@ -40,7 +46,20 @@ struct SellView {
   const T* val;        // [nnz_pad]
   int32_t nslices;
   int32_t rows;        // logical rows (<= 32 * nslices)
+  // Column runs.  soff[s] is off[s] with, in its low bits, kRunsOne (kRunsTwo)
+  // where every k-column of the slice's group is one run (at most two runs) of
+  // consecutive column indices over the lanes; runs[off/32 + k] then replaces the
+  // 128 B of indices by 8 B: lanes below `split` gather x + lane, the others
+  // y + lane - split, with y in the low kRunBits bits of the second word and split
+  // above them.
+  const int32_t* soff;  // [nslices + 1]
+  const int2* runs;     // [nnz_pad / 32]
 };
+
+__device__ __forceinline__ int run_col(int2 r, int lane) {
+  const int split = (int)((unsigned)r.y >> kRunBits);
+  return lane < split ? r.x + lane : (r.y & ((1 << kRunBits) - 1)) + lane - split;
+}
 
 // Device-resident solver state: every scalar decision of the PDHG loop lives
 // here, so the loop never waits on the host.

@@ -22,8 +22,10 @@ struct DevSell {
   int32_t nchunks = 0;        // 0: a slice exceeds kStageEntries (no staged kernels)
   int32_t* chunks2 = nullptr;  // chunks of the row-staged kernels
   int32_t nchunks2 = 0;
-  SellView<double> v64() const { return {off, col, val64, nslices, rows}; }
-  SellView<float> v32() const { return {off, col, val32, nslices, rows}; }
+  int32_t* soff = nullptr;  // column runs (SellView)
+  int32_t* runs = nullptr;
+  SellView<double> v64() const { return {off, col, val64, nslices, rows, soff, (const int2*)runs}; }
+  SellView<float> v32() const { return {off, col, val32, nslices, rows, soff, (const int2*)runs}; }
 };
 
 // Iterate buffers of one precision.
@@ -47,10 +49,12 @@ struct HostLayout {
   std::vector<int32_t> perm_row, perm_col;  // internal -> original
   std::vector<int32_t> k_off, k_col, k_src;
   std::vector<int32_t> t_off, t_col, t_src;
+  std::vector<int32_t> k_soff, k_runs, t_soff, t_runs;  // column runs (SellView)
 };
 
 int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& row_ptr,
-                 const std::vector<int32_t>& col, HostLayout* out, std::string* err);
+                 const std::vector<int32_t>& col, const std::vector<double>& val, HostLayout* out,
+                 std::string* err);
 
 // Per-round initialisation of the device state.
 struct RoundInit {

@@ -32,9 +32,10 @@ static int fail(int code, const std::string& msg) {
 template <class P>
 static cudaError_t dalloc(Workspace* w, P** p, size_t count) {
   void* q = nullptr;
-  // lengths rounded up to whole 32-row slices: the row-staged kernels copy the
-  // operand rows of whole slices
-  count = (count + 31) / 32 * 32;
+  // lengths rounded up to whole groups of slices: the per-attempt kernels read
+  // the operand rows of whole groups
+  constexpr size_t kRows = kSlice * kGroup;
+  count = (count + kRows - 1) / kRows * kRows;
   cudaError_t e = cudaMalloc(&q, count * sizeof(P) + 16);
   if (e == cudaSuccess) {
     w->allocs.push_back(q);
@@ -659,9 +660,12 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   // structure to the host
   std::vector<int64_t> rp(w->m + 1);
   std::vector<int32_t> col(w->nnz);
+  std::vector<double> val(w->nnz);  // guides the internal order only; solves read the values afresh
   if (cudaMemcpyAsync(rp.data(), prob->row_ptr, sizeof(int64_t) * (w->m + 1), cudaMemcpyDeviceToHost,
                       s) != cudaSuccess ||
       (w->nnz > 0 && cudaMemcpyAsync(col.data(), prob->col, sizeof(int32_t) * w->nnz,
+                                     cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+      (w->nnz > 0 && cudaMemcpyAsync(val.data(), prob->val, sizeof(double) * w->nnz,
                                      cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return bail(fail(PDHG_ERR_CUDA, "copying the CSR structure to the host failed"));
@@ -670,7 +674,7 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
     if (rp[i + 1] < rp[i]) return bail(fail(PDHG_ERR_INVALID_ARG, "row_ptr not monotone"));
   HostLayout L;
   std::string err;
-  rc = build_layout(w->n, w->m, w->m_eq, rp, col, &L, &err);
+  rc = build_layout(w->n, w->m, w->m_eq, rp, col, val, &L, &err);
   if (rc != PDHG_OK) return bail(fail(rc, err));
   auto up = [&](int32_t** dst, const std::vector<int32_t>& v) -> int {
     cudaError_t e = dalloc(w, dst, v.size() + 1);
@@ -701,7 +705,8 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   }
   if (up(&w->perm_row, L.perm_row) || up(&w->perm_col, L.perm_col) || up(&w->K.off, L.k_off) ||
       up(&w->K.col, L.k_col) || up(&w->K.src, L.k_src) || up(&w->KT.off, L.t_off) ||
-      up(&w->KT.col, L.t_col) || up(&w->KT.src, L.t_src))
+      up(&w->KT.col, L.t_col) || up(&w->KT.src, L.t_src) || up(&w->K.soff, L.k_soff) ||
+      up(&w->K.runs, L.k_runs) || up(&w->KT.soff, L.t_soff) || up(&w->KT.runs, L.t_runs))
     return bail(fail(PDHG_ERR_NOMEM, "device allocation/upload of the layout failed"));
   {
     int r2 = PDHG_OK;

@@ -18,101 +18,97 @@
 
 namespace ucpdhg {
 
-// Row dot products of U consecutive slices (lane = row within each slice)
-// with x.  Entries are consumed in predicated chunks of 4 per slice, so every
-// column/value load of the U short rows (UC rows have 2-25 entries) is in
-// flight before the dependent gathers of x.  U > 1 raises the bytes in flight
-// per warp; the autotuner picks U per matrix.
-// Slice offsets off[s0 .. s0+U] (clamped past the end, giving empty slices).
-// The per-attempt kernels load the NEXT group's offsets one iteration ahead,
-// so this L2 round trip is off the critical path.
+// Row dot products of U consecutive slices (U = 1, or 2 or 4 slices of one group:
+// one width w) with x1 and, if TWO, with x2 in the same matrix pass; lane = row
+// within each slice.  The columns of a slice come from its runs (8 B per 32
+// entries: the gather is then one or two contiguous pieces and needs no index
+// load of its own) or, where it has none, from the explicit indices.
+//
+// What bounds these sweeps is not DRAM but the instructions and dependent round
+// trips per 32 rows (the time per row is the same for a matrix that stays in L2),
+// so a warp takes U slices whose entries and operand rows lie at fixed distances:
+// loads without predicates or address arithmetic of their own, U E entries and
+// 4 U (5 U) operands in flight before the dependent gathers.
+//
+// soff[s0] and soff[s0 + U] (clamped past the end, giving empty slices).  The
+// per-attempt kernels load the NEXT group's offsets one iteration ahead, so this
+// L2 round trip is off the critical path.
+struct SliceSpan {
+  int o, w, mode;  // first slot, entries per row, kRuns*
+};
 template <class T, int U>
-__device__ __forceinline__ void slice_offsets(const SellView<T>& A, int s0, int (&ob)[U + 1]) {
-#pragma unroll
-  for (int u = 0; u <= U; ++u) ob[u] = __ldg(A.off + min(s0 + u, A.nslices));
+__device__ __forceinline__ int2 slice_offsets(const SellView<T>& A, int s0) {
+  return make_int2(__ldg(A.soff + min(s0, A.nslices)), __ldg(A.soff + min(s0 + U, A.nslices)));
+}
+template <int U>
+__device__ __forceinline__ SliceSpan slice_span(int2 ob) {
+  return {ob.x & ~(kSlice - 1), ((ob.y >> 5) - (ob.x >> 5)) / U, ob.x & (kSlice - 1)};
 }
 
-template <class T, int U>
-__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, const int (&ob)[U + 1], int lane,
-                                             const T* __restrict__ x, T (&acc)[U]) {
-  int o0[U], w[U];
-  int wmax = 0;
+template <class T, int U, int E, int MODE, bool TWO, bool TAIL>
+__device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan& g, int k0, int lane,
+                                          const T* __restrict__ x1, const T* __restrict__ x2,
+                                          T (&acc1)[U], T (&acc2)[U]) {
+  int c[U][E];
+  T v[U][E];
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    o0[u] = ob[u] + lane;
-    w[u] = (ob[u + 1] - ob[u]) >> 5;
-    wmax = max(wmax, w[u]);
-    acc[u] = 0;
-  }
-  for (int k0 = 0; k0 < wmax; k0 += 4) {
-    int c[U][4];
-    T v[U][4];
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int e = 0; e < E; ++e) {
+      const bool ok = !TAIL || k0 + e < g.w;
+      const int slot = g.o + (u * g.w + k0 + e) * kSlice;
+      if (MODE == kRunsOne)
+        c[u][e] = ok ? __ldg(&A.runs[slot >> 5].x) + lane : 0;
+      else if (MODE == kRunsTwo)
+        c[u][e] = ok ? run_col(__ldg(A.runs + (slot >> 5)), lane) : 0;
+      else
+        c[u][e] = ok ? __ldg(A.col + slot + lane) : 0;
+      v[u][e] = ok ? __ldg(A.val + slot + lane) : (T)0;
+    }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const bool ok = k0 + e < w[u];
-        c[u][e] = ok ? __ldg(A.col + o0[u] + (k0 + e) * kSlice) : 0;
-        v[u][e] = ok ? __ldg(A.val + o0[u] + (k0 + e) * kSlice) : (T)0;
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (!TAIL || k0 + e < g.w) {
+        acc1[u] += v[u][e] * __ldg(x1 + c[u][e]);
+        if (TWO) acc2[u] += v[u][e] * __ldg(x2 + c[u][e]);
       }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (k0 + e < w[u]) acc[u] += v[u][e] * __ldg(x + c[u][e]);
-  }
 }
 
-// Two row products at once, K x1 and K x2, sharing the matrix stream (the
-// second gather hits L2: the iterate vectors are a few MB).
-template <class T, int U>
-__device__ __forceinline__ void sell_dot2_pre(const SellView<T>& A, const int (&ob)[U + 1], int lane,
+template <class T, int U, int MODE, bool TWO>
+__device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceSpan& g, int k0, int lane,
                                               const T* __restrict__ x1, const T* __restrict__ x2,
                                               T (&acc1)[U], T (&acc2)[U]) {
-  int o0[U], w[U];
-  int wmax = 0;
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    o0[u] = ob[u] + lane;
-    w[u] = (ob[u + 1] - ob[u]) >> 5;
-    wmax = max(wmax, w[u]);
-    acc1[u] = 0;
-    acc2[u] = 0;
-  }
-  for (int k0 = 0; k0 < wmax; k0 += 4) {
-    int c[U][4];
-    T v[U][4];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const bool ok = k0 + e < w[u];
-        c[u][e] = ok ? __ldg(A.col + o0[u] + (k0 + e) * kSlice) : 0;
-        v[u][e] = ok ? __ldg(A.val + o0[u] + (k0 + e) * kSlice) : (T)0;
-      }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (k0 + e < w[u]) {
-          acc1[u] += v[u][e] * __ldg(x1 + c[u][e]);
-          acc2[u] += v[u][e] * __ldg(x2 + c[u][e]);
-        }
+  if constexpr (U == 1) {
+    if (g.w - k0 <= 2)
+      dot_chunk<T, U, 2, MODE, TWO, true>(A, g, k0, lane, x1, x2, acc1, acc2);
+    else
+      for (; k0 < g.w; k0 += 4) dot_chunk<T, U, 4, MODE, TWO, true>(A, g, k0, lane, x1, x2, acc1, acc2);
+  } else {
+    for (; k0 + 2 <= g.w; k0 += 2) dot_chunk<T, U, 2, MODE, TWO, false>(A, g, k0, lane, x1, x2, acc1, acc2);
+    if (k0 < g.w) dot_chunk<T, U, 1, MODE, TWO, false>(A, g, k0, lane, x1, x2, acc1, acc2);
   }
 }
 
-template <class T, int U>
-__device__ __forceinline__ void sell_dot_multi(const SellView<T>& A, int s0, int lane,
-                                               const T* __restrict__ x, T (&acc)[U]) {
-  int ob[U + 1];
-  slice_offsets<T, U>(A, s0, ob);
-  sell_dot_pre<T, U>(A, ob, lane, x, acc);
+template <class T, int U, bool TWO>
+__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int2 ob, int lane,
+                                             const T* __restrict__ x1, const T* __restrict__ x2,
+                                             T (&acc1)[U], T (&acc2)[U]) {
+  const SliceSpan g = slice_span<U>(ob);
+#pragma unroll
+  for (int u = 0; u < U; ++u) acc1[u] = acc2[u] = 0;
+  if (g.mode == kRunsOne)
+    sell_dot_mode<T, U, kRunsOne, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
+  else if (g.mode == kRunsTwo)
+    sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
+  else
+    sell_dot_mode<T, U, kRunsNone, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
 }
 
 template <class T>
 __device__ __forceinline__ T sell_dot(const SellView<T>& A, int s, int lane, const T* __restrict__ x) {
-  T acc[1];
-  sell_dot_multi<T, 1>(A, s, lane, x, acc);
+  T acc[1], unused[1];
+  sell_dot_pre<T, 1, false>(A, slice_offsets<T, 1>(A, s), lane, x, x, acc, unused);
   return acc[0];
 }
 
@@ -122,8 +118,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
-  int ob[U + 1];
-  slice_offsets<T, U>(a.K, gw * U, ob);  // matrix only: before the previous kernel ends
+  int2 ob = slice_offsets<T, U>(a.K, gw * U);  // matrix only: before the previous kernel ends
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ DualScalars<T> sc;
@@ -142,40 +137,34 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   // throughput on this GPU is ~1/60 of FP32); the step rule is a heuristic
   T acc_dy2 = 0, acc_int = 0;
   for (int s0 = gw * U; s0 < a.K.nslices; s0 += nw * U) {
-    int nb[U + 1];
-    slice_offsets<T, U>(a.K, s0 + nw * U, nb);  // next group, one iteration ahead
+    const int2 nb = slice_offsets<T, U>(a.K, s0 + nw * U);  // next group, one iteration ahead
+    const int i0 = s0 * kSlice + lane;
     // row operands do not depend on the product: load them first so their
-    // latency overlaps the matrix stream
+    // latency overlaps the matrix stream (vectors are allocated in whole groups)
     T yo[U], qi[U], lo[U], yb[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = (s0 + u) * kSlice + lane;
-      yo[u] = qi[u] = lo[u] = yb[u] = 0;
-      if (i < a.m) {
-        yo[u] = yc[i];
-        qi[u] = a.q[i];
-        if (i >= a.m_eq) lo[u] = dual_floor(a.ylo, i, a.m_eq);
-        if (has_pw) yb[u] = a.ybar[i];
-      }
+      const int i = i0 + u * kSlice;
+      yo[u] = yc[i];
+      qi[u] = a.q[i];
+      lo[u] = a.ylo ? a.ylo[i] : (T)0;
+      yb[u] = has_pw ? a.ybar[i] : (T)0;
     }
     // FP32: K x' and K x in one pass (K x recomputed: an L2 gather instead of
     // a stream read and write of m values).  FP64: K x' only, K x read.
     T kx[U], ko[U];
     if constexpr (StoresKx<T>::value) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = (s0 + u) * kSlice + lane;
-        ko[u] = i < a.m ? a.Kx[p][i] : (T)0;
-      }
-      sell_dot_pre<T, U>(a.K, ob, lane, xn, kx);
+      for (int u = 0; u < U; ++u) ko[u] = a.Kx[p][i0 + u * kSlice];
+      T unused[U];
+      sell_dot_pre<T, U, false>(a.K, ob, lane, xn, xn, kx, unused);
     } else {
-      sell_dot2_pre<T, U>(a.K, ob, lane, xn, xc, kx, ko);
+      sell_dot_pre<T, U, true>(a.K, ob, lane, xn, xc, kx, ko);
     }
-#pragma unroll
-    for (int u = 0; u <= U; ++u) ob[u] = nb[u];
+    ob = nb;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = (s0 + u) * kSlice + lane;
+      const int i = i0 + u * kSlice;
       if (i < a.m) {
         T t = qi[u] - (T)2 * kx[u];
         t = t + ko[u];
@@ -208,8 +197,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
-  int ob[U + 1];
-  slice_offsets<T, U>(a.KT, gw * U, ob);  // matrix only: before the previous kernel ends
+  int2 ob = slice_offsets<T, U>(a.KT, gw * U);  // matrix only: before the previous kernel ends
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ AdjScalars<T> sc;
@@ -227,30 +215,29 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
   T* __restrict__ xn = a.x[1 - p];
   T acc_dx2 = 0;
   for (int s0 = gw * U; s0 < a.KT.nslices; s0 += nw * U) {
-    int nb[U + 1];
-    if (acc_last) slice_offsets<T, U>(a.KT, s0 + nw * U, nb);  // one iteration ahead
+    const int2 nb = slice_offsets<T, U>(a.KT, s0 + nw * U);  // one iteration ahead
+    const int j0 = s0 * kSlice + lane;
     T x0[U], cj[U], lj[U], uj[U], xb[U], g[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = (s0 + u) * kSlice + lane;
-      x0[u] = cj[u] = lj[u] = uj[u] = xb[u] = g[u] = 0;
-      if (j < a.n) {
-        x0[u] = xc[j];
-        cj[u] = a.c[j];
-        lj[u] = a.l[j];
-        uj[u] = a.u[j];
-        if (upd_avg) xb[u] = a.xbar[j];
-        if (!acc_last) g[u] = kty[j];
-      }
+      const int j = j0 + u * kSlice;
+      x0[u] = xc[j];
+      cj[u] = a.c[j];
+      lj[u] = a.l[j];
+      uj[u] = a.u[j];
+      xb[u] = upd_avg ? a.xbar[j] : (T)0;
     }
     if (acc_last) {
-      sell_dot_pre<T, U>(a.KT, ob, lane, yc, g);
+      T unused[U];
+      sell_dot_pre<T, U, false>(a.KT, ob, lane, yc, yc, g, unused);
+    } else {
 #pragma unroll
-      for (int u = 0; u <= U; ++u) ob[u] = nb[u];
+      for (int u = 0; u < U; ++u) g[u] = kty[j0 + u * kSlice];
     }
+    ob = nb;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = (s0 + u) * kSlice + lane;
+      const int j = j0 + u * kSlice;
       if (j < a.n) {
         if (acc_last) kty[j] = g[u];
         if (upd_avg) a.xbar[j] = xb[u] + wlT * x0[u];
@@ -284,55 +271,43 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
 
 constexpr int kStage = 4;
 
+// Explicit column indices here: the runs' second word would take four more
+// registers of the two stages (spills at 48 registers: 75 against 50 us for K x').
 template <class T>
 struct SliceStage {
-  int o0, w;          // first slot of this lane, entries per row
+  SliceSpan g;
   int c[kStage];
   T v[kStage];
 };
 
 template <class T>
-__device__ __forceinline__ void stage_slice(const SellView<T>& A, int ob, int oe, int lane,
-                                            SliceStage<T>& g) {
-  g.o0 = ob + lane;
-  g.w = (oe - ob) >> 5;
+__device__ __forceinline__ void stage_slice(const SellView<T>& A, int2 ob, int lane, SliceStage<T>& st) {
+  st.g = slice_span<1>(ob);
+  const int o = st.g.o + lane, w = st.g.w;
 #pragma unroll
   for (int e = 0; e < kStage; ++e) {
-    const bool ok = e < g.w;
-    g.c[e] = ok ? __ldg(A.col + g.o0 + e * kSlice) : 0;
-    g.v[e] = ok ? __ldg(A.val + g.o0 + e * kSlice) : (T)0;
+    const bool ok = e < w;
+    st.c[e] = ok ? __ldg(A.col + o + e * kSlice) : 0;
+    st.v[e] = ok ? __ldg(A.val + o + e * kSlice) : (T)0;
   }
 }
 
 // Row products of a staged slice with x1 and (if TWO) x2.
 template <class T, bool TWO>
-__device__ __forceinline__ void staged_dot(const SellView<T>& A, const SliceStage<T>& g,
+__device__ __forceinline__ void staged_dot(const SellView<T>& A, const SliceStage<T>& st, int lane,
                                            const T* __restrict__ x1, const T* __restrict__ x2,
                                            T& acc1, T& acc2) {
-  acc1 = 0;
-  acc2 = 0;
+  T a1[1] = {0}, a2[1] = {0};
 #pragma unroll
   for (int e = 0; e < kStage; ++e)
-    if (e < g.w) {
-      acc1 += g.v[e] * __ldg(x1 + g.c[e]);
-      if (TWO) acc2 += g.v[e] * __ldg(x2 + g.c[e]);
+    if (e < st.g.w) {
+      a1[0] += st.v[e] * __ldg(x1 + st.c[e]);
+      if (TWO) a2[0] += st.v[e] * __ldg(x2 + st.c[e]);
     }
-  for (int k0 = kStage; k0 < g.w; k0 += 4) {
-    int c[4];
-    T v[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const bool ok = k0 + e < g.w;
-      c[e] = ok ? __ldg(A.col + g.o0 + (k0 + e) * kSlice) : 0;
-      v[e] = ok ? __ldg(A.val + g.o0 + (k0 + e) * kSlice) : (T)0;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (k0 + e < g.w) {
-        acc1 += v[e] * __ldg(x1 + c[e]);
-        if (TWO) acc2 += v[e] * __ldg(x2 + c[e]);
-      }
-  }
+  for (int k0 = kStage; k0 < st.g.w; k0 += 4)
+    dot_chunk<T, 1, 4, kRunsNone, TWO, true>(A, st.g, k0, lane, x1, x2, a1, a2);
+  acc1 = a1[0];
+  acc2 = a2[0];
 }
 
 template <class T, int MINB>
@@ -345,11 +320,8 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual_pipe(IterArgs<T> a) {
   // matrix only before the previous kernel ends: the warp's first slice
   // (entries) and the offsets of its second
   SliceStage<T> cur;
-  {
-    const int s = min(gw, ns);
-    stage_slice<T>(a.K, __ldg(a.K.off + s), __ldg(a.K.off + min(s + 1, ns)), lane, cur);
-  }
-  int nb0 = __ldg(a.K.off + min(gw + nw, ns)), nb1 = __ldg(a.K.off + min(gw + nw + 1, ns));
+  stage_slice<T>(a.K, slice_offsets<T, 1>(a.K, gw), lane, cur);
+  int2 nb = slice_offsets<T, 1>(a.K, gw + nw);
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ DualScalars<T> sc;
@@ -383,17 +355,16 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual_pipe(IterArgs<T> a) {
     // next slice: entries and row operands; offsets two slices ahead
     SliceStage<T> nxt;
     T yo2, qi2, lo2, yb2, kxo2;
-    stage_slice<T>(a.K, nb0, nb1, lane, nxt);
+    stage_slice<T>(a.K, nb, lane, nxt);
     row_ops(s + nw, yo2, qi2, lo2, yb2, kxo2);
-    nb0 = __ldg(a.K.off + min(s + 2 * nw, ns));
-    nb1 = __ldg(a.K.off + min(s + 2 * nw + 1, ns));
+    nb = slice_offsets<T, 1>(a.K, s + 2 * nw);
     T kx, ko;
     if constexpr (kStored) {
       T unused;
-      staged_dot<T, false>(a.K, cur, xn, xn, kx, unused);
+      staged_dot<T, false>(a.K, cur, lane, xn, xn, kx, unused);
       ko = kxo;
     } else {
-      staged_dot<T, true>(a.K, cur, xn, xc, kx, ko);
+      staged_dot<T, true>(a.K, cur, lane, xn, xc, kx, ko);
     }
     const int i = s * kSlice + lane;
     if (i < a.m) {
@@ -436,11 +407,8 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint_pipe(IterArgs<T> a) {
   // matrix only before the previous kernel ends (used only if the step it
   // decides is accepted)
   SliceStage<T> cur;
-  {
-    const int s = min(gw, ns);
-    stage_slice<T>(a.KT, __ldg(a.KT.off + s), __ldg(a.KT.off + min(s + 1, ns)), lane, cur);
-  }
-  int nb0 = __ldg(a.KT.off + min(gw + nw, ns)), nb1 = __ldg(a.KT.off + min(gw + nw + 1, ns));
+  stage_slice<T>(a.KT, slice_offsets<T, 1>(a.KT, gw), lane, cur);
+  int2 nb = slice_offsets<T, 1>(a.KT, gw + nw);
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ AdjScalars<T> sc;
@@ -473,17 +441,16 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint_pipe(IterArgs<T> a) {
   col_ops(gw, x0, cj, lj, uj, xb, g);
   for (int s = gw; s < ns; s += nw) {
     SliceStage<T> nxt;
-    nxt.w = 0;
+    nxt.g.w = 0;
     T x2, c2, l2, u2, b2, g2;
     if (acc_last) {
-      stage_slice<T>(a.KT, nb0, nb1, lane, nxt);
-      nb0 = __ldg(a.KT.off + min(s + 2 * nw, ns));
-      nb1 = __ldg(a.KT.off + min(s + 2 * nw + 1, ns));
+      stage_slice<T>(a.KT, nb, lane, nxt);
+      nb = slice_offsets<T, 1>(a.KT, s + 2 * nw);
     }
     col_ops(s + nw, x2, c2, l2, u2, b2, g2);
     if (acc_last) {
       T unused;
-      staged_dot<T, false>(a.KT, cur, yc, yc, g, unused);
+      staged_dot<T, false>(a.KT, cur, lane, yc, yc, g, unused);
     }
     const int j = s * kSlice + lane;
     if (j < a.n) {

@@ -1,11 +1,12 @@
 // Internal layout (length-sorted orderings, sliced ELL) and the rescaling pass.
 //
 // Rows of K are reordered by decreasing length inside the equality block and
-// inside the inequality block (stable), columns by decreasing column count, so
-// that each 32-row slice holds rows of (nearly) equal length and padding stays
-// negligible on the UC sparsity (rows of 2 to ~25 entries).  K and K^T are both
-// kept in this layout; every vector the iterations touch lives in the internal
-// order, so no permutation is applied inside the PDHG loop.
+// inside the inequality block, columns by decreasing column count, so that each
+// 32-row slice holds rows of (nearly) equal length and padding stays negligible
+// on the UC sparsity (rows of 2 to ~25 entries); rows (columns) of one length are
+// grouped so that a slice's gathers are contiguous (order_by_signature).  K and
+// K^T are both kept in this layout; every vector the iterations touch lives in
+// the internal order, so no permutation is applied inside the PDHG loop.
 //
 // Rescaling (the PDLP preconditioning of Applegate et al., cited in Sec. II.E):
 // Ruiz l_inf passes r_i = 1/sqrt(max_j |K~_ij|), s_j = 1/sqrt(max_i |K~_ij|),
@@ -13,16 +14,135 @@
 // taken from the same K~.  The factors accumulate in Dr, Dc and the matrix is
 // formed once at the end as K~_ij = K_ij (Dr_i Dc_j).
 #include <algorithm>
+#include <cstring>
 #include <numeric>
 
 #include "internal.cuh"
 
 namespace ucpdhg {
 
+namespace {
+
+// Finalizer of a 64-bit hash (the multiply-xorshift of SplitMix64).
+inline uint64_t mix64(uint64_t z) {
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
+  return z ^ (z >> 31);
+}
+
+// Internal order of a set of rows (columns): by decreasing length, equal
+// lengths grouped by signature in the order the signatures first occur, equal
+// signatures in their original order.  perm receives `count` ids from `first`;
+// members (optional) the size of each id's group.
+void order_by_signature(int64_t first, int64_t count, const std::vector<int32_t>& len,
+                        const std::vector<uint64_t>& sig, int32_t* perm, int32_t* members) {
+  if (count == 0) return;
+  // group ids by first occurrence (open addressing; lengths are part of the key)
+  size_t cap = 16;
+  while (cap < (size_t)count * 2) cap <<= 1;
+  std::vector<int32_t> table(cap, -1), gid(count), glen;
+  std::vector<int64_t> gsize;
+  std::vector<int64_t> grep;  // a member of the group
+  for (int64_t t = 0; t < count; ++t) {
+    const int64_t i = first + t;
+    size_t h = mix64(sig[i] + (uint64_t)len[i]) & (cap - 1);
+    for (;; h = (h + 1) & (cap - 1)) {
+      const int32_t g = table[h];
+      if (g < 0) {
+        table[h] = gid[t] = (int32_t)glen.size();
+        glen.push_back(len[i]);
+        gsize.push_back(1);
+        grep.push_back(i);
+        break;
+      }
+      if (glen[g] == len[i] && sig[grep[g]] == sig[i]) {
+        gid[t] = g;
+        ++gsize[g];
+        break;
+      }
+    }
+  }
+  std::vector<int32_t> order(glen.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return glen[a] > glen[b]; });
+  std::vector<int64_t> pos(glen.size());
+  int64_t at = 0;
+  for (int32_t g : order) {
+    pos[g] = at;
+    at += gsize[g];
+  }
+  for (int64_t t = 0; t < count; ++t) {
+    perm[pos[gid[t]]++] = (int32_t)(first + t);
+    if (members) members[t] = (int32_t)gsize[gid[t]];
+  }
+}
+
+// Offsets of the 32-row slices over the internal order.  Slices come in aligned
+// groups of kGroup of one width, so that a warp sweeping a group (or half of one)
+// finds its entries at fixed distances.  Returns the number of slices (a multiple
+// of kGroup), -1 if the entries exceed 2^31.
+int64_t slice_offsets_of(const std::vector<int32_t>& len, const std::vector<int32_t>& perm,
+                         std::vector<int32_t>* off) {
+  const int64_t rows = (int64_t)perm.size();
+  const int64_t ng = (rows + kSlice * kGroup - 1) / (kSlice * kGroup);
+  off->assign(ng * kGroup + 1, 0);
+  int64_t tot = 0;
+  for (int64_t g = 0; g < ng; ++g) {
+    int32_t w = 0;
+    const int64_t end = std::min(rows, (g + 1) * kSlice * kGroup);
+    for (int64_t i = g * kSlice * kGroup; i < end; ++i) w = std::max(w, len[perm[i]]);
+    for (int s = 0; s < kGroup; ++s) {
+      tot += (int64_t)w * kSlice;
+      if (tot >= (int64_t)1 << 31) return -1;
+      (*off)[g * kGroup + s + 1] = (int32_t)tot;
+    }
+  }
+  return ng * kGroup;
+}
+
+// Column runs of a sliced-ELL matrix (see SellView::runs).
+void build_runs(const std::vector<int32_t>& off, const std::vector<int32_t>& col,
+                const std::vector<int32_t>& src, int64_t ncols, std::vector<int32_t>* soff,
+                std::vector<int32_t>* runs) {
+  const int64_t ns = (int64_t)off.size() - 1;
+  soff->assign(off.begin(), off.end());
+  runs->assign((size_t)off[ns] / kSlice * 2, 0);
+  for (int64_t g = 0; g < ns; g += kGroup) {
+    const int64_t o0 = off[g], o1 = off[g + kGroup];
+    int mode = ncols < ((int64_t)1 << kRunBits) ? kRunsOne : kRunsNone;
+    for (int64_t o = o0; o < o1 && mode != kRunsNone; o += kSlice) {
+      int32_t prev = -1, start[2] = {0, 0}, split = kSlice, pieces = 0;
+      for (int lane = 0; lane < kSlice; ++lane) {
+        // a padding slot (value 0) continues the run it follows, inside the vector
+        int32_t c = col[o + lane];
+        if (src[o + lane] < 0) c = (lane > 0 && prev + 1 < ncols) ? prev + 1 : 0;
+        if (lane == 0 || c != prev + 1) {
+          if (pieces == 2) {
+            mode = kRunsNone;
+            break;
+          }
+          if (pieces == 1) {
+            split = lane;
+            mode = kRunsTwo;
+          }
+          start[pieces++] = c;
+        }
+        prev = c;
+      }
+      (*runs)[o / kSlice * 2] = start[0];
+      (*runs)[o / kSlice * 2 + 1] = (int32_t)(((uint32_t)split << kRunBits) | (uint32_t)start[1]);
+    }
+    for (int s = 0; s < kGroup; ++s) (*soff)[g + s] |= mode;
+  }
+}
+
+}  // namespace
+
 int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& rp,
-                 const std::vector<int32_t>& col, HostLayout* L, std::string* err) {
+                 const std::vector<int32_t>& col, const std::vector<double>& val, HostLayout* L,
+                 std::string* err) {
   std::vector<int32_t> rlen(m), clen(n, 0);
-  for (int64_t i = 0; i < m; ++i) rlen[i] = (int32_t)(rp[i + 1] - rp[i]);
+  std::vector<uint64_t> rsig(m), csig(n, 0);
   for (size_t e = 0; e < col.size(); ++e) {
     if (col[e] < 0 || col[e] >= n) {
       *err = "column index out of range in CSR";
@@ -30,36 +150,49 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
     }
     clen[col[e]]++;
   }
-  L->perm_row.resize(m);
-  std::iota(L->perm_row.begin(), L->perm_row.end(), 0);
-  auto by_rlen = [&](int32_t a, int32_t b) { return rlen[a] > rlen[b]; };
-  std::stable_sort(L->perm_row.begin(), L->perm_row.begin() + m_eq, by_rlen);
-  std::stable_sort(L->perm_row.begin() + m_eq, L->perm_row.end(), by_rlen);
+  // Signatures that do not see a translation of the columns: a row's are its
+  // values and its column distances from its first column, a column's are the
+  // signatures of its rows and its place in them.  In a time-expanded model the
+  // rows of one line (unit, bus) share a signature over all periods, and so do
+  // its columns, so equal signatures kept in their original order run through
+  // time and row r + 1 gathers column c + 1 where row r gathers column c.  Rows
+  // that differ only in the unit they belong to (minimum up times: all values
+  // +-1) are told apart by the signature of one of their columns, the one with
+  // the most members: the others may be the few of the first or last periods.
+  for (int64_t i = 0; i < m; ++i) {
+    rlen[i] = (int32_t)(rp[i + 1] - rp[i]);
+    uint64_t h = 0;
+    for (int64_t e = rp[i]; e < rp[i + 1]; ++e) {
+      uint64_t bits;
+      std::memcpy(&bits, &val[e], sizeof(bits));
+      h = mix64(h + (uint64_t)(col[e] - col[rp[i]]) + 0x9E3779B97F4A7C15ULL) + bits;
+    }
+    rsig[i] = mix64(h);
+    for (int64_t e = rp[i]; e < rp[i + 1]; ++e) csig[col[e]] += mix64(rsig[i] + (uint64_t)(e - rp[i]));
+  }
+  std::vector<int32_t> members(n);
   L->perm_col.resize(n);
-  std::iota(L->perm_col.begin(), L->perm_col.end(), 0);
-  std::stable_sort(L->perm_col.begin(), L->perm_col.end(),
-                   [&](int32_t a, int32_t b) { return clen[a] > clen[b]; });
+  order_by_signature(0, n, clen, csig, L->perm_col.data(), members.data());
+  for (int64_t i = 0; i < m; ++i) {
+    int32_t best = -1;
+    for (int64_t e = rp[i]; e < rp[i + 1]; ++e)
+      if (best < 0 || members[col[e]] > members[best]) best = col[e];
+    if (best >= 0) rsig[i] = mix64(rsig[i] + csig[best]);
+  }
+  L->perm_row.resize(m);
+  order_by_signature(0, m_eq, rlen, rsig, L->perm_row.data(), nullptr);
+  order_by_signature(m_eq, m - m_eq, rlen, rsig, L->perm_row.data() + m_eq, nullptr);
   std::vector<int32_t> inv_row(m), inv_col(n);
   for (int64_t i = 0; i < m; ++i) inv_row[L->perm_row[i]] = (int32_t)i;
   for (int64_t j = 0; j < n; ++j) inv_col[L->perm_col[j]] = (int32_t)j;
 
   // ---- K in sliced ELL over internal rows ----
-  const int64_t ks = (m + kSlice - 1) / kSlice;
-  L->k_off.assign(ks + 1, 0);
-  int64_t tot = 0;
-  for (int64_t s = 0; s < ks; ++s) {
-    int32_t w = 0;
-    for (int lane = 0; lane < kSlice; ++lane) {
-      int64_t i = s * kSlice + lane;
-      if (i < m) w = std::max(w, rlen[L->perm_row[i]]);
-    }
-    tot += (int64_t)w * kSlice;
-    if (tot >= (int64_t)1 << 31) {
-      *err = "padded nnz of K exceeds 2^31";
-      return PDHG_ERR_UNSUPPORTED;
-    }
-    L->k_off[s + 1] = (int32_t)tot;
+  const int64_t ks = slice_offsets_of(rlen, L->perm_row, &L->k_off);
+  if (ks < 0) {
+    *err = "padded nnz of K exceeds 2^31";
+    return PDHG_ERR_UNSUPPORTED;
   }
+  int64_t tot = L->k_off[ks];
   L->k_col.assign(tot, 0);
   L->k_src.assign(tot, -1);
   for (int64_t s = 0; s < ks; ++s) {
@@ -89,22 +222,12 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
         csrc[pos] = (int32_t)e;
       }
   }
-  const int64_t ts = (n + kSlice - 1) / kSlice;
-  L->t_off.assign(ts + 1, 0);
-  tot = 0;
-  for (int64_t s = 0; s < ts; ++s) {
-    int32_t w = 0;
-    for (int lane = 0; lane < kSlice; ++lane) {
-      int64_t j = s * kSlice + lane;
-      if (j < n) w = std::max(w, clen[L->perm_col[j]]);
-    }
-    tot += (int64_t)w * kSlice;
-    if (tot >= (int64_t)1 << 31) {
-      *err = "padded nnz of K^T exceeds 2^31";
-      return PDHG_ERR_UNSUPPORTED;
-    }
-    L->t_off[s + 1] = (int32_t)tot;
+  const int64_t ts = slice_offsets_of(clen, L->perm_col, &L->t_off);
+  if (ts < 0) {
+    *err = "padded nnz of K^T exceeds 2^31";
+    return PDHG_ERR_UNSUPPORTED;
   }
+  tot = L->t_off[ts];
   L->t_col.assign(tot, 0);
   L->t_src.assign(tot, -1);
   for (int64_t s = 0; s < ts; ++s) {
@@ -119,6 +242,8 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
       }
     }
   }
+  build_runs(L->k_off, L->k_col, L->k_src, n, &L->k_soff, &L->k_runs);
+  build_runs(L->t_off, L->t_col, L->t_src, m, &L->t_soff, &L->t_runs);
   return PDHG_OK;
 }
 
