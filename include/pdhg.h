@@ -112,7 +112,10 @@ typedef struct pdhg_opts {
                                with a device-side while loop (for profilers) (0)      */
   int32_t autotune;         /* 1: time the launch variants of the per-attempt kernels
                                at the first solve of each precision and keep the
-                               fastest; 0: fixed defaults (1)                         */
+                               fastest; small LPs run the 64 attempts between two
+                               checks as one launch instead, unless kernel_variant,
+                               kernel_grid or launch_overlap asks for the separate
+                               kernels; 0: fixed defaults (1)                         */
   volatile int32_t *cancel_flag; /* host-mapped int polled at every check, or NULL    */
   int32_t kernel_variant;   /* -1: the autotuner decides, variant 1 when autotune is 0;
                                0, 1, 2, 4, 8, 9, 16-21: that variant of both
@@ -327,7 +330,9 @@ int pdhg_get_trace(void *ws, double *attempts, int64_t cap_a, double *checks, in
  * staged in shared memory by TMA bulk copies, one or two slices per warp at a
  * time; 18, 19: the same with the row (column) operands staged too; 20, 21:
  * a per-warp shared-memory ring filled by cp.async two or three slices ahead.
- * A precision not yet solved reports unroll -1 and grid 0. */
+ * A precision not yet solved reports unroll -1 and grid 0; one whose attempts
+ * run as one launch (see autotune) reports the defaults that the separate kernels
+ * would start from. */
 int pdhg_get_tuning(void *ws, int32_t *cfg);
 
 /* Launch the two per-attempt kernels of `precision` `reps` times each on

@@ -35,6 +35,7 @@ CUDA_SOURCES = [
     "pdhg_staged.cu",
     "pdhg_rowstaged.cu",
     "pdhg_ring.cu",
+    "pdhg_resident.cu",
 ]
 
 

@@ -111,9 +111,9 @@ struct DevState {
   double inv_dp, inv_dd;      // 1/Delta_P, 1/Delta_D
   double gap_w;               // Delta of round 0 / Delta of this round (weights the gap in KKT_w)
   double const_p, const_d;    // c~^T x*, q~^T y*
-  // last-block counters of the reducing kernels
+  // last-block counter of the reducing kernels
   uint32_t counter;
-  uint32_t counter2;
+  uint32_t bar;  // arrivals at the barrier of the resident attempts, 0 between launches
 };
 
 // Pointers of one precision's iteration.

@@ -90,6 +90,18 @@ struct RoundContinue {
 struct Tune {
   int unroll_dual = 1, grid_dual = 0, unroll_adj = 1, grid_adj = 0;
   bool done = false;
+  bool untimed = false;  // defaults taken because the attempts run resident
+};
+
+// 64 attempts in one launch (pdhg_resident.cu): blocks, shared memory, and where
+// each slice's entries lie in its block's shared memory.
+struct ResidentPlan {
+  bool done = false, on = false, cluster = false;
+  int grid = 0, warps = 0;
+  size_t smem = 0;
+  int32_t kcap = 0, tcap = 0, rcap = 0, ccap = 0;
+  int32_t* kloc = nullptr;
+  int32_t* tloc = nullptr;
 };
 
 struct Workspace {
@@ -126,6 +138,8 @@ struct Workspace {
   bool solved = false;      // x_star/y_star hold a solution
   int grid_k = 0, grid_kt = 0, grid_vec = 0;
   Tune tune[2];  // [0] FP64, [1] FP32
+  ResidentPlan resident[2];
+  std::vector<int32_t> koff_h, toff_h;  // slice offsets of K and K^T
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
   cudaGraph_t graph[2] = {nullptr, nullptr};
@@ -177,6 +191,13 @@ void launch_dual_ring(const IterArgs<T>& a, int grid, cudaStream_t s, int slots)
 template <class T>
 void launch_adjoint_ring(const IterArgs<T>& a, int grid, cudaStream_t s, int slots);
 int ring_setup();
+// pdhg_resident.cu: 64 attempts of a small LP in one launch.  plan_resident: false
+// if the LP does not fit the blocks' shared memory or the device refuses the launch.
+template <class T>
+bool plan_resident(const std::vector<int32_t>& koff, const std::vector<int32_t>& toff, int sms,
+                   ResidentPlan* pl, std::vector<int32_t>* kloc, std::vector<int32_t>* tloc);
+template <class T>
+void launch_resident(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_t s);
 // chunks of consecutive slices with at most max_entries entries and max_slices
 // slices each; false if a single slice is larger
 bool build_chunks(const std::vector<int32_t>& off, std::vector<int32_t>* chunks, int max_entries,

@@ -177,6 +177,47 @@ static void run_adjoint(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
   launch_adjoint<T>(a, t.grid_adj, s, t.unroll_adj);
 }
 
+// The 64 attempts between two checks.
+template <class T>
+static void run_attempts(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
+  const ResidentPlan& pl = w->resident[sizeof(T) == 8 ? 0 : 1];
+  if (pl.on) {
+    launch_resident<T>(a, pl, s);
+    return;
+  }
+  for (int k = 0; k < kCheckEvery; ++k) {
+    run_dual<T>(w, a, s);
+    run_adjoint<T>(w, a, s);
+  }
+}
+
+// Decides once per precision whether the attempts run resident: the LP fits, and
+// nothing asks for the separate per-attempt kernels.
+template <class T>
+static int setup_resident(Workspace* w) {
+  ResidentPlan& pl = w->resident[sizeof(T) == 8 ? 0 : 1];
+  const pdhg_opts& o = w->opts;
+  const bool wanted = o.autotune && o.kernel_variant < 0 && o.kernel_grid == 0 && !o.launch_overlap;
+  Tune& t = w->tune[sizeof(T) == 8 ? 0 : 1];
+  if (!wanted) {
+    pl.on = false;
+    if (t.untimed) t.done = t.untimed = false;
+    return PDHG_OK;
+  }
+  if (!pl.done) {
+    std::vector<int32_t> kloc, tloc;
+    pl.done = true;
+    if (plan_resident<T>(w->koff_h, w->toff_h, w->num_sms, &pl, &kloc, &tloc)) {
+      DALLOC(pl.kloc, kloc.size());
+      DALLOC(pl.tloc, tloc.size());
+      CK(cudaMemcpy(pl.kloc, kloc.data(), sizeof(int32_t) * kloc.size(), cudaMemcpyHostToDevice));
+      CK(cudaMemcpy(pl.tloc, tloc.data(), sizeof(int32_t) * tloc.size(), cudaMemcpyHostToDevice));
+    }
+  }
+  pl.on = pl.kloc && pl.tloc;
+  return PDHG_OK;
+}
+
 // Picks, by timing on this workspace's matrix, the variant (1, 2 or 4 slices
 // a warp sweeps together, or 0: the software-pipelined single-slice form) and
 // the grid size (2 to 8 blocks per SM) of each per-attempt kernel.  The
@@ -191,7 +232,7 @@ static int autotune(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
   t.unroll_dual = t.unroll_adj = fixed_variant >= 0 ? fixed_variant : 1;
   t.grid_dual = w->grid_k;
   t.grid_adj = w->grid_kt;
-  if (!w->opts.autotune || fixed_variant >= 0) {
+  if (!w->opts.autotune || fixed_variant >= 0 || w->resident[pi].on) {
     if ((fixed_variant == 16 || fixed_variant == 17) &&
         (w->K.nchunks == 0 || w->KT.nchunks == 0 || staged_setup() != 0))
       return fail(PDHG_ERR_UNSUPPORTED,
@@ -203,6 +244,7 @@ static int autotune(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
     if ((fixed_variant == 20 || fixed_variant == 21) && ring_setup() != 0)
       return fail(PDHG_ERR_CUDA, "kernel_variant 20/21: shared-memory opt-in refused");
     if (w->opts.kernel_grid > 0) t.grid_dual = t.grid_adj = w->opts.kernel_grid;
+    t.untimed = w->resident[pi].on;
     t.done = true;
     return PDHG_OK;
   }
@@ -278,14 +320,20 @@ static int autotune(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
 template <class T>
 static int build_graph_once(Workspace* w);
 
-// The solve graph; built with programmatic dependent launches of the
-// per-attempt kernels when enabled, and once more without them if the driver
-// refuses that graph.
+// The solve graph; built with the resident attempts or with programmatic
+// dependent launches of the per-attempt kernels when enabled, and once more
+// without them if the driver refuses that graph.
 template <class T>
 static int build_graph(Workspace* w) {
   const int pi = sizeof(T) == 8 ? 0 : 1;
   if (w->graph_exec[pi]) return PDHG_OK;
   int rc = build_graph_once<T>(w);
+  if (rc != PDHG_OK && w->resident[pi].on) {
+    cudaGetLastError();
+    w->resident[pi].on = false;
+    g_err.clear();
+    rc = build_graph_once<T>(w);
+  }
   if (rc != PDHG_OK && w->opts.launch_overlap && !w->overlap_refused) {
     cudaGetLastError();
     w->overlap_refused = true;
@@ -318,10 +366,7 @@ static int build_graph_once(Workspace* w) {
   IterArgs<T> a = make_args<T>(w);
   a.in_graph = 1;
   a.cond = (unsigned long long)h;
-  for (int k = 0; k < kCheckEvery; ++k) {
-    run_dual<T>(w, a, w->cap_stream);
-    run_adjoint<T>(w, a, w->cap_stream);
-  }
+  run_attempts<T>(w, a, w->cap_stream);
   launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->cap_stream);
   cudaGraph_t captured = nullptr;
   cudaError_t e = cudaStreamEndCapture(w->cap_stream, &captured);
@@ -406,6 +451,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
     if ((rc = alloc_bufs(w, &w->b64)) != PDHG_OK) return rc;
   }
   if ((rc = ensure_trace(w)) != PDHG_OK) return rc;
+  if ((rc = setup_resident<T>(w)) != PDHG_OK) return rc;
   const pdhg_opts& o = w->opts;
   CK(cudaEventRecord(w->ev[0], s));
   launch_prepare(w, s);
@@ -422,8 +468,9 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
   // kernels launched by this call: preparation (8 + 4 per rescaling pass),
   // FP32 copies, then per round: correction build 4; for the first round state
   // 1, init vectors 2, first primal step 1, initial check 3, for a continued
-  // round re-centering 1 and state 1; one 64-attempt body (2 per attempt + a
-  // 4-kernel check) per executed check, accumulate 1; output 1.
+  // round re-centering 1 and state 1; one 64-attempt body (2 per attempt, or 1
+  // in all if resident, + a 4-kernel check) per executed check, accumulate 1;
+  // output 1.
   const int passes = o.ruiz_iters + (o.pock_chambolle ? 1 : 0);
   int64_t launches = 8 + 4 * passes + (mixed ? 2 : 0) + 1;
   // Bound/objective rescaling is round 0 of the refinement form: the solver
@@ -506,10 +553,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
       // Same kernels as the graph body, launched from the host; the done flag
       // is read after every check (one host wait per 64 attempts).
       for (;;) {
-        for (int k = 0; k < kCheckEvery; ++k) {
-          run_dual<T>(w, a, s);
-          run_adjoint<T>(w, a, s);
-        }
+        run_attempts<T>(w, a, s);
         launch_check<T>(a, w->grid_k, w->grid_kt, 0, s);
         CK(cudaMemcpyAsync(w->st_host, w->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -524,12 +568,12 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
     CK(cudaGetLastError());
     const DevState& h = *w->st_host;
     if (h.wait_timeout)
-      return fail(PDHG_ERR_TIMEOUT, "a staged per-attempt kernel's bounded wait for its bulk copy gave up");
+      return fail(PDHG_ERR_TIMEOUT, "a per-attempt kernel's bounded wait gave up");
     k_done += h.k;
     accepted += h.accepted;
     restarts += h.restarts;
     checks += h.checks;
-    launches += h.checks * (2 * kCheckEvery + 4) + 1;
+    launches += h.checks * ((w->resident[mixed ? 1 : 0].on ? 1 : 2 * kCheckEvery) + 4) + 1;
     rounds = r;
     status = h.status;
     if (h.status != 0) break;  // optimal or a limit
@@ -684,6 +728,8 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
       return PDHG_ERR_CUDA;
     return PDHG_OK;
   };
+  w->koff_h = L.k_off;
+  w->toff_h = L.t_off;
   w->K.nslices = (int32_t)(L.k_off.size() - 1);
   w->K.rows = (int32_t)w->m;
   w->K.nnz_pad = L.k_col.size();

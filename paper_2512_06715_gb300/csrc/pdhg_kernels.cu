@@ -586,7 +586,6 @@ __global__ void k_state_init(DevState* st, RoundInit r, const double* scalars) {
   st->const_d = scalars[7];
   st->refine = r.refine;
   st->counter = 0;
-  st->counter2 = 0;
 }
 
 // ---------------------------------------------------------------------------

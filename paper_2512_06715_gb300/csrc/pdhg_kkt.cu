@@ -563,7 +563,6 @@ __global__ void k_state_continue(DevState* st, RoundContinue rc, const double* s
   st->status = 0;
   st->fold = 0;
   st->counter = 0;
-  st->counter2 = 0;
 }
 
 // Correction LP of a refinement round (Gleixner, Steffy and Wolter's
