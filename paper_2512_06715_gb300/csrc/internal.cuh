@@ -155,15 +155,18 @@ extern thread_local std::string g_err;
 
 // pdhg_layout.cu
 void launch_prepare(Workspace* w, cudaStream_t s);
-void launch_spmv64(const SellView<double>& A, const double* x, double* y, int grid, cudaStream_t s);
-void launch_spmv32(const SellView<float>& A, const float* x, float* y, int grid, cudaStream_t s);
-void launch_gather_perm(const int32_t* perm, const double* in, double* out, int64_t n, cudaStream_t s);
+template <class T>
+void launch_gather_perm(const int32_t* perm, const double* in, T* out, int64_t n, cudaStream_t s);
 void launch_scatter_perm(const int32_t* perm, const double* in, double* out, int64_t n,
                          cudaStream_t s);
 void launch_to_f32(const double* in, float* out, int64_t n, cudaStream_t s);
-void launch_to_f64(const float* in, double* out, int64_t n, cudaStream_t s);
 
 // pdhg_kernels.cu
+// y = A x, and out[perm[r]] = (A x)_r
+template <class T>
+void launch_spmv(const SellView<T>& A, const T* x, T* y, cudaStream_t s);
+template <class T>
+void launch_spmv_scatter(const SellView<T>& A, const T* x, const int32_t* perm, double* out, cudaStream_t s);
 template <class T>
 void launch_init_iterates(const IterArgs<T>& a, int grid, cudaStream_t s);
 template <class T>

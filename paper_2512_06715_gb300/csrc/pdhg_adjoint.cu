@@ -561,8 +561,8 @@ static int cg_run(Workspace* w, AdjBufs* ab, int mode, double tol, int64_t max_i
 // Active set of the last solve: masks, fixed values, counts (one host wait).
 static int classify(Workspace* w, AdjBufs* ab, cudaStream_t s, int64_t* nA, int64_t* nF) {
   const int64_t n = w->n, m = w->m;
-  launch_spmv64(w->K.v64(), w->x_star, ab->Kx, w->grid_k, s);
-  launch_spmv64(w->KT.v64(), w->y_star, ab->KTy, w->grid_kt, s);
+  launch_spmv<double>(w->K.v64(), w->x_star, ab->Kx, s);
+  launch_spmv<double>(w->KT.v64(), w->y_star, ab->KTy, s);
   const int gN = vg(n > m ? n : m);
   double* scal = w->scalars + 8;  // [8..15] scratch scalars
   k_classify<<<gN, kBlock, 0, s>>>(w->x_star, w->y_star, ab->Kx, ab->KTy, w->q_s, w->c_s, w->l_s, w->u_s,
@@ -603,20 +603,22 @@ extern "C" int pdhg_backward(void* ws, double g_cost, const double* g_x, double*
     g_err = "pdhg_backward: no solution in this workspace (call pdhg_solve first)";
     return PDHG_ERR_INVALID_ARG;
   }
-  AdjBufs* ab = nullptr;
-  int rc = adj_bufs(w, &ab);
-  if (rc != PDHG_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = w->n, m = w->m;
-  int64_t nA = 0, nF = 0;
-  if ((rc = classify(w, ab, s, &nA, &nF)) != PDHG_OK) return rc;
   const bool has_gx = g_x != nullptr;
-  if (has_gx && nA != nF) {
-    g_err = "pdhg_backward: the active set is not square (" + std::to_string(nA) + " active rows, " +
-            std::to_string(nF) + " free variables): the LP is degenerate at this solution";
-    return PDHG_ERR_NUMERIC;
-  }
+  const double *mu = nullptr, *rowA = nullptr;
+  // the cost alone needs no active set: d cost / d(q, c) = (y*, x*)
   if (has_gx) {
+    AdjBufs* ab = nullptr;
+    int rc = adj_bufs(w, &ab);
+    if (rc != PDHG_OK) return rc;
+    int64_t nA = 0, nF = 0;
+    if ((rc = classify(w, ab, s, &nA, &nF)) != PDHG_OK) return rc;
+    if (nA != nF) {
+      g_err = "pdhg_backward: the active set is not square (" + std::to_string(nA) + " active rows, " +
+              std::to_string(nF) + " free variables): the LP is degenerate at this solution";
+      return PDHG_ERR_NUMERIC;
+    }
     // r = Dc g_F (internal order); S~^T mu = r
     launch_gather_perm(w->perm_col, g_x, ab->T, n, s);
     k_mask_mul<<<vg(n), kBlock, 0, s>>>(ab->T, ab->colF, ab->r, n, w->Dc);
@@ -628,9 +630,11 @@ extern "C" int pdhg_backward(void* ws, double g_cost, const double* g_x, double*
               " iterations)";
       return PDHG_ERR_NUMERIC;
     }
+    mu = ab->z;
+    rowA = ab->rowA;
   }
   k_backward_out<<<vg(n > m ? n : m), kBlock, 0, s>>>(w->perm_row, w->perm_col, w->Dr, w->Dc, w->y_star,
-                                                      w->x_star, ab->z, ab->rowA, g_cost,
+                                                      w->x_star, mu, rowA, g_cost,
                                                       has_gx ? 1 : 0, grad_q, grad_c, n, m);
   cudaError_t e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -668,7 +672,7 @@ extern "C" int pdhg_polish(void* ws, double* x_out, double* y_out, pdhg_polish_r
   }
   // primal: x_B at its bounds, S~ x_F = rowA .* (q~ - K~ x_B), x_F = S~^T z
   k_fixed_part<<<vg(n), kBlock, 0, s>>>(ab->xfix, ab->colF, ab->xp, n);
-  launch_spmv64(w->K.v64(), ab->xp, ab->Kx, w->grid_k, s);
+  launch_spmv<double>(w->K.v64(), ab->xp, ab->Kx, s);
   k_polish_rhs<<<vg(m), kBlock, 0, s>>>(w->q_s, ab->Kx, ab->rowA, ab->b, m);
   CGState sp, sd;
   if ((rc = cg_run(w, ab, 1, 1e-13, cg_max_it(nA), s, &sp)) != PDHG_OK) return rc;
@@ -679,8 +683,8 @@ extern "C" int pdhg_polish(void* ws, double* x_out, double* y_out, pdhg_polish_r
   if ((rc = cg_run(w, ab, 0, 1e-13, cg_max_it(nA), s, &sd)) != PDHG_OK) return rc;
   k_mask_mul<<<vg(m), kBlock, 0, s>>>(ab->z, ab->rowA, ab->yp, m, nullptr);
   // optimality measures of the polished point (unscaled LP)
-  launch_spmv64(w->K.v64(), ab->xp, ab->Kx, w->grid_k, s);
-  launch_spmv64(w->KT.v64(), ab->yp, ab->KTy, w->grid_kt, s);
+  launch_spmv<double>(w->K.v64(), ab->xp, ab->Kx, s);
+  launch_spmv<double>(w->KT.v64(), ab->yp, ab->KTy, s);
   const int gN = vg(n > m ? n : m);
   k_polish_kkt<<<gN, kBlock, 0, s>>>(ab->xp, ab->yp, ab->Kx, ab->KTy, w->q_s, w->c_s, w->l_s, w->u_s,
                                      w->Dr, w->Dc, w->iDr, w->iDc, n, m, w->m_eq, w->partials);

@@ -895,28 +895,17 @@ extern "C" int pdhg_apply_K(void* ws, int32_t transpose, int32_t precision, cons
   const bool tr = transpose != 0;
   const int32_t* perm_in = tr ? w->perm_row : w->perm_col;
   const int32_t* perm_out = tr ? w->perm_col : w->perm_row;
-  const int64_t nin = tr ? w->m : w->n, nout = tr ? w->n : w->m;
-  double* tin = tr ? w->scr_m : w->scr_n;
-  double* tout = tr ? w->scr_n : w->scr_m;
-  launch_gather_perm(perm_in, in, tin, nin, s);
+  const int64_t nin = tr ? w->m : w->n;
   if (precision == PDHG_PREC_FP64) {
-    launch_spmv64(tr ? w->KT.v64() : w->K.v64(), tin, tout, tr ? w->grid_kt : w->grid_k, s);
+    double* tin = tr ? w->scr_m : w->scr_n;
+    launch_gather_perm<double>(perm_in, in, tin, nin, s);
+    launch_spmv_scatter<double>(tr ? w->KT.v64() : w->K.v64(), tin, perm_out, out, s);
   } else {
     if (!w->values_f32) return fail(PDHG_ERR_INVALID_ARG, "FP32 values not prepared");
-    float* fin = (float*)w->Kz_avg;  // scratch reuse: m doubles hold n or m floats
-    float* fout = (float*)w->KTz_avg;
-    if (tr) {
-      fin = (float*)w->KTz_avg;
-      fout = (float*)w->Kz_avg;
-    }
-    // Kz_avg has m doubles, KTz_avg n doubles: each holds 2x as many floats
-    launch_to_f32(tin, tr ? (float*)w->Kz_avg : (float*)w->KTz_avg, nin, s);
-    fin = tr ? (float*)w->Kz_avg : (float*)w->KTz_avg;
-    fout = tr ? (float*)w->KTz_avg : (float*)w->Kz_avg;
-    launch_spmv32(tr ? w->KT.v32() : w->K.v32(), fin, fout, tr ? w->grid_kt : w->grid_k, s);
-    launch_to_f64(fout, tout, nout, s);
+    float* tin = (float*)(tr ? w->scr_m : w->scr_n);
+    launch_gather_perm<float>(perm_in, in, tin, nin, s);
+    launch_spmv_scatter<float>(tr ? w->KT.v32() : w->K.v32(), tin, perm_out, out, s);
   }
-  launch_scatter_perm(perm_out, tout, out, nout, s);
   CK(cudaStreamSynchronize(s));
   CK(cudaGetLastError());
   return PDHG_OK;

@@ -105,13 +105,6 @@ __device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int2 ob, int 
     sell_dot_mode<T, U, kRunsNone, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
 }
 
-template <class T>
-__device__ __forceinline__ T sell_dot(const SellView<T>& A, int s, int lane, const T* __restrict__ x) {
-  T acc[1], unused[1];
-  sell_dot_pre<T, 1, false>(A, slice_offsets<T, 1>(A, s), lane, x, x, acc, unused);
-  return acc[0];
-}
-
 template <class T, int U, int MINB>
 __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   grid_launch_dependents();
@@ -507,16 +500,33 @@ __global__ void k_init_vectors(IterArgs<T> a) {
   }
 }
 
-template <class T>
-__global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __restrict__ x,
-                                                      T* __restrict__ y) {
+// y = A x, or with perm the FP64 result in another order, out[perm[r]] = (A x)_r
+// (pdhg_apply_K: the unscrambling, and for FP32 the widening, in the same pass).
+// Two slices per warp, one pass over the matrix without a loop: a sweep this
+// short is all latency.
+template <class T, int U>
+__global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __restrict__ x, T* __restrict__ y,
+                                                      const int32_t* __restrict__ perm, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * kBlock) >> 5;
-  for (int s = gw; s < A.nslices; s += nw) {
-    const T v = sell_dot(A, s, lane, x);
-    const int r = s * kSlice + lane;
-    if (r < A.rows) y[r] = v;
+  const int s0 = ((blockIdx.x * kBlock + threadIdx.x) >> 5) * U;
+  if (s0 >= A.nslices) return;
+  T acc[U], unused[U];
+  int to[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int r = (s0 + u) * kSlice + lane;
+    to[u] = perm && r < A.rows ? __ldg(perm + r) : r;
+  }
+  sell_dot_pre<T, U, false>(A, slice_offsets<T, U>(A, s0), lane, x, x, acc, unused);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int r = (s0 + u) * kSlice + lane;
+    if (r < A.rows) {
+      if (perm)
+        out[to[u]] = (double)acc[u];
+      else
+        y[r] = acc[u];
+    }
   }
 }
 
@@ -597,17 +607,28 @@ static int vgrid(int64_t n) {
 }
 
 template <class T>
+static void spmv_any(const SellView<T>& A, const T* x, T* y, const int32_t* perm, double* out, cudaStream_t s) {
+  const int64_t warps = (A.nslices + 1) / 2;
+  const unsigned grid = (unsigned)((warps + kWarps - 1) / kWarps);
+  k_spmv_into<T, 2><<<grid < 1 ? 1 : grid, kBlock, 0, s>>>(A, x, y, perm, out);
+}
+
+template <class T>
+void launch_spmv(const SellView<T>& A, const T* x, T* y, cudaStream_t s) {
+  spmv_any<T>(A, x, y, nullptr, nullptr, s);
+}
+
+template <class T>
+void launch_spmv_scatter(const SellView<T>& A, const T* x, const int32_t* perm, double* out, cudaStream_t s) {
+  spmv_any<T>(A, x, nullptr, perm, out, s);
+}
+
+template <class T>
 void launch_init_iterates(const IterArgs<T>& a, int grid, cudaStream_t s) {
   (void)grid;
   k_init_vectors<T><<<vgrid(a.n > a.m ? a.n : a.m), kBlock, 0, s>>>(a);
-  int gt = (a.KT.nslices + kWarps - 1) / kWarps;
-  if (gt > kMaxBlocks) gt = kMaxBlocks;
-  k_spmv_into<T><<<gt < 1 ? 1 : gt, kBlock, 0, s>>>(a.KT, a.y[0], a.KTy[0]);
-  if (StoresKx<T>::value) {
-    int gk = (a.K.nslices + kWarps - 1) / kWarps;
-    if (gk > kMaxBlocks) gk = kMaxBlocks;
-    k_spmv_into<T><<<gk < 1 ? 1 : gk, kBlock, 0, s>>>(a.K, a.x[0], a.Kx[0]);
-  }
+  launch_spmv<T>(a.KT, a.y[0], a.KTy[0], s);
+  if (StoresKx<T>::value) launch_spmv<T>(a.K, a.x[0], a.Kx[0], s);
 }
 
 // Variants: 1, 2, 4 slices per warp; 0 software pipelined; 8 and 9 are the
@@ -707,6 +728,12 @@ int blocks_per_sm_iter() {
   return best < 1 ? 1 : best;
 }
 
+template void launch_spmv<double>(const SellView<double>&, const double*, double*, cudaStream_t);
+template void launch_spmv<float>(const SellView<float>&, const float*, float*, cudaStream_t);
+template void launch_spmv_scatter<double>(const SellView<double>&, const double*, const int32_t*, double*,
+                                          cudaStream_t);
+template void launch_spmv_scatter<float>(const SellView<float>&, const float*, const int32_t*, double*,
+                                         cudaStream_t);
 template void launch_init_iterates<double>(const IterArgs<double>&, int, cudaStream_t);
 template void launch_init_iterates<float>(const IterArgs<float>&, int, cudaStream_t);
 template void launch_dual<double>(const IterArgs<double>&, int, cudaStream_t, int);

@@ -670,8 +670,8 @@ void launch_state_continue(DevState* st, const RoundContinue& rc, const double* 
 }
 
 void launch_ir_build(Workspace* w, double dp, double dd, bool make_f32, cudaStream_t s) {
-  launch_spmv64(w->K.v64(), w->x_star, w->scr_m, w->grid_k, s);
-  launch_spmv64(w->KT.v64(), w->y_star, w->scr_n, w->grid_kt, s);
+  launch_spmv<double>(w->K.v64(), w->x_star, w->scr_m, s);
+  launch_spmv<double>(w->KT.v64(), w->y_star, w->scr_n, s);
   const int g = vgrid(w->n > w->m ? w->n : w->m);
   k_ir_build<<<g, kBlock, 0, s>>>(w->q_s, w->c_s, w->l_s, w->u_s, w->x_star, w->y_star, w->scr_m,
                                   w->scr_n, dp, dd, w->n, w->m, w->m_eq, w->q_h, w->c_h, w->l_h,

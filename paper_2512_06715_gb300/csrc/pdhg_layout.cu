@@ -428,34 +428,12 @@ __global__ void k_to_f32(const double* __restrict__ in, float* __restrict__ out,
     out[t] = (float)in[t];
 }
 
-__global__ void k_to_f64(const float* __restrict__ in, double* __restrict__ out, int64_t n) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = (double)in[t];
-}
-
 template <class T>
-__global__ void __launch_bounds__(kBlock) k_spmv(SellView<T> A, const T* __restrict__ x,
-                                                 T* __restrict__ y) {
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int s = gw; s < A.nslices; s += nw) {
-    const int o0 = A.off[s], w = (A.off[s + 1] - o0) >> 5;
-    const int32_t* cp = A.col + o0 + lane;
-    const T* vp = A.val + o0 + lane;
-    T acc = 0;
-    for (int k = 0; k < w; ++k) acc += __ldg(vp + k * kSlice) * __ldg(x + __ldg(cp + k * kSlice));
-    const int r = s * kSlice + lane;
-    if (r < A.rows) y[r] = acc;
-  }
-}
-
 __global__ void k_gather_perm(const int32_t* __restrict__ perm, const double* __restrict__ in,
-                              double* __restrict__ out, int64_t n) {
+                              T* __restrict__ out, int64_t n) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = in[perm[t]];
+    out[t] = (T)in[perm[t]];
 }
 
 __global__ void k_scatter_perm(const int32_t* __restrict__ perm, const double* __restrict__ in,
@@ -475,16 +453,12 @@ static int vec_grid(int64_t n, int sms) {
   return (int)(g < 1 ? 1 : g);
 }
 
-void launch_spmv64(const SellView<double>& A, const double* x, double* y, int grid, cudaStream_t s) {
-  k_spmv<double><<<grid, kBlock, 0, s>>>(A, x, y);
+template <class T>
+void launch_gather_perm(const int32_t* perm, const double* in, T* out, int64_t n, cudaStream_t s) {
+  k_gather_perm<T><<<vec_grid(n, 152), kBlock, 0, s>>>(perm, in, out, n);
 }
-void launch_spmv32(const SellView<float>& A, const float* x, float* y, int grid, cudaStream_t s) {
-  k_spmv<float><<<grid, kBlock, 0, s>>>(A, x, y);
-}
-void launch_gather_perm(const int32_t* perm, const double* in, double* out, int64_t n,
-                        cudaStream_t s) {
-  k_gather_perm<<<vec_grid(n, 152), kBlock, 0, s>>>(perm, in, out, n);
-}
+template void launch_gather_perm<double>(const int32_t*, const double*, double*, int64_t, cudaStream_t);
+template void launch_gather_perm<float>(const int32_t*, const double*, float*, int64_t, cudaStream_t);
 void launch_scatter_perm(const int32_t* perm, const double* in, double* out, int64_t n,
                          cudaStream_t s) {
   k_scatter_perm<<<vec_grid(n, 152), kBlock, 0, s>>>(perm, in, out, n);
@@ -492,10 +466,6 @@ void launch_scatter_perm(const int32_t* perm, const double* in, double* out, int
 void launch_to_f32(const double* in, float* out, int64_t n, cudaStream_t s) {
   k_to_f32<<<vec_grid(n, 152), kBlock, 0, s>>>(in, out, n);
 }
-void launch_to_f64(const float* in, double* out, int64_t n, cudaStream_t s) {
-  k_to_f64<<<vec_grid(n, 152), kBlock, 0, s>>>(in, out, n);
-}
-
 void launch_prepare(Workspace* w, cudaStream_t s) {
   const int sms = w->num_sms;
   k_load_vals<<<vec_grid(w->K.nnz_pad, sms), kBlock, 0, s>>>(w->K.src, w->prob.val, w->K.val64,
