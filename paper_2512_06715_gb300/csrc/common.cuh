@@ -179,30 +179,93 @@ struct IterArgs {
   double* KTy_anc;  // [n] K~^T y of the restart anchor
 };
 
+// FP64 on GB300 retires two lanes per cycle and SM, against 128 FP32 or integer
+// lanes: a conversion or a comparison that an integer instruction can make is
+// worth dozens of integer instructions.
+
+// (double)x: exact.  Zeros and normal numbers by moving bits; subnormals,
+// infinities and NaNs by the conversion instruction.
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned f = __float_as_uint(x), a = f & 0x7fffffffu;
+  if (a != 0 && a - 0x00800000u >= 0x7f000000u) return (double)x;
+  const unsigned hi = (f & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(f << 29));
+}
+__device__ __forceinline__ double to_f64(double x) { return x; }
+
+// fmax(v, 0) and fmin(v, 0) (a NaN gives 0)
+__device__ __forceinline__ double pos_part(double v) {
+  return (unsigned)__double2hiint(v) <= 0x7ff00000u ? v : 0.0;
+}
+__device__ __forceinline__ double neg_part(double v) {
+  return (unsigned)__double2hiint(v) - 0x80000000u <= 0x7ff00000u ? v : 0.0;
+}
+__device__ __forceinline__ bool is_neg(double v) { return __double2hiint(v) < 0; }
+__device__ __forceinline__ bool non_zero(double v) {
+  return ((unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v)) != 0;
+}
+__device__ __forceinline__ bool non_zero(float v) { return __float_as_uint(v) << 1 != 0; }
+__device__ __forceinline__ bool finite_bits(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
 
+// Warp totals of NV values: while values are left to split, each step hands half
+// of a lane's values to its partner and adds the other half, so 16 values take 16
+// additions instead of 80.  out[k] receives the total of v[k].
+template <int NV>
+__device__ __forceinline__ void warp_sums(const double (&v)[NV], double* out) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int base = 0; base < NV; base += 16) {
+    constexpr int kAll = 16;
+    const int n = NV - base < kAll ? NV - base : kAll;
+    const int P = n > 8 ? 16 : n > 4 ? 8 : n > 2 ? 4 : n > 1 ? 2 : 1;
+    double w[kAll];
+#pragma unroll
+    for (int k = 0; k < kAll; ++k)
+      if (k < P) w[k] = k < n ? v[base + k < NV ? base + k : 0] : 0.0;
+    int o = 16, shift = 5;
+#pragma unroll
+    for (int cnt = kAll; cnt > 1; cnt >>= 1)
+      if (cnt <= P) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < kAll / 2; ++k)
+          if (k < cnt / 2) {
+            const double keep = up ? w[k + cnt / 2] : w[k], send = up ? w[k] : w[k + cnt / 2];
+            w[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        o >>= 1;
+        --shift;
+      }
+#pragma unroll
+    for (int r = 16; r > 0; r >>= 1)
+      if (r <= o) w[0] += __shfl_xor_sync(0xffffffffu, w[0], r);
+    const int k = lane >> shift;
+    if ((lane & ((1 << shift) - 1)) == 0 && k < n) out[base + k] = w[0];
+  }
+}
+
 // Deterministic block sum of NV values per thread; result valid in thread 0.
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double* smem /* [kWarps*NV] */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) smem[wid * NV + k] = v[k];
+  warp_sums<NV>(v, smem + (threadIdx.x >> 5) * NV);
   __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = 0.0;
-      for (int w = 0; w < kWarps; ++w) s += smem[w * NV + k];
-      v[k] = s;
-    }
+  if (threadIdx.x < NV) {
+    double s = 0.0;
+    for (int w = 0; w < kWarps; ++w) s += smem[w * NV + threadIdx.x];
+    smem[threadIdx.x] = s;  // read above by this thread alone
   }
+  __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = smem[k];
   __syncthreads();
 }
 
@@ -239,6 +302,26 @@ __device__ __forceinline__ void final_sum(const double* partials, int nblocks, d
   block_sum<NV>(v, smem);
 #pragma unroll
   for (int k = 0; k < NV; ++k) out[k] = v[k];
+}
+
+// The same total left in shared memory: out[NV], valid in every thread.
+template <int NV>
+__device__ __forceinline__ void final_sum_shared(const double* partials, int nblocks, double* out) {
+  __shared__ double smem[kWarps * NV];
+  double v[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] += __ldcg(partials + (size_t)b * NV + k);
+  warp_sums<NV>(v, smem + (threadIdx.x >> 5) * NV);
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double s = 0.0;
+    for (int w = 0; w < kWarps; ++w) s += smem[w * NV + threadIdx.x];
+    out[threadIdx.x] = s;
+  }
+  __syncthreads();
 }
 
 // The same last-block reduction with the partials kept in the iterate type T

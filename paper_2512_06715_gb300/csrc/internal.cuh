@@ -154,12 +154,11 @@ struct Workspace {
 extern thread_local std::string g_err;
 
 // pdhg_layout.cu
-void launch_prepare(Workspace* w, cudaStream_t s);
+void launch_prepare(Workspace* w, bool f32, cudaStream_t s);  // f32: also the FP32 values
 template <class T>
 void launch_gather_perm(const int32_t* perm, const double* in, T* out, int64_t n, cudaStream_t s);
 void launch_scatter_perm(const int32_t* perm, const double* in, double* out, int64_t n,
                          cudaStream_t s);
-void launch_to_f32(const double* in, float* out, int64_t n, cudaStream_t s);
 
 // pdhg_kernels.cu
 // y = A x, and out[perm[r]] = (A x)_r
@@ -208,7 +207,8 @@ bool build_chunks(const std::vector<int32_t>& off, std::vector<int32_t>* chunks,
 
 // pdhg_kkt.cu
 template <class T>
-void launch_check(const IterArgs<T>& a, int grid_k, int grid_kt, int init, cudaStream_t s);
+void launch_check(const IterArgs<T>& a, int grid_k, int grid_kt, int init, bool flushed,
+                  cudaStream_t s);  // flushed: the x window sums are in xbar64
 template <class T>
 void launch_accumulate(const IterArgs<T>& a, double* x_star, double* y_star, int grid,
                        cudaStream_t s);

@@ -367,7 +367,7 @@ static int build_graph_once(Workspace* w) {
   a.in_graph = 1;
   a.cond = (unsigned long long)h;
   run_attempts<T>(w, a, w->cap_stream);
-  launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->cap_stream);
+  launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->resident[pi].on, w->cap_stream);
   cudaGraph_t captured = nullptr;
   cudaError_t e = cudaStreamEndCapture(w->cap_stream, &captured);
   if (e != cudaSuccess) {
@@ -454,25 +454,20 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
   if ((rc = setup_resident<T>(w)) != PDHG_OK) return rc;
   const pdhg_opts& o = w->opts;
   CK(cudaEventRecord(w->ev[0], s));
-  launch_prepare(w, s);
-  if (mixed) {
-    launch_to_f32(w->K.val64, w->K.val32, w->K.nnz_pad, s);
-    launch_to_f32(w->KT.val64, w->KT.val32, w->KT.nnz_pad, s);
-    w->values_f32 = true;
-  }
+  launch_prepare(w, mixed, s);
   CK(cudaMemsetAsync(w->x_star, 0, sizeof(double) * w->n, s));
   CK(cudaMemsetAsync(w->y_star, 0, sizeof(double) * w->m, s));
   const int max_rounds = mixed ? 1 + o.ir_max_rounds : 1;
   const bool fixed = o.fixed_eta > 0.0;
   int64_t k_done = 0, accepted = 0, restarts = 0, checks = 0;
-  // kernels launched by this call: preparation (8 + 4 per rescaling pass),
-  // FP32 copies, then per round: correction build 4; for the first round state
+  // kernels launched by this call: preparation (5 + 1 per rescaling pass),
+  // then per round: correction build 4; for the first round state
   // 1, init vectors 2, first primal step 1, initial check 3, for a continued
-  // round re-centering 1 and state 1; one 64-attempt body (2 per attempt, or 1
-  // in all if resident, + a 4-kernel check) per executed check, accumulate 1;
-  // output 1.
+  // round re-centering 1 and state 1; one 64-attempt body (2 per attempt and, FP32,
+  // the flush of the x window, or 1 in all if resident, + a 4-kernel check) per
+  // executed check, accumulate 1; output 1.
   const int passes = o.ruiz_iters + (o.pock_chambolle ? 1 : 0);
-  int64_t launches = 8 + 4 * passes + (mixed ? 2 : 0) + 1;
+  int64_t launches = 5 + passes + 1;
   // Bound/objective rescaling is round 0 of the refinement form: the solver
   // iterates on q^ = dp0 q~, [l^,u^] = dp0 [l~,u~], c^ = dd0 c~.
   double dp0 = 1.0, dd0 = 1.0, omega0 = 0.0;
@@ -546,7 +541,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
       launch_state_init(w->st, ri, w->scalars, s);
       launch_init_iterates<T>(a, 0, s);
       run_adjoint<T>(w, a, s);
-      launch_check<T>(a, w->grid_k, w->grid_kt, 1, s);
+      launch_check<T>(a, w->grid_k, w->grid_kt, 1, true, s);
       launches += 4 + 1 + 2 + 1 + 3;
     }
     if (o.host_loop) {
@@ -554,7 +549,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
       // is read after every check (one host wait per 64 attempts).
       for (;;) {
         run_attempts<T>(w, a, s);
-        launch_check<T>(a, w->grid_k, w->grid_kt, 0, s);
+        launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->resident[mixed ? 1 : 0].on, s);
         CK(cudaMemcpyAsync(w->st_host, w->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (w->st_host->done) break;
@@ -573,7 +568,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
     accepted += h.accepted;
     restarts += h.restarts;
     checks += h.checks;
-    launches += h.checks * ((w->resident[mixed ? 1 : 0].on ? 1 : 2 * kCheckEvery) + 4) + 1;
+    launches += h.checks * ((w->resident[mixed ? 1 : 0].on ? 1 : 2 * kCheckEvery + (mixed ? 1 : 0)) + 4) + 1;
     rounds = r;
     status = h.status;
     if (h.status != 0) break;  // optimal or a limit
@@ -863,10 +858,7 @@ extern "C" int pdhg_prepare(void* ws, void* stream) {
   if (!ws) return fail(PDHG_ERR_INVALID_ARG, "workspace is NULL");
   Workspace* w = (Workspace*)ws;
   cudaStream_t s = (cudaStream_t)stream;
-  launch_prepare(w, s);
-  launch_to_f32(w->K.val64, w->K.val32, w->K.nnz_pad, s);
-  launch_to_f32(w->KT.val64, w->KT.val32, w->KT.nnz_pad, s);
-  w->values_f32 = true;
+  launch_prepare(w, true, s);
   CK(cudaStreamSynchronize(s));
   CK(cudaGetLastError());
   return PDHG_OK;

@@ -1407,9 +1407,7 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
   if (!bt->tuned) {
     // time the sweeps' launch shapes on this batch (real attempts on scratch
     // state, re-initialised below), before the graph captures them
-    launch_prepare(w, s);
-    launch_to_f32(w->K.val64, w->K.val32, w->K.nnz_pad, s);
-    launch_to_f32(w->KT.val64, w->KT.val32, w->KT.nnz_pad, s);
+    launch_prepare(w, true, s);
     int rc = autotune_batched<BP>(w, bt, a, B, l_b, u_b, s);
     if (rc != PDHG_OK) return rc;
   }
@@ -1418,10 +1416,7 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
     if (rc != PDHG_OK) return rc;
   }
   cudaEventRecord(w->ev[0], s);
-  launch_prepare(w, s);
-  launch_to_f32(w->K.val64, w->K.val32, w->K.nnz_pad, s);
-  launch_to_f32(w->KT.val64, w->KT.val32, w->KT.nnz_pad, s);
-  w->values_f32 = true;
+  launch_prepare(w, true, s);
   batched_start<BP>(w, bt, a, B, l_b, u_b, s);
   if (o.host_loop) {
     // the graph body's kernels launched from the host (profilers cannot see
@@ -1457,7 +1452,7 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
   int64_t checks_max = 0;
   for (int b = 0; b < B; ++b) checks_max = std::max(checks_max, bt->inst_host[b].checks);
   const int passes = o.ruiz_iters + (o.pock_chambolle ? 1 : 0);
-  const int64_t launches = 8 + 4 * passes + 2 + 6 + 4 + (checks_max + 1) * (2 * kCheckEvery + 4) + 1;
+  const int64_t launches = 5 + passes + 6 + 4 + (checks_max + 1) * (2 * kCheckEvery + 4) + 1;
   bool numeric = false;
   for (int b = 0; b < B; ++b) {
     const BInst& I = bt->inst_host[b];

@@ -39,6 +39,56 @@ __device__ __forceinline__ double* region(double* partials, int r) {
 // Column-side: 0 ||r_d~||^2, 1 ||r_d||^2, 2 c~^T x, 3 bound term of D(y),
 // 4 ||x - x_anchor||^2, 5 dual-ray lambda violations^2, 6 bound term of the
 // dual ray, 7 primal-ray bound violations^2, 8 c~^T dx.
+//
+// What bounds the two kernels is the FP64 pipe, so they spend FP64 instructions
+// only where a sum can change: the x-average sums arrive flushed (one FP64 gather
+// and two products per entry), conversions, signs and zero tests are integer
+// instructions, and what is zero for a whole warp is left out -- the sides that an
+// inequality or a bound absorbs, and the dual sums of rows without duals (most
+// line limits), which the internal order brings together.  6717 buses, 96
+// periods: row side 360 (FP32 iterates) and 323 us (FP64) before, 228 and 191 us
+// now; column
+// side 279 and 263 us before, 165 and 148 us now; k_control 48 us
+// before (its two candidates one after the other), 27 us now.
+
+// xbar64 += xbar: the window's sums join the FP64 sums before a check.
+__global__ void k_flush_x(IterArgs<float> a) {
+  if (a.st->done) return;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < a.n; j += gridDim.x * blockDim.x) {
+    const float w = a.xbar[j];
+    if (non_zero(w)) {
+      a.xbar64[j] += to_f64(w);
+      a.xbar[j] = 0.f;
+    }
+  }
+}
+
+// Products of one slice (lane = row) with two vectors, FP64 throughout.
+template <class T>
+__device__ __forceinline__ void kkt_dots(const SellView<double>& A, int s, int lane, const T* __restrict__ x,
+                                         const double* __restrict__ xs, bool two, double& d0, double& d1) {
+  const int o = A.off[s] + lane, w = (A.off[s + 1] - A.off[s]) >> 5;
+  d0 = d1 = 0.0;
+  for (int k0 = 0; k0 < w; k0 += 4) {
+    double v[4], b[4];
+    T g[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool ok = k0 + e < w;
+      v[e] = ok ? __ldg(A.val + o + (k0 + e) * kSlice) : 0.0;
+      const int c = ok ? __ldg(A.col + o + (k0 + e) * kSlice) : 0;
+      g[e] = ok ? x[c] : (T)0;
+      b[e] = ok && two ? xs[c] : 0.0;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (k0 + e < w) {
+        d0 += v[e] * to_f64(g[e]);
+        if (two) d1 += v[e] * b[e];
+      }
+  }
+}
+
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_kkt_row(IterArgs<T> a, int init) {
   DevState* st = a.st;
@@ -48,67 +98,102 @@ __global__ void __launch_bounds__(kBlock) k_kkt_row(IterArgs<T> a, int init) {
   const bool has_avg = wsum > 0.0;
   const double iw = has_avg ? 1.0 / wsum : 0.0;
   const T* __restrict__ xc = a.x[p];
-  const T* __restrict__ xb = a.xbar;
   const T* __restrict__ yc = a.y[p];
+  const double* xsum;  // step-weighted sum of the iterates since the last restart
+  if constexpr (sizeof(T) == 4)
+    xsum = a.xbar64;
+  else
+    xsum = (const double*)a.xbar;
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
+  const T pwT = (T)pw;
   double acc[2 * kRowSums];
 #pragma unroll
   for (int k = 0; k < 2 * kRowSums; ++k) acc[k] = 0.0;
   const SellView<double>& A = a.K64;
   for (int s = gw; s < A.nslices; s += nw) {
-    const int o0 = A.off[s], w = (A.off[s + 1] - o0) >> 5;
-    double d0 = 0.0, d1 = 0.0;
-    for (int k = 0; k < w; ++k) {
-      const int slot = o0 + k * kSlice + lane;
-      const double v = __ldg(A.val + slot);
-      const int c = __ldg(A.col + slot);
-      d0 += v * (double)xc[c];
-      if (has_avg) d1 += v * ((double)xb[c] + (a.xbar64 ? a.xbar64[c] : 0.0));
-    }
     const int i = s * kSlice + lane;
-    if (i < a.m) {
-      const T yo = yc[i];
-      T yb = a.ybar[i];
-      if (pw != 0.0) {
-        yb = yb + (T)pw * yo;
-        a.ybar[i] = yb;
-      }
-      double ybs = (double)yb;  // the sum since the last restart
-      if (a.ybar64) {
-        ybs += a.ybar64[i];
-        a.ybar64[i] = ybs;
-        a.ybar[i] = 0;
-      }
-      const double kx_avg = has_avg ? d1 * iw : d0;
+    const bool in = i < a.m;
+    const bool ineq = i >= a.m_eq;
+    T yo = 0, yb = 0, ya = 0;
+    double yb64 = 0.0, qr = 0.0, qo = 0.0, idr = 0.0, dr = 0.0, kanc = 0.0;
+    if (in) {
+      yo = yc[i];
+      yb = a.ybar[i];
+      ya = a.ya[i];
+      if constexpr (sizeof(T) == 4) yb64 = a.ybar64[i];
+      qr = a.q_res[i];
+      qo = a.q_obj[i];
+      idr = a.iDr[i];
+      dr = a.Dr[i];
+      if (!init) kanc = a.Kx_anc[i];
+    }
+    double d0, d1;
+    kkt_dots<T>(A, s, lane, xc, xsum, has_avg, d0, d1);
+    const double kx_avg = has_avg ? d1 * iw : d0;
+    if (init) kanc = d0;
+    if (in) {
       if (has_avg) a.Kz_avg[i] = kx_avg;
       a.Kz_cur[i] = d0;
       if (init) a.Kx_anc[i] = d0;
-      const double kanc = init ? d0 : a.Kx_anc[i];
-      const double y_avg = has_avg ? ybs * iw : (double)yo;
-      const double qr = a.q_res[i], qo = a.q_obj[i], idr = a.iDr[i], sr = inv_dp * idr;
-      const double dr = a.Dr[i];
-      const double yanc = (double)a.ya[i];
-      const bool ineq = i >= a.m_eq;
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double kx = c ? kx_avg : d0;
-        const double yv = c ? y_avg : (double)yo;
-        double r = qr - kx;
-        if (ineq) r = fmax(r, 0.0);
-        const double ru = r * sr;
-        const double dd = yv - yanc;
-        const double kdx = (kx - kanc) * idr;                    // (K dx)_i, unscaled
-        const double vr = ineq ? fmin(kdx, 0.0) : kdx;           // primal-ray row violation
-        const double vs = ineq ? fmin(dd, 0.0) * dr : 0.0;       // dual-ray sign violation
-        acc[c * kRowSums + 0] += r * r;
-        acc[c * kRowSums + 1] += ru * ru;
-        acc[c * kRowSums + 2] += qo * yv;
-        acc[c * kRowSums + 3] += dd * dd;
-        acc[c * kRowSums + 4] += vr * vr;
-        acc[c * kRowSums + 5] += vs * vs;
-        acc[c * kRowSums + 6] += qo * dd;
+    }
+    // primal side
+    double r0 = in ? qr - d0 : 0.0, r1 = in ? qr - kx_avg : 0.0;
+    double v0 = in ? d0 - kanc : 0.0, v1 = in ? kx_avg - kanc : 0.0;  // K dx of the rays
+    if (ineq) {
+      r0 = pos_part(r0);
+      r1 = pos_part(r1);
+      v0 = neg_part(v0);
+      v1 = neg_part(v1);
+    }
+    const bool any_r = __any_sync(0xffffffffu, non_zero(r0) || non_zero(r1));
+    const bool any_v = __any_sync(0xffffffffu, non_zero(v0) || non_zero(v1));
+    if (any_r || any_v) {
+      const double idr2 = idr * idr;
+      if (any_r) {
+        const double q0 = r0 * r0, q1 = r1 * r1;
+        acc[0] += q0;
+        acc[1] += q0 * idr2;
+        acc[kRowSums + 0] += q1;
+        acc[kRowSums + 1] += q1 * idr2;
+      }
+      if (any_v) {
+        acc[4] += (v0 * v0) * idr2;
+        acc[kRowSums + 4] += (v1 * v1) * idr2;
+      }
+    }
+    // dual side: nothing to add where the row has never had a dual since the
+    // last restart
+    const bool live = non_zero(yo) || non_zero(yb) || non_zero(yb64) || non_zero(ya);
+    if (__any_sync(0xffffffffu, live)) {
+      if (pw != 0.0) {
+        yb = yb + pwT * yo;
+        if (in && sizeof(T) == 8) a.ybar[i] = yb;
+      }
+      double ybs = to_f64(yb);  // the sum since the last restart
+      if constexpr (sizeof(T) == 4) {
+        ybs += yb64;
+        if (in) {
+          a.ybar64[i] = ybs;
+          a.ybar[i] = 0;
+        }
+      }
+      const double y0 = to_f64(yo), yan = to_f64(ya);
+      const double y1 = has_avg ? ybs * iw : y0;
+      const double dd0 = y0 - yan, dd1 = y1 - yan;
+      const double s0 = dd0 * dd0, s1 = dd1 * dd1;
+      acc[2] += qo * y0;
+      acc[3] += s0;
+      acc[6] += qo * dd0;
+      acc[kRowSums + 2] += qo * y1;
+      acc[kRowSums + 3] += s1;
+      acc[kRowSums + 6] += qo * dd1;
+      const bool n0 = ineq && is_neg(dd0), n1 = ineq && is_neg(dd1);
+      if (__any_sync(0xffffffffu, n0 || n1)) {
+        const double dr2 = dr * dr;
+        acc[5] += (n0 ? s0 : 0.0) * dr2;
+        acc[kRowSums + 5] += (n1 ? s1 : 0.0) * dr2;
       }
     }
   }
@@ -116,6 +201,9 @@ __global__ void __launch_bounds__(kBlock) k_kkt_row(IterArgs<T> a, int init) {
   block_sum<2 * kRowSums>(acc, smem);
   if (threadIdx.x == 0) {
     double* out = region(a.partials, 1) + (size_t)blockIdx.x * 2 * kRowSums;
+    const double idp2 = inv_dp * inv_dp;  // ||r_p|| is measured in the unscaled LP
+    acc[1] *= idp2;
+    acc[kRowSums + 1] *= idp2;
 #pragma unroll
     for (int k = 0; k < 2 * kRowSums; ++k) out[k] = acc[k];
   }
@@ -130,8 +218,15 @@ __global__ void __launch_bounds__(kBlock) k_kkt_col(IterArgs<T> a, int init) {
   const bool has_avg = wsum > 0.0;
   const double iw = has_avg ? 1.0 / wsum : 0.0;
   const T* __restrict__ yc = a.y[p];
-  const T* __restrict__ yb = a.ybar;
   const T* __restrict__ xc = a.x[p];
+  const double *xsum, *ysum;  // FP32 iterates: k_kkt_row has flushed the y window
+  if constexpr (sizeof(T) == 4) {
+    xsum = a.xbar64;
+    ysum = a.ybar64;
+  } else {
+    xsum = (const double*)a.xbar;
+    ysum = (const double*)a.ybar;
+  }
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
@@ -140,64 +235,71 @@ __global__ void __launch_bounds__(kBlock) k_kkt_col(IterArgs<T> a, int init) {
   for (int k = 0; k < 2 * kColSums; ++k) acc[k] = 0.0;
   const SellView<double>& A = a.KT64;
   for (int s = gw; s < A.nslices; s += nw) {
-    const int o0 = A.off[s], w = (A.off[s + 1] - o0) >> 5;
-    double e0 = 0.0, e1 = 0.0;
-    for (int k = 0; k < w; ++k) {
-      const int slot = o0 + k * kSlice + lane;
-      const double v = __ldg(A.val + slot);
-      const int c = __ldg(A.col + slot);
-      e0 += v * (double)yc[c];
-      // FP32 iterates: k_kkt_row has just flushed the window sums into ybar64
-      // and zeroed ybar, so the FP64 sum alone is the y-average sum
-      if (has_avg) e1 += v * (a.ybar64 ? a.ybar64[c] : (double)yb[c]);
-    }
     const int j = s * kSlice + lane;
-    if (j < a.n) {
-      const double kty_avg = has_avg ? e1 * iw : e0;
+    const bool in = j < a.n;
+    T x0t = 0, xat = 0;
+    double xs = 0.0, lo = 0.0, up = 0.0, idc = 0.0, dc = 0.0, cr = 0.0, co = 0.0, kanc = 0.0;
+    if (in) {
+      x0t = xc[j];
+      xat = a.xa[j];
+      xs = xsum[j];
+      lo = a.l_obj[j];
+      up = a.u_obj[j];
+      idc = a.iDc[j];
+      dc = a.Dc[j];
+      cr = a.c_res[j];
+      co = a.c_obj[j];
+      if (!init) kanc = a.KTy_anc[j];
+    }
+    double e0, e1;
+    kkt_dots<T>(A, s, lane, yc, ysum, has_avg, e0, e1);
+    const double kty_avg = has_avg ? e1 * iw : e0;
+    if (init) kanc = e0;
+    if (in) {
       if (has_avg) a.KTz_avg[j] = kty_avg;
       a.KTz_cur[j] = e0;
       if (init) a.KTy_anc[j] = e0;
-      const double kanc = init ? e0 : a.KTy_anc[j];
-      double xbs = (double)a.xbar[j];  // the sum since the last restart
-      if (a.xbar64) {
-        xbs += a.xbar64[j];
-        a.xbar64[j] = xbs;
-        a.xbar[j] = 0;
-      }
-      const double x_avg = has_avg ? xbs * iw : (double)xc[j];
-      const double lo = a.l_obj[j], up = a.u_obj[j];
-      const bool lf = isfinite(lo), uf = isfinite(up);
-      const double idc = a.iDc[j], dc = a.Dc[j];
-      const double cr = a.c_res[j], co = a.c_obj[j], sc = inv_dd * idc;
-      const double xanc = (double)a.xa[j];
+    }
+    const bool lf = finite_bits(lo), uf = finite_bits(up);
+    const double x0 = to_f64(x0t), xan = to_f64(xat);
+    const double x1 = has_avg ? xs * iw : x0;
+    const bool any_c = __any_sync(0xffffffffu, non_zero(co));
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double kty = c ? kty_avg : e0;
-        const double xv = c ? x_avg : (double)xc[j];
-        const double lam = cr - kty;
-        const double proj = (lf ? fmax(lam, 0.0) : 0.0) + (uf ? fmin(lam, 0.0) : 0.0);
-        const double rd = lam - proj;
-        const double rdu = rd * sc;
-        const double lp = proj * inv_dd;
-        const double bnd = (lf ? lo * fmax(lp, 0.0) : 0.0) - (uf ? up * fmax(-lp, 0.0) : 0.0);
-        const double dx = xv - xanc;
-        // dual ray: lambda~ = -K~^T dy~ (scaled; l~ lambda~ = l lambda), unscaled / Dc
-        const double lr = kanc - kty;
-        const double lru = lr * idc;
-        const double vl = (lf ? 0.0 : fmax(lru, 0.0)) + (uf ? 0.0 : fmin(lru, 0.0));
-        const double bray = (lf ? lo * fmax(lr, 0.0) : 0.0) - (uf ? up * fmax(-lr, 0.0) : 0.0);
-        // primal ray: dx unscaled = Dc dx~
-        const double dxu = dx * dc;
-        const double vb = (lf ? fmin(dxu, 0.0) : 0.0) + (uf ? fmax(dxu, 0.0) : 0.0);
-        acc[c * kColSums + 0] += rd * rd;
-        acc[c * kColSums + 1] += rdu * rdu;
-        acc[c * kColSums + 2] += co * xv;
-        acc[c * kColSums + 3] += bnd;
-        acc[c * kColSums + 4] += dx * dx;
-        acc[c * kColSums + 5] += vl * vl;
-        acc[c * kColSums + 6] += bray;
-        acc[c * kColSums + 7] += vb * vb;
-        acc[c * kColSums + 8] += co * dx;
+    for (int c = 0; c < 2; ++c) {
+      double* ac = acc + c * kColSums;
+      const double kty = c ? kty_avg : e0;
+      const double xv = c ? x1 : x0;
+      // reduced cost: the part a finite bound absorbs enters D with that bound,
+      // the rest is the dual residual
+      const double lam = in ? cr - kty : 0.0;
+      const bool ln = is_neg(lam), la = ln ? uf : lf;
+      const double rd = la ? 0.0 : lam;
+      ac[3] += (la ? (ln ? up : lo) : 0.0) * lam;
+      // dual ray: lambda~ = -K~^T dy~ (scaled; l~ lambda~ = l lambda)
+      const double lr = in ? kanc - kty : 0.0;
+      const bool rn = is_neg(lr), ra = rn ? uf : lf;
+      const double vl = ra ? 0.0 : lr;
+      ac[6] += (ra ? (rn ? up : lo) : 0.0) * lr;
+      const bool any_rd = __any_sync(0xffffffffu, non_zero(rd));
+      const bool any_vl = __any_sync(0xffffffffu, non_zero(vl));
+      if (any_rd || any_vl) {
+        const double idc2 = idc * idc;
+        if (any_rd) {
+          const double q = rd * rd;
+          ac[0] += q;
+          ac[1] += q * idc2;
+        }
+        if (any_vl) ac[5] += (vl * vl) * idc2;
+      }
+      if (any_c) ac[2] += co * xv;
+      // primal ray
+      const double dx = in ? xv - xan : 0.0;
+      if (__any_sync(0xffffffffu, non_zero(dx))) {
+        const double q = dx * dx;
+        ac[4] += q;
+        if (any_c) ac[8] += co * dx;
+        const bool bad = non_zero(dx) && (is_neg(dx) ? lf : uf);
+        if (__any_sync(0xffffffffu, bad)) ac[7] += (bad ? q : 0.0) * (dc * dc);
       }
     }
   }
@@ -205,6 +307,12 @@ __global__ void __launch_bounds__(kBlock) k_kkt_col(IterArgs<T> a, int init) {
   block_sum<2 * kColSums>(acc, smem);
   if (threadIdx.x == 0) {
     double* out = region(a.partials, 2) + (size_t)blockIdx.x * 2 * kColSums;
+    const double idd2 = inv_dd * inv_dd;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {  // the unscaled LP's measures
+      acc[c * kColSums + 1] *= idd2;
+      acc[c * kColSums + 3] *= inv_dd;
+    }
 #pragma unroll
     for (int k = 0; k < 2 * kColSums; ++k) out[k] = acc[k];
   }
@@ -218,15 +326,17 @@ __global__ void __launch_bounds__(kBlock) k_control(IterArgs<T> a, int nb_row, i
     if (a.in_graph && threadIdx.x == 0) cudaGraphSetConditional(a.cond, 0);
     return;
   }
-  double rs[2 * kRowSums], cs[2 * kColSums];
-  final_sum<2 * kRowSums>(region(a.partials, 1), nb_row, rs);
-  final_sum<2 * kColSums>(region(a.partials, 2), nb_col, cs);
-  if (threadIdx.x != 0) return;
+  __shared__ double rs[2 * kRowSums], cs[2 * kColSums];
+  final_sum_shared<2 * kRowSums>(region(a.partials, 1), nb_row, rs);
+  final_sum_shared<2 * kColSums>(region(a.partials, 2), nb_col, cs);
+  // the measures of the two candidates side by side (one thread each: their
+  // divisions and square roots are a chain of FP64 latencies)
+  __shared__ double rel[2], relp[2], reld[2], relg[2], P[2], D[2], kw[2], rp2s[2], rd2s[2], gh[2], dxa[2],
+      dya[2], d_viol[2], p_viol[2];
   const double omega = st->omega;
-  const double dp = 1.0 / st->inv_dp, dd = 1.0 / st->inv_dd;
-  double rel[2], relp[2], reld[2], relg[2], P[2], D[2], kw[2], rp2s[2], rd2s[2], gh[2], dxa[2],
-      dya[2];
-  for (int c = 0; c < 2; ++c) {
+  if (threadIdx.x < 2) {
+    const int c = threadIdx.x;
+    const double dp = 1.0 / st->inv_dp, dd = 1.0 / st->inv_dd;
     rp2s[c] = rs[c * kRowSums + 0];
     const double rp2u = rs[c * kRowSums + 1];
     const double qy = rs[c * kRowSums + 2];
@@ -236,19 +346,25 @@ __global__ void __launch_bounds__(kBlock) k_control(IterArgs<T> a, int nb_row, i
     const double cx = cs[c * kColSums + 2];
     const double bnd = cs[c * kColSums + 3];
     dxa[c] = cs[c * kColSums + 4];
-    P[c] = cx * st->inv_dp + st->const_p;
-    D[c] = qy * st->inv_dd + st->const_d + bnd;
+    const double Pc = cx * st->inv_dp + st->const_p;
+    const double Dc = qy * st->inv_dd + st->const_d + bnd;
+    P[c] = Pc;
+    D[c] = Dc;
     relp[c] = sqrt(rp2u) / (1.0 + st->qnorm);
     reld[c] = sqrt(rd2u) / (1.0 + st->cnorm);
-    relg[c] = fabs(P[c] - D[c]) / (1.0 + fabs(P[c]) + fabs(D[c]));
+    relg[c] = fabs(Pc - Dc) / (1.0 + fabs(Pc) + fabs(Dc));
     rel[c] = fmax(relp[c], fmax(reld[c], relg[c]));
     // Correction LP of a refinement round: residuals scale with Delta, the
     // gap with Delta^2.  Weighting the gap by Delta_0/Delta keeps KKT_w (and
     // with it the restart decisions) what it is for the same point in round 0,
     // up to a factor common to the whole round.
-    gh[c] = (P[c] - D[c]) * dp * dd * st->gap_w;
+    gh[c] = (Pc - Dc) * dp * dd * st->gap_w;
     kw[c] = sqrt(omega * rp2s[c] + rd2s[c] / omega + gh[c] * gh[c]);
+    d_viol[c] = sqrt(rs[c * kRowSums + 5] + cs[c * kColSums + 5]);
+    p_viol[c] = sqrt(rs[c * kRowSums + 4] + cs[c * kColSums + 7]);
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   const bool has_avg = st->wsum > 0.0;
   if (init) {
     st->kkt0 = kw[0];
@@ -311,13 +427,11 @@ __global__ void __launch_bounds__(kBlock) k_control(IterArgs<T> a, int nb_row, i
     // certificates from the candidates' rays (see the note above k_kkt_row)
     for (int c = 0; c < 2 && !done; ++c) {
       const double d_obj = rs[c * kRowSums + 6] + cs[c * kColSums + 6];
-      const double d_viol = sqrt(rs[c * kRowSums + 5] + cs[c * kColSums + 5]);
       const double p_obj = cs[c * kColSums + 8];
-      const double p_viol = sqrt(rs[c * kRowSums + 4] + cs[c * kColSums + 7]);
-      if (d_obj > 0.0 && d_viol <= st->infeas_eps * d_obj) {
+      if (d_obj > 0.0 && d_viol[c] <= st->infeas_eps * d_obj) {
         done = 1;
         status = PDHG_STATUS_PRIMAL_INFEASIBLE;
-      } else if (p_obj < 0.0 && p_viol <= st->infeas_eps * (-p_obj)) {
+      } else if (p_obj < 0.0 && p_viol[c] <= st->infeas_eps * (-p_obj)) {
         done = 1;
         status = PDHG_STATUS_DUAL_INFEASIBLE;
       }
@@ -645,7 +759,9 @@ static int vgrid(int64_t n) {
 }
 
 template <class T>
-void launch_check(const IterArgs<T>& a, int grid_k, int grid_kt, int init, cudaStream_t s) {
+void launch_check(const IterArgs<T>& a, int grid_k, int grid_kt, int init, bool flushed, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (!init && !flushed) k_flush_x<<<vgrid(a.n), kBlock, 0, s>>>(a);
   k_kkt_row<T><<<grid_k, kBlock, 0, s>>>(a, init);
   k_kkt_col<T><<<grid_kt, kBlock, 0, s>>>(a, init);
   k_control<T><<<1, kBlock, 0, s>>>(a, grid_k, grid_kt, init);
@@ -687,8 +803,8 @@ void launch_output(Workspace* w, double* x_out, double* y_out, cudaStream_t s) {
       w->perm_col, w->perm_row, w->Dc, w->Dr, w->x_star, w->y_star, x_out, y_out, w->n, w->m);
 }
 
-template void launch_check<double>(const IterArgs<double>&, int, int, int, cudaStream_t);
-template void launch_check<float>(const IterArgs<float>&, int, int, int, cudaStream_t);
+template void launch_check<double>(const IterArgs<double>&, int, int, int, bool, cudaStream_t);
+template void launch_check<float>(const IterArgs<float>&, int, int, int, bool, cudaStream_t);
 template void launch_accumulate<double>(const IterArgs<double>&, double*, double*, int,
                                         cudaStream_t);
 template void launch_accumulate<float>(const IterArgs<float>&, double*, double*, int, cudaStream_t);

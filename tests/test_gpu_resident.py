@@ -48,7 +48,8 @@ def test_fixed_steps(size, precision):
     kw = dict(precision=precision, max_iters=192, fixed_eta=fixed["eta"], fixed_omega=fixed["omega"])
     x, y, r = _solve(inst, **kw)
     x1, y1, r1 = _solve(inst, kernel_variant=1, **kw)
-    assert r["iterations"] == 192 and r["kernel_launches"] == r1["kernel_launches"] - 3 * 127
+    more = 127 if precision == "fp64" else 128  # FP32: the separate kernels flush the x window in a launch
+    assert r["iterations"] == 192 and r["kernel_launches"] == r1["kernel_launches"] - 3 * more
     ref = pdhg_solve(lp, fixed=fixed, stop_after=192)
     err = rel_err(x, y, returned_candidate(lp, ref, r))
     assert err <= (1e-10 if precision == "fp64" else 1e-4), err
