@@ -24,6 +24,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -76,8 +77,20 @@ struct BInst {
   double const_p, const_d;
   double t_tol[3];
   int64_t k_tol[3];
-  uint32_t pad2, pad3;
+  // what the sweeps read of the above, converted where it changes (a block that
+  // multiplies or divides in FP64 at its start waits for it): eta omega, eta /
+  // omega, pending_w, w_last; and 1 / omega for the step decision
+  float sigma, tau, pend, last;
+  double inv_omega;
 };
+
+__device__ __forceinline__ void set_steps(BInst& I) {
+  I.inv_omega = 1.0 / I.omega;
+  I.sigma = (float)(I.eta * I.omega);
+  I.tau = (float)(I.eta * I.inv_omega);
+  I.pend = (float)I.pending_w;
+  I.last = (float)I.w_last;
+}
 
 struct BGlobal {
   double tol, red;
@@ -120,10 +133,75 @@ struct BArgs {
   int32_t in_graph;
 };
 
-__device__ __forceinline__ double* preg(double* p, int r) { return p + (size_t)r * 8192 * 64 * 20; }
+// A lane's H = BP / 32 instances are neighbours, b = H lane + h, so that their
+// values are one 8-byte access where both take part; idx is the first one's.
+template <int H>
+__device__ __forceinline__ void load_inst(const float* __restrict__ v, size_t idx, float (&o)[H]) {
+  if constexpr (H == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(v + idx);
+    o[0] = t.x;
+    o[1] = t.y;
+  } else {
+    o[0] = v[idx];
+  }
+}
+template <int H>
+__device__ __forceinline__ void gather_inst(const float* __restrict__ v, size_t idx, float (&o)[H]) {
+  if constexpr (H == 2) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(v + idx));
+    o[0] = t.x;
+    o[1] = t.y;
+  } else {
+    o[0] = __ldg(v + idx);
+  }
+}
+template <int H>
+__device__ __forceinline__ void load_inst(const double* __restrict__ v, size_t idx, double (&o)[H]) {
+  if constexpr (H == 2) {
+    const double2 t = *reinterpret_cast<const double2*>(v + idx);
+    o[0] = t.x;
+    o[1] = t.y;
+  } else {
+    o[0] = v[idx];
+  }
+}
+template <int H>
+__device__ __forceinline__ void store_inst(float* __restrict__ v, size_t idx, const float (&o)[H]) {
+  if constexpr (H == 2)
+    *reinterpret_cast<float2*>(v + idx) = make_float2(o[0], o[1]);
+  else
+    v[idx] = o[0];
+}
+template <int H, class T>
+__device__ __forceinline__ void store_inst(T* __restrict__ v, size_t idx, const T (&o)[H], const bool (&on)[H]) {
+  if constexpr (H == 2) {
+    if (on[0] && on[1]) {
+      if constexpr (sizeof(T) == 4)
+        *reinterpret_cast<float2*>(v + idx) = make_float2(o[0], o[1]);
+      else
+        *reinterpret_cast<double2*>(v + idx) = make_double2(o[0], o[1]);
+      return;
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+    if (on[h]) v[idx + h] = o[h];
+}
+// The same from the buffers that each instance's parity selects.
+template <int H>
+__device__ __forceinline__ void load_par(float* const (&v)[2], const int (&par)[H], size_t idx, float (&o)[H]) {
+  if (H == 1 || par[0] == par[H - 1]) {
+    load_inst<H>(par[0] ? v[1] : v[0], idx, o);
+    return;
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) o[h] = (par[h] ? v[1] : v[0])[idx + h];
+}
+
+__host__ __device__ __forceinline__ double* preg(double* p, int r) { return p + (size_t)r * 8192 * 64 * 20; }
 
 // Per-instance block reduction of NV values held by each lane for its
-// instances b = lane + 32 h; result written to part[block][b][k] by threads
+// instances b = H lane + h; result written to part[block][b][k] by threads
 // b < BP.  smem: [warps][BP][NV].
 template <int BP, int NV, int WARPS>
 __device__ __forceinline__ void block_inst_sum(const double (&v)[BP / 32][NV], double* smem, double* out) {
@@ -131,7 +209,7 @@ __device__ __forceinline__ void block_inst_sum(const double (&v)[BP / 32][NV], d
 #pragma unroll
   for (int h = 0; h < BP / 32; ++h)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) smem[(wid * BP + lane + 32 * h) * NV + k] = v[h][k];
+    for (int k = 0; k < NV; ++k) smem[(wid * BP + lane * (BP / 32) + h) * NV + k] = v[h][k];
   __syncthreads();
   if (threadIdx.x < BP) {
     const int b = threadIdx.x;
@@ -158,6 +236,7 @@ __device__ __forceinline__ void inst_final_sum(const double* part, int nblocks, 
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = 0.0;
   if (c < C)
+#pragma unroll 8  // loads in flight: one block sums what the whole grid wrote
     for (int blk = c; blk < nblocks; blk += C)
 #pragma unroll
       for (int k = 0; k < NV; ++k) v[k] += __ldcg(part + ((size_t)blk * BP + b) * NV + k);
@@ -195,99 +274,132 @@ __device__ __forceinline__ bool last_block(uint32_t* counter) {
 template <int BP, int RW>
 __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
   BGlobal* g = a.g;
-  if (g->all_done) return;
   constexpr int H = BP / 32;
   __shared__ float s_sigma[BP], s_pw[BP];
   __shared__ int s_par[BP], s_act[BP];
+  const int all_done = g->all_done;  // read with the instances' state, not before it
   if (threadIdx.x < BP) {
     const BInst& I = a.inst[threadIdx.x];
-    s_sigma[threadIdx.x] = (float)(I.eta * I.omega);
-    s_pw[threadIdx.x] = (float)I.pending_w;
+    s_sigma[threadIdx.x] = I.sigma;
+    s_pw[threadIdx.x] = I.pend;
     s_par[threadIdx.x] = I.par;
     s_act[threadIdx.x] = I.act;
   }
   __syncthreads();
+  if (all_done) return;
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBThreads + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBThreads) >> 5;
-  float a_dy2[H], a_int[H];
-#pragma unroll
-  for (int h = 0; h < H; ++h) a_dy2[h] = a_int[h] = 0.f;
-  // gather base of each lane's instances (null: instance idle)
-  const float* xg[H];
+  float a_dy2[H], a_int[H], sigma[H], pw[H];
+  int par[H];
+  bool on[H], upd[H];
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    const int b = lane + 32 * h;
-    xg[h] = s_act[b] ? a.x[1 - s_par[b]] + b : nullptr;
+    const int b = H * lane + h;
+    a_dy2[h] = a_int[h] = 0.f;
+    sigma[h] = s_sigma[b];
+    pw[h] = s_pw[b];
+    par[h] = s_par[b];
+    on[h] = s_act[b];
+    upd[h] = on[h] && pw[h] != 0.f;
   }
+  // Where a lane's instances agree on what they do and on their buffers (always
+  // with one instance per lane; with two until a step of one is rejected) every
+  // access is one of the lane's pair; else they go one by one.  64 node LPs of 6049
+  // buses x 48 periods: 615 us in pairs (1.25 ms with K^T y' before, 1.07 now), of
+  // 455 us for the vectors alone at the copy bandwidth.
   const int nq = (a.m + RW - 1) / RW;
-  for (int qd = gw; qd < nq; qd += nw) {
-    const int i0 = qd * RW;  // RW consecutive rows of one slice
-    const int s = i0 >> 5;
-    const int o_s = __ldg(a.K.off + s);
-    const int base = o_s + (i0 & 31);
-    const int w = (__ldg(a.K.off + s + 1) - o_s) >> 5;
-    // row operands do not depend on the products: issue them first so their
-    // latency overlaps the matrix stream and the gathers
-    float ko[RW][H], yo[RW][H], qv[RW][H], lo[RW][H],
-        yb[RW][H];
+  auto sweep = [&](auto paired) {
+    constexpr int S = decltype(paired)::value ? H : 1;  // instances per access
+    constexpr int N = H / S;                            // accesses per lane
+    const float *xg[N], *kxr[N], *yr[N];
+    float *kxw[N], *yw[N];
 #pragma unroll
-    for (int r = 0; r < RW; ++r)
-#pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h, i = i0 + r;
-        ko[r][h] = yo[r][h] = qv[r][h] = lo[r][h] = yb[r][h] = 0.f;
-        if (i < a.m && xg[h]) {
-          const size_t idx = (size_t)i * BP + b;
-          const int p = s_par[b];
-          ko[r][h] = a.Kx[p][idx];
-          yo[r][h] = a.y[p][idx];
-          qv[r][h] = a.qf[idx];
-          if (i >= a.m_eq) lo[r][h] = a.ylf[idx];
-          if (s_pw[b] != 0.f) yb[r][h] = a.ybar[idx];
-        }
-      }
-    float acc[RW][H];
-#pragma unroll
-    for (int r = 0; r < RW; ++r)
-#pragma unroll
-      for (int h = 0; h < H; ++h) acc[r][h] = 0.f;
-    // entry k of the group's rows: RW adjacent slots (16 B aligned:
-    // slice offsets are multiples of 32 and i0 of RW)
-#pragma unroll 2
-    for (int k = 0; k < w; ++k) {
-      int c[RW];
-      float v[RW];
-      load_slots<RW>(a.K.col + base + k * kSlice, a.K.val + base + k * kSlice, c, v);
+    for (int g = 0; g < N; ++g) {
+      const int p = par[g * S];
+      xg[g] = on[g * S] ? a.x[1 - p] + H * lane + g * S : nullptr;
+      kxr[g] = a.Kx[p];
+      yr[g] = a.y[p];
+      kxw[g] = a.Kx[1 - p];
+      yw[g] = a.y[1 - p];
+    }
+    for (int qd = gw; qd < nq; qd += nw) {
+      const int i0 = qd * RW;  // RW consecutive rows of one slice
+      const int s = i0 >> 5;
+      const int o_s = __ldg(a.K.off + s);
+      const int base = o_s + (i0 & 31);
+      const int w = (__ldg(a.K.off + s + 1) - o_s) >> 5;
+      // row operands do not depend on the products: issue them first so their
+      // latency overlaps the matrix stream and the gathers
+      float ko[RW][N][S], yo[RW][N][S], qv[RW][N][S], lo[RW][N][S], yb[RW][N][S], acc[RW][N][S];
 #pragma unroll
       for (int r = 0; r < RW; ++r)
 #pragma unroll
-        for (int h = 0; h < H; ++h)
-          if (xg[h]) acc[r][h] += v[r] * __ldg(xg[h] + (size_t)c[r] * BP);
-    }
+        for (int g = 0; g < N; ++g) {
+          const int i = i0 + r;
 #pragma unroll
-    for (int r = 0; r < RW; ++r) {
-      const int i = i0 + r;
-      if (i >= a.m) continue;
+          for (int t = 0; t < S; ++t)
+            ko[r][g][t] = yo[r][g][t] = qv[r][g][t] = lo[r][g][t] = yb[r][g][t] = acc[r][g][t] = 0.f;
+          if (i < a.m && xg[g]) {
+            const size_t idx = (size_t)i * BP + H * lane + g * S;
+            load_inst<S>(kxr[g], idx, ko[r][g]);
+            load_inst<S>(yr[g], idx, yo[r][g]);
+            load_inst<S>(a.qf, idx, qv[r][g]);
+            if (i >= a.m_eq) load_inst<S>(a.ylf, idx, lo[r][g]);
+            if (upd[g * S]) load_inst<S>(a.ybar, idx, yb[r][g]);
+          }
+        }
+      // entry k of the group's rows: RW adjacent slots (16 B aligned:
+      // slice offsets are multiples of 32 and i0 of RW)
+#pragma unroll 2
+      for (int k = 0; k < w; ++k) {
+        int c[RW];
+        float v[RW];
+        load_slots<RW>(a.K.col + base + k * kSlice, a.K.val + base + k * kSlice, c, v);
 #pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h;
-        if (!xg[h]) continue;
-        const size_t idx = (size_t)i * BP + b;
-        const int p = s_par[b];
-        float t = qv[r][h] - 2.f * acc[r][h];
-        t = t + ko[r][h];
-        float v = yo[r][h] + s_sigma[b] * t;
-        if (i >= a.m_eq) v = fmaxf(v, lo[r][h]);
-        a.Kx[1 - p][idx] = acc[r][h];
-        a.y[1 - p][idx] = v;
-        if (s_pw[b] != 0.f) a.ybar[idx] = yb[r][h] + s_pw[b] * yo[r][h];
-        const float dy = v - yo[r][h], dk = acc[r][h] - ko[r][h];
-        a_dy2[h] += dy * dy;
-        a_int[h] += dy * dk;
+        for (int r = 0; r < RW; ++r)
+#pragma unroll
+          for (int g = 0; g < N; ++g)
+            if (xg[g]) {
+              float x[S];
+              gather_inst<S>(xg[g], (size_t)c[r] * BP, x);
+#pragma unroll
+              for (int t = 0; t < S; ++t) acc[r][g][t] += v[r] * x[t];
+            }
+      }
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const int i = i0 + r;
+        if (i >= a.m) continue;
+#pragma unroll
+        for (int g = 0; g < N; ++g) {
+          if (!xg[g]) continue;
+          const size_t idx = (size_t)i * BP + H * lane + g * S;
+          float vn[S], bn[S];
+#pragma unroll
+          for (int t = 0; t < S; ++t) {
+            const int h = g * S + t;
+            float z = qv[r][g][t] - 2.f * acc[r][g][t];
+            z = z + ko[r][g][t];
+            float v = yo[r][g][t] + sigma[h] * z;
+            if (i >= a.m_eq) v = fmaxf(v, lo[r][g][t]);
+            vn[t] = v;
+            bn[t] = yb[r][g][t] + pw[h] * yo[r][g][t];
+            const float dy = v - yo[r][g][t], dk = acc[r][g][t] - ko[r][g][t];
+            a_dy2[h] += dy * dy;
+            a_int[h] += dy * dk;
+          }
+          store_inst<S>(kxw[g], idx, acc[r][g]);
+          store_inst<S>(yw[g], idx, vn);
+          if (upd[g * S]) store_inst<S>(a.ybar, idx, bn);
+        }
       }
     }
-  }
+  };
+  if (__all_sync(0xffffffffu, H == 1 || (par[0] == par[H - 1] && on[0] == on[H - 1] && upd[0] == upd[H - 1])))
+    sweep(std::true_type{});
+  else
+    sweep(std::false_type{});
   __shared__ double smem[kBWarps * BP * 2];
   double v[H][2];
 #pragma unroll
@@ -297,36 +409,40 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
   }
   block_inst_sum<BP, 2, kBWarps>(v, smem, a.part);
   if (last_block(&g->counter)) {
-    double tot[2];
+    double tot[2], down = 0.0, up = 0.0;
+    if (threadIdx.x < BP) {  // does not depend on the sums
+      const int64_t k = a.inst[threadIdx.x].k_total + 2;
+      down = 1.0 - step_power(k, g->red_exp);
+      up = 1.0 + step_power(k, g->grow_exp);
+    }
     inst_final_sum<BP, 2>(a.part, gridDim.x, smem, tot);
     if (threadIdx.x < BP) {
       const int b = threadIdx.x;
       BInst& I = a.inst[b];
       if (I.act) {
+        // attempts of all rounds (a refinement round is a change of coordinates)
         const double dy2 = tot[0], inter = tot[1];
         const double eta = I.eta, omega = I.omega;
-        const double movement = omega * I.dx2 + dy2 / omega;
+        const double movement = omega * I.dx2 + dy2 * I.inv_omega;
         const double interaction = 2.0 * fabs(inter);
         const double eta_max = interaction > 0.0 ? movement / interaction : INFINITY;
+        const double eta_next = fmin(down * eta_max, up * eta);
+        const int accept = eta <= eta_max;
+        const double w = accept ? eta : 0.0;
         I.k += 1;
         I.k_total += 1;
-        // attempts of all rounds (a refinement round is a change of coordinates)
-        const double eta_next = fmin((1.0 - step_power(I.k_total + 1, g->red_exp)) * eta_max,
-                                     (1.0 + step_power(I.k_total + 1, g->grow_exp)) * eta);
-        const int accept = eta <= eta_max;
         if (accept) {
           I.par = 1 - I.par;
-          I.w_last = eta;
-          I.pending_w = eta;
           I.wsum += eta;
           I.accepted += 1;
-        } else {
-          I.w_last = 0.0;
-          I.pending_w = 0.0;
         }
+        I.w_last = I.pending_w = w;
+        I.last = I.pend = (float)w;
         I.accepted_last = accept;
         I.since_restart += 1;
         I.eta = eta_next;
+        I.tau = (float)(eta_next * I.inv_omega);
+        I.sigma = (float)(eta_next * omega);
       }
     }
     if (threadIdx.x == 0) g->counter = 0;
@@ -338,100 +454,123 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
 template <int BP, int RW>
 __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
   BGlobal* g = a.g;
-  if (g->all_done) return;
   constexpr int H = BP / 32;
   __shared__ float s_tau[BP], s_wl[BP];
   __shared__ int s_par[BP], s_act[BP], s_acc[BP];
+  const int all_done = g->all_done;
   if (threadIdx.x < BP) {
     const BInst& I = a.inst[threadIdx.x];
-    s_tau[threadIdx.x] = (float)(I.eta / I.omega);
-    s_wl[threadIdx.x] = (float)I.w_last;
+    s_tau[threadIdx.x] = I.tau;
+    s_wl[threadIdx.x] = I.last;
     s_par[threadIdx.x] = I.par;
     s_act[threadIdx.x] = I.act;
     s_acc[threadIdx.x] = I.act && I.accepted_last;
   }
   __syncthreads();
+  if (all_done) return;
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBThreads + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBThreads) >> 5;
-  float a_dx2[H];
-#pragma unroll
-  for (int h = 0; h < H; ++h) a_dx2[h] = 0.f;
-  // gather base of each lane's instances (null: no new K^T y this attempt)
-  const float* yg[H];
+  float a_dx2[H], tau[H], wl[H];
+  int par[H];
+  bool on[H], got[H], upd[H];  // active; new K^T y this attempt; the x-average moves
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    const int b = lane + 32 * h;
-    yg[h] = s_acc[b] ? a.y[s_par[b]] + b : nullptr;
+    const int b = H * lane + h;
+    a_dx2[h] = 0.f;
+    tau[h] = s_tau[b];
+    wl[h] = s_wl[b];
+    par[h] = s_par[b];
+    on[h] = s_act[b];
+    got[h] = s_acc[b];
+    upd[h] = got[h] && wl[h] != 0.f;
   }
   const int nq = (a.n + RW - 1) / RW;
-  for (int qd = gw; qd < nq; qd += nw) {
-    const int j0 = qd * RW;  // RW consecutive columns of one slice
-    const int s = j0 >> 5;
-    const int o_s = __ldg(a.KT.off + s);
-    const int base = o_s + (j0 & 31);
-    const int w = (__ldg(a.KT.off + s + 1) - o_s) >> 5;
-    float x0[RW][H], cv[RW][H], lv[RW][H], uv[RW][H],
-        xb[RW][H], go[RW][H];
+  auto sweep = [&](auto paired) {  // as in kb_dual
+    constexpr int S = decltype(paired)::value ? H : 1;
+    constexpr int N = H / S;
+    const float *yg[N], *xr[N];
+    float *kty[N], *xw[N];
 #pragma unroll
-    for (int r = 0; r < RW; ++r)
-#pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h, j = j0 + r;
-        x0[r][h] = cv[r][h] = lv[r][h] = uv[r][h] = xb[r][h] = go[r][h] = 0.f;
-        if (j < a.n && s_act[b]) {
-          const size_t idx = (size_t)j * BP + b;
-          const int p = s_par[b];
-          x0[r][h] = a.x[p][idx];
-          cv[r][h] = a.cf[idx];
-          lv[r][h] = a.lf[idx];
-          uv[r][h] = a.uf[idx];
-          if (!s_acc[b]) go[r][h] = a.KTy[p][idx];
-          if (s_acc[b] && s_wl[b] != 0.f) xb[r][h] = a.xbar[idx];
-        }
-      }
-    float acc[RW][H];
-#pragma unroll
-    for (int r = 0; r < RW; ++r)
-#pragma unroll
-      for (int h = 0; h < H; ++h) acc[r][h] = 0.f;
-#pragma unroll 2
-    for (int k = 0; k < w; ++k) {
-      int c[RW];
-      float v[RW];
-      load_slots<RW>(a.KT.col + base + k * kSlice, a.KT.val + base + k * kSlice, c, v);
+    for (int g = 0; g < N; ++g) {
+      const int p = par[g * S];
+      yg[g] = got[g * S] ? a.y[p] + H * lane + g * S : nullptr;
+      xr[g] = a.x[p];
+      xw[g] = a.x[1 - p];
+      kty[g] = a.KTy[p];
+    }
+    for (int qd = gw; qd < nq; qd += nw) {
+      const int j0 = qd * RW;  // RW consecutive columns of one slice
+      const int s = j0 >> 5;
+      const int o_s = __ldg(a.KT.off + s);
+      const int base = o_s + (j0 & 31);
+      const int w = (__ldg(a.KT.off + s + 1) - o_s) >> 5;
+      float x0[RW][N][S], cv[RW][N][S], lv[RW][N][S], uv[RW][N][S], xb[RW][N][S], acc[RW][N][S];
 #pragma unroll
       for (int r = 0; r < RW; ++r)
 #pragma unroll
-        for (int h = 0; h < H; ++h)
-          if (yg[h]) acc[r][h] += v[r] * __ldg(yg[h] + (size_t)c[r] * BP);
-    }
+        for (int g = 0; g < N; ++g) {
+          const int j = j0 + r;
 #pragma unroll
-    for (int r = 0; r < RW; ++r) {
-      const int j = j0 + r;
-      if (j >= a.n) continue;
-#pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h;
-        if (!s_act[b]) continue;
-        const size_t idx = (size_t)j * BP + b;
-        const int p = s_par[b];
-        float gval;
-        if (s_acc[b]) {
-          gval = acc[r][h];
-          a.KTy[p][idx] = gval;
-          if (s_wl[b] != 0.f) a.xbar[idx] = xb[r][h] + s_wl[b] * x0[r][h];
-        } else {
-          gval = go[r][h];
+          for (int t = 0; t < S; ++t)
+            x0[r][g][t] = cv[r][g][t] = lv[r][g][t] = uv[r][g][t] = xb[r][g][t] = acc[r][g][t] = 0.f;
+          if (j < a.n && on[g * S]) {
+            const size_t idx = (size_t)j * BP + H * lane + g * S;
+            load_inst<S>(xr[g], idx, x0[r][g]);
+            load_inst<S>(a.cf, idx, cv[r][g]);
+            load_inst<S>(a.lf, idx, lv[r][g]);
+            load_inst<S>(a.uf, idx, uv[r][g]);
+            if (!yg[g]) load_inst<S>(kty[g], idx, acc[r][g]);  // the old K^T y
+            if (upd[g * S]) load_inst<S>(a.xbar, idx, xb[r][g]);
+          }
         }
-        float v = x0[r][h] - s_tau[b] * (cv[r][h] - gval);
-        v = fminf(fmaxf(v, lv[r][h]), uv[r][h]);
-        a.x[1 - p][idx] = v;
-        const float d = v - x0[r][h];
-        a_dx2[h] += d * d;
+#pragma unroll 2
+      for (int k = 0; k < w; ++k) {
+        int c[RW];
+        float v[RW];
+        load_slots<RW>(a.KT.col + base + k * kSlice, a.KT.val + base + k * kSlice, c, v);
+#pragma unroll
+        for (int r = 0; r < RW; ++r)
+#pragma unroll
+          for (int g = 0; g < N; ++g)
+            if (yg[g]) {
+              float y[S];
+              gather_inst<S>(yg[g], (size_t)c[r] * BP, y);
+#pragma unroll
+              for (int t = 0; t < S; ++t) acc[r][g][t] += v[r] * y[t];
+            }
+      }
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const int j = j0 + r;
+        if (j >= a.n) continue;
+#pragma unroll
+        for (int g = 0; g < N; ++g) {
+          if (!on[g * S]) continue;
+          const size_t idx = (size_t)j * BP + H * lane + g * S;
+          float vn[S], bn[S];
+#pragma unroll
+          for (int t = 0; t < S; ++t) {
+            const int h = g * S + t;
+            bn[t] = xb[r][g][t] + wl[h] * x0[r][g][t];
+            float v = x0[r][g][t] - tau[h] * (cv[r][g][t] - acc[r][g][t]);
+            v = fminf(fmaxf(v, lv[r][g][t]), uv[r][g][t]);
+            vn[t] = v;
+            const float d = v - x0[r][g][t];
+            a_dx2[h] += d * d;
+          }
+          if (yg[g]) store_inst<S>(kty[g], idx, acc[r][g]);
+          if (upd[g * S]) store_inst<S>(a.xbar, idx, bn);
+          store_inst<S>(xw[g], idx, vn);
+        }
       }
     }
-  }
+  };
+  if (__all_sync(0xffffffffu, H == 1 || (par[0] == par[H - 1] && on[0] == on[H - 1] && got[0] == got[H - 1] &&
+                                         upd[0] == upd[H - 1])))
+    sweep(std::true_type{});
+  else
+    sweep(std::false_type{});
   __shared__ double smem[kBWarps * BP];
   double v[H][1];
 #pragma unroll
@@ -450,94 +589,202 @@ __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
 
 // ---------------------------------------------------------------- checks (FP64)
 
+// xbar64 += xbar: the window's sums join the FP64 sums before a check, so that the
+// row side gathers one of them.
+template <int BP>
+__global__ void kb_flush_x(BArgs<BP> a) {
+  if (a.g->all_done) return;
+  const size_t N = (size_t)a.n * BP / 4;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < N; t += (size_t)gridDim.x * blockDim.x) {
+    const float4 w = reinterpret_cast<const float4*>(a.xbar)[t];
+    if (!(non_zero(w.x) || non_zero(w.y) || non_zero(w.z) || non_zero(w.w))) continue;
+    double2* d = reinterpret_cast<double2*>(a.xbar64) + 2 * t;
+    double2 p = d[0], q = d[1];
+    p.x += to_f64(w.x);
+    p.y += to_f64(w.y);
+    q.x += to_f64(w.z);
+    q.y += to_f64(w.w);
+    d[0] = p;
+    d[1] = q;
+    reinterpret_cast<float4*>(a.xbar)[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// Products of row i with two vectors of every instance, FP64 throughout; o, w: the
+// first slot and the entries of its slice (loaded a row ahead).  E entries are in
+// flight: four on the row side, so that most rows cost one round trip for the
+// entries and one for the gathers; two on the column side, whose sums leave no
+// registers for more (5.4 against 6.1 ms).
+template <int BP, int E>
+__device__ __forceinline__ void kb_dots(const SellView<double>& A, int o, int w, int i, int lane,
+                                        float* const (&x)[2], const int (&par)[BP / 32],
+                                        const double* __restrict__ xs, bool some, double (&d0)[BP / 32],
+                                        double (&d1)[BP / 32]) {
+  constexpr int H = BP / 32;
+#pragma unroll
+  for (int h = 0; h < H; ++h) d0[h] = d1[h] = 0.0;
+  if (!some) return;
+  for (int k0 = 0; k0 < w; k0 += E) {
+    float g[E][H];
+    double t[E][H], v[E];
+    int c[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const bool ok = k0 + e < w;
+      const int slot = o + (k0 + (ok ? e : 0)) * kSlice + (i & 31);
+      c[e] = __ldg(A.col + slot);
+      v[e] = __ldg(A.val + slot);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (k0 + e < w) {
+        const size_t ci = (size_t)c[e] * BP + H * lane;
+        load_par<H>(x, par, ci, g[e]);
+        load_inst<H>(xs, ci, t[e]);
+      }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (k0 + e < w)
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          d0[h] += v[e] * to_f64(g[e][h]);
+          d1[h] += v[e] * t[e][h];
+        }
+  }
+}
+
 // The infeasibility rays of each instance are the differences of its current
 // and average iterates from its last restart anchor, tested as in the
 // single-instance check (pdhg_kkt.cu): the anchors' FP64 products Kxa, KTya are
 // seeded at the first check and moved at restarts and refinement folds.
+// FP64-pipe bound like that check, and written like it; here a warp holds one
+// row (column) of all instances, so what is left out as zero is a row inactive
+// in every node LP.  64 node LPs of 6049 buses x 48 periods: row side 10.3 ms
+// before, 5.6 ms now; column side 10.9 ms before, 5.4 ms now
+// (row side at 80% of the FP64 pipe).
 template <int BP>
 __global__ void __launch_bounds__(kKktWarps * 32) kb_kkt_row(BArgs<BP> a, int init) {
   BGlobal* g = a.g;
   if (g->all_done) return;
   constexpr int H = BP / 32;
-  __shared__ double s_iw[BP], s_idp[BP], s_pw[BP];
-  __shared__ int s_par[BP], s_act[BP];
-  if (threadIdx.x < BP) {
-    const BInst& I = a.inst[threadIdx.x];
-    s_iw[threadIdx.x] = I.wsum > 0.0 ? 1.0 / I.wsum : 0.0;
-    s_idp[threadIdx.x] = 1.0 / I.dp;
-    s_pw[threadIdx.x] = I.pending_w;
-    s_par[threadIdx.x] = I.par;
-    s_act[threadIdx.x] = I.act;
-  }
-  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  double acc[H][2 * kRowS];
+  double acc[H][2 * kRowS], iw[H], idp2[H];
+  float pw[H];
+  int par[H];
+  bool on[H], has_avg[H];
+  bool some = false;
 #pragma unroll
-  for (int h = 0; h < H; ++h)
+  for (int h = 0; h < H; ++h) {
+    const BInst& I = a.inst[H * lane + h];
+    has_avg[h] = I.wsum > 0.0;
+    iw[h] = has_avg[h] ? 1.0 / I.wsum : 0.0;
+    idp2[h] = 1.0 / (I.dp * I.dp);
+    pw[h] = (float)I.pending_w;
+    par[h] = I.par;
+    on[h] = I.act;
+    some = some || on[h];
 #pragma unroll
     for (int k = 0; k < 2 * kRowS; ++k) acc[h][k] = 0.0;
+  }
+  int o_next = 0, e_next = 0;  // the next row's slice
+  if (gw < a.m) {
+    o_next = __ldg(a.K64.off + (gw >> 5));
+    e_next = __ldg(a.K64.off + (gw >> 5) + 1);
+  }
   for (int i = gw; i < a.m; i += nw) {
-    const int s = i >> 5, r = i & 31;
-    const int o0 = __ldg(a.K64.off + s) + r;
-    const int w = (__ldg(a.K64.off + s + 1) - __ldg(a.K64.off + s)) >> 5;
-    double d0[H], d1[H];
-#pragma unroll
-    for (int h = 0; h < H; ++h) d0[h] = d1[h] = 0.0;
-    for (int k = 0; k < w; ++k) {
-      const int c = __ldg(a.K64.col + o0 + k * kSlice);
-      const double v = __ldg(a.K64.val + o0 + k * kSlice);
-#pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h;
-        if (!s_act[b]) continue;
-        const size_t ci = (size_t)c * BP + b;
-        d0[h] += v * (double)a.x[s_par[b]][ci];
-        if (s_iw[b] > 0.0) d1[h] += v * ((double)a.xbar[ci] + a.xbar64[ci]);
-      }
+    const size_t idx = (size_t)i * BP + H * lane;
+    const int o = o_next, w = (e_next - o_next) >> 5;
+    if (i + nw < a.m) {
+      o_next = __ldg(a.K64.off + ((i + nw) >> 5));
+      e_next = __ldg(a.K64.off + ((i + nw) >> 5) + 1);
     }
-    const double qo = a.q_obj[i], sr0 = a.iDr[i], dr0 = a.Dr[i];
+    float yo[H], yb[H], ya[H];
+    double yb64[H], qr[H], kanc[H], d0[H], d1[H];
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-      const int b = lane + 32 * h;
-      if (!s_act[b]) continue;
-      const size_t idx = (size_t)i * BP + b;
-      const bool has_avg = s_iw[b] > 0.0;
-      const float yo = a.y[s_par[b]][idx];
-      float yb = a.ybar[idx];
-      if (s_pw[b] != 0.0) yb = yb + (float)s_pw[b] * yo;
-      const double ybs = (double)yb + a.ybar64[idx];
-      a.ybar64[idx] = ybs;
-      a.ybar[idx] = 0.f;
-      const double kx_avg = has_avg ? d1[h] * s_iw[b] : d0[h];
-      a.Kzc[idx] = d0[h];
-      a.Kza[idx] = kx_avg;
-      if (init) a.Kxa[idx] = d0[h];
-      const double kanc = init ? d0[h] : a.Kxa[idx];
-      const double y_avg = has_avg ? ybs * s_iw[b] : (double)yo;
-      const double qr = a.qh[idx], sr = s_idp[b] * sr0;
-      const double yanc = (double)a.ya[idx];
-      const bool ineq = i >= a.m_eq;
+      yo[h] = yb[h] = ya[h] = 0.f;
+      yb64[h] = qr[h] = kanc[h] = 0.0;
+    }
+    if (some) {
+      load_par<H>(a.y, par, idx, yo);
+      load_inst<H>(a.ybar, idx, yb);
+      load_inst<H>(a.ya, idx, ya);
+      load_inst<H>(a.ybar64, idx, yb64);
+      load_inst<H>(a.qh, idx, qr);
+      if (!init) load_inst<H>(a.Kxa, idx, kanc);
+    }
+    const double qo = a.q_obj[i], idr = a.iDr[i], dr = a.Dr[i];
+    kb_dots<BP, 4>(a.K64, o, w, i, lane, a.x, par, a.xbar64, some, d0, d1);
+    const bool ineq = i >= a.m_eq;
+    const double idr2 = idr * idr;
 #pragma unroll
-      for (int cnd = 0; cnd < 2; ++cnd) {
-        const double kx = cnd ? kx_avg : d0[h];
-        const double yv = cnd ? y_avg : (double)yo;
-        double rr = qr - kx;
-        if (ineq) rr = fmax(rr, 0.0);
-        const double ru = rr * sr, dd = yv - yanc;
-        const double kdx = (kx - kanc) * sr0;
-        const double vr = ineq ? fmin(kdx, 0.0) : kdx;
-        const double vs = ineq ? fmin(dd, 0.0) * dr0 : 0.0;
-        acc[h][cnd * kRowS + 0] += rr * rr;
-        acc[h][cnd * kRowS + 1] += ru * ru;
-        acc[h][cnd * kRowS + 2] += qo * yv;
-        acc[h][cnd * kRowS + 3] += dd * dd;
-        acc[h][cnd * kRowS + 4] += vr * vr;
-        acc[h][cnd * kRowS + 5] += vs * vs;
-        acc[h][cnd * kRowS + 6] += qo * dd;
+    for (int h = 0; h < H; ++h) {
+      d1[h] = has_avg[h] ? d1[h] * iw[h] : d0[h];
+      if (init) kanc[h] = d0[h];
+    }
+    store_inst<H, double>(a.Kzc, idx, d0, on);
+    store_inst<H, double>(a.Kza, idx, d1, on);
+    if (init) store_inst<H, double>(a.Kxa, idx, d0, on);
+    bool live = false;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      double r0 = on[h] ? qr[h] - d0[h] : 0.0, r1 = on[h] ? qr[h] - d1[h] : 0.0;
+      double v0 = on[h] ? d0[h] - kanc[h] : 0.0, v1 = on[h] ? d1[h] - kanc[h] : 0.0;
+      if (ineq) {
+        r0 = pos_part(r0);
+        r1 = pos_part(r1);
+        v0 = neg_part(v0);
+        v1 = neg_part(v1);
+      }
+      if (__any_sync(0xffffffffu, non_zero(r0) || non_zero(r1))) {
+        const double q0 = r0 * r0, q1 = r1 * r1;
+        acc[h][0] += q0;
+        acc[h][1] += q0 * idr2;
+        acc[h][kRowS + 0] += q1;
+        acc[h][kRowS + 1] += q1 * idr2;
+      }
+      if (__any_sync(0xffffffffu, non_zero(v0) || non_zero(v1))) {
+        acc[h][4] += (v0 * v0) * idr2;
+        acc[h][kRowS + 4] += (v1 * v1) * idr2;
+      }
+      live = live || (on[h] && (non_zero(yo[h]) || non_zero(yb[h]) || non_zero(yb64[h]) || non_zero(ya[h])));
+    }
+    if (!__any_sync(0xffffffffu, live)) continue;
+    double ybs[H];
+    float zero[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      if (pw[h] != 0.f) yb[h] = yb[h] + pw[h] * yo[h];
+      ybs[h] = to_f64(yb[h]) + yb64[h];
+      zero[h] = 0.f;
+    }
+    store_inst<H, double>(a.ybar64, idx, ybs, on);
+    store_inst<H, float>(a.ybar, idx, zero, on);
+    const double dr2 = dr * dr;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const double y0 = on[h] ? to_f64(yo[h]) : 0.0, yan = on[h] ? to_f64(ya[h]) : 0.0;
+      const double y1 = on[h] ? (has_avg[h] ? ybs[h] * iw[h] : y0) : 0.0;
+      const double dd0 = y0 - yan, dd1 = y1 - yan, s0 = dd0 * dd0, s1 = dd1 * dd1;
+      acc[h][2] += qo * y0;
+      acc[h][3] += s0;
+      acc[h][6] += qo * dd0;
+      acc[h][kRowS + 2] += qo * y1;
+      acc[h][kRowS + 3] += s1;
+      acc[h][kRowS + 6] += qo * dd1;
+      const bool n0 = ineq && is_neg(dd0), n1 = ineq && is_neg(dd1);
+      if (__any_sync(0xffffffffu, n0 || n1)) {
+        acc[h][5] += (n0 ? s0 : 0.0) * dr2;
+        acc[h][kRowS + 5] += (n1 ? s1 : 0.0) * dr2;
       }
     }
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) {  // the unscaled LP's residual
+    acc[h][1] *= idp2[h];
+    acc[h][kRowS + 1] *= idp2[h];
   }
   __shared__ double smem[kKktWarps * BP * 2 * kRowS];
   block_inst_sum<BP, 2 * kRowS, kKktWarps>(acc, smem, preg(a.part, 1));
@@ -548,107 +795,159 @@ __global__ void __launch_bounds__(kKktWarps * 32) kb_kkt_col(BArgs<BP> a, int in
   BGlobal* g = a.g;
   if (g->all_done) return;
   constexpr int H = BP / 32;
-  __shared__ double s_iw[BP], s_idd[BP];
-  __shared__ int s_par[BP], s_act[BP];
-  if (threadIdx.x < BP) {
-    const BInst& I = a.inst[threadIdx.x];
-    s_iw[threadIdx.x] = I.wsum > 0.0 ? 1.0 / I.wsum : 0.0;
-    s_idd[threadIdx.x] = 1.0 / I.dd;
-    s_par[threadIdx.x] = I.par;
-    s_act[threadIdx.x] = I.act;
-  }
-  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  double acc[H][2 * kColS];
+  double acc[H][2 * kColS], iw[H], idd[H];
+  int par[H];
+  bool on[H], has_avg[H];
+  bool some = false;
 #pragma unroll
-  for (int h = 0; h < H; ++h)
+  for (int h = 0; h < H; ++h) {
+    const BInst& I = a.inst[H * lane + h];
+    has_avg[h] = I.wsum > 0.0;
+    iw[h] = has_avg[h] ? 1.0 / I.wsum : 0.0;
+    idd[h] = 1.0 / I.dd;
+    par[h] = I.par;
+    on[h] = I.act;
+    some = some || on[h];
 #pragma unroll
     for (int k = 0; k < 2 * kColS; ++k) acc[h][k] = 0.0;
+  }
+  int o_next = 0, e_next = 0;  // the next row's slice
+  if (gw < a.n) {
+    o_next = __ldg(a.KT64.off + (gw >> 5));
+    e_next = __ldg(a.KT64.off + (gw >> 5) + 1);
+  }
   for (int j = gw; j < a.n; j += nw) {
-    const int s = j >> 5, r = j & 31;
-    const int o0 = __ldg(a.KT64.off + s) + r;
-    const int w = (__ldg(a.KT64.off + s + 1) - __ldg(a.KT64.off + s)) >> 5;
-    double e0[H], e1[H];
-#pragma unroll
-    for (int h = 0; h < H; ++h) e0[h] = e1[h] = 0.0;
-    for (int k = 0; k < w; ++k) {
-      const int c = __ldg(a.KT64.col + o0 + k * kSlice);
-      const double v = __ldg(a.KT64.val + o0 + k * kSlice);
-#pragma unroll
-      for (int h = 0; h < H; ++h) {
-        const int b = lane + 32 * h;
-        if (!s_act[b]) continue;
-        const size_t ci = (size_t)c * BP + b;
-        e0[h] += v * (double)a.y[s_par[b]][ci];
-        if (s_iw[b] > 0.0) e1[h] += v * ((double)a.ybar[ci] + a.ybar64[ci]);
-      }
+    const size_t idx = (size_t)j * BP + H * lane;
+    const int o = o_next, w = (e_next - o_next) >> 5;
+    if (j + nw < a.n) {
+      o_next = __ldg(a.KT64.off + ((j + nw) >> 5));
+      e_next = __ldg(a.KT64.off + ((j + nw) >> 5) + 1);
     }
-    const double co = a.c_obj[j], sc0 = a.iDc[j], dc0 = a.Dc[j];
+    float x0t[H], xat[H];
+    double xs[H], lo[H], up[H], cr[H], kanc[H], e0[H], e1[H];
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-      const int b = lane + 32 * h;
-      if (!s_act[b]) continue;
-      const size_t idx = (size_t)j * BP + b;
-      const bool has_avg = s_iw[b] > 0.0;
-      const double kty_avg = has_avg ? e1[h] * s_iw[b] : e0[h];
-      a.KTzc[idx] = e0[h];
-      a.KTza[idx] = kty_avg;
-      if (init) a.KTya[idx] = e0[h];
-      const double kanc = init ? e0[h] : a.KTya[idx];
-      const double xc = (double)a.x[s_par[b]][idx];
-      const double xbs = (double)a.xbar[idx] + a.xbar64[idx];
-      a.xbar64[idx] = xbs;
-      a.xbar[idx] = 0.f;
-      const double x_avg = has_avg ? xbs * s_iw[b] : xc;
-      const double lo = a.lo[idx], up = a.uo[idx];
-      const bool lf = isfinite(lo), uf = isfinite(up);
-      const double cr = a.ch[idx], sc = s_idd[b] * sc0, xanc = (double)a.xa[idx];
+      x0t[h] = xat[h] = 0.f;
+      xs[h] = lo[h] = up[h] = cr[h] = kanc[h] = 0.0;
+    }
+    if (some) {
+      load_par<H>(a.x, par, idx, x0t);
+      load_inst<H>(a.xa, idx, xat);
+      load_inst<H>(a.xbar64, idx, xs);
+      load_inst<H>(a.lo, idx, lo);
+      load_inst<H>(a.uo, idx, up);
+      load_inst<H>(a.ch, idx, cr);
+      if (!init) load_inst<H>(a.KTya, idx, kanc);
+    }
+    const double co = a.c_obj[j], idc = a.iDc[j], dc = a.Dc[j];
+    // kb_kkt_row has flushed the y window into ybar64
+    kb_dots<BP, 2>(a.KT64, o, w, j, lane, a.y, par, a.ybar64, some, e0, e1);
+    const double idc2 = idc * idc, dc2 = dc * dc;
+    const bool cost = non_zero(co);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      e1[h] = has_avg[h] ? e1[h] * iw[h] : e0[h];
+      if (init) kanc[h] = e0[h];
+    }
+    store_inst<H, double>(a.KTzc, idx, e0, on);
+    store_inst<H, double>(a.KTza, idx, e1, on);
+    if (init) store_inst<H, double>(a.KTya, idx, e0, on);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const bool lf = finite_bits(lo[h]), uf = finite_bits(up[h]);
+      const double x0 = on[h] ? to_f64(x0t[h]) : 0.0, xan = on[h] ? to_f64(xat[h]) : 0.0;
+      const double x1 = on[h] ? (has_avg[h] ? xs[h] * iw[h] : x0) : 0.0;
 #pragma unroll
       for (int cnd = 0; cnd < 2; ++cnd) {
-        const double kty = cnd ? kty_avg : e0[h];
-        const double xv = cnd ? x_avg : xc;
-        const double lam = cr - kty;
-        const double proj = (lf ? fmax(lam, 0.0) : 0.0) + (uf ? fmin(lam, 0.0) : 0.0);
-        const double rd = lam - proj, rdu = rd * sc, lp = proj * s_idd[b];
-        const double bnd = (lf ? lo * fmax(lp, 0.0) : 0.0) - (uf ? up * fmax(-lp, 0.0) : 0.0);
-        const double dx = xv - xanc;
-        const double lr = kanc - kty, lru = lr * sc0;
-        const double vl = (lf ? 0.0 : fmax(lru, 0.0)) + (uf ? 0.0 : fmin(lru, 0.0));
-        const double bray = (lf ? lo * fmax(lr, 0.0) : 0.0) - (uf ? up * fmax(-lr, 0.0) : 0.0);
-        const double dxu = dx * dc0;
-        const double vb = (lf ? fmin(dxu, 0.0) : 0.0) + (uf ? fmax(dxu, 0.0) : 0.0);
-        acc[h][cnd * kColS + 0] += rd * rd;
-        acc[h][cnd * kColS + 1] += rdu * rdu;
-        acc[h][cnd * kColS + 2] += co * xv;
-        acc[h][cnd * kColS + 3] += bnd;
-        acc[h][cnd * kColS + 4] += dx * dx;
-        acc[h][cnd * kColS + 5] += vl * vl;
-        acc[h][cnd * kColS + 6] += bray;
-        acc[h][cnd * kColS + 7] += vb * vb;
-        acc[h][cnd * kColS + 8] += co * dx;
+        double* ac = acc[h] + cnd * kColS;
+        const double kty = cnd ? e1[h] : e0[h];
+        const double xv = cnd ? x1 : x0;
+        const double lam = on[h] ? cr[h] - kty : 0.0;
+        const bool ln = is_neg(lam), la = ln ? uf : lf;
+        const double rd = la ? 0.0 : lam;
+        ac[3] += (la ? (ln ? up[h] : lo[h]) : 0.0) * lam;
+        const double lr = on[h] ? kanc[h] - kty : 0.0;
+        const bool rn = is_neg(lr), ra = rn ? uf : lf;
+        const double vl = ra ? 0.0 : lr;
+        ac[6] += (ra ? (rn ? up[h] : lo[h]) : 0.0) * lr;
+        if (__any_sync(0xffffffffu, non_zero(rd))) {
+          const double q = rd * rd;
+          ac[0] += q;
+          ac[1] += q * idc2;
+        }
+        if (__any_sync(0xffffffffu, non_zero(vl))) ac[5] += (vl * vl) * idc2;
+        if (cost) ac[2] += co * xv;
+        const double dx = xv - xan;
+        if (__any_sync(0xffffffffu, non_zero(dx))) {
+          const double q = dx * dx;
+          ac[4] += q;
+          if (cost) ac[8] += co * dx;
+          const bool bad = non_zero(dx) && (is_neg(dx) ? lf : uf);
+          if (__any_sync(0xffffffffu, bad)) ac[7] += (bad ? q : 0.0) * dc2;
+        }
       }
     }
   }
+#pragma unroll
+  for (int h = 0; h < H; ++h)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {  // the unscaled LP's measures
+      acc[h][c * kColS + 1] *= idd[h] * idd[h];
+      acc[h][c * kColS + 3] *= idd[h];
+    }
   __shared__ double smem[kKktWarps * BP * 2 * kColS];
   block_inst_sum<BP, 2 * kColS, kKktWarps>(acc, smem, preg(a.part, 2));
+}
+
+// Fixed-order totals of the check's partials, one block per instance (one block
+// for all of them took 0.7 to 1.2 ms, these 12 to 29 us): tot[b][0..14) of the rows,
+// tot[b][14..32) of the columns.
+constexpr int kCheckS = 2 * (kRowS + kColS);
+template <int BP>
+__global__ void __launch_bounds__(kBlock) kb_check_sums(const BGlobal* g, const double* row, int nb_row,
+                                                        const double* col, int nb_col, double* tot) {
+  if (g->all_done) return;
+  const int b = blockIdx.x;
+  __shared__ double smem[kWarps * 2 * kColS];
+  double r[2 * kRowS], c[2 * kColS];
+#pragma unroll
+  for (int k = 0; k < 2 * kRowS; ++k) r[k] = 0.0;
+#pragma unroll
+  for (int k = 0; k < 2 * kColS; ++k) c[k] = 0.0;
+  for (int t = threadIdx.x; t < nb_row; t += kBlock)
+#pragma unroll
+    for (int k = 0; k < 2 * kRowS; ++k) r[k] += __ldcg(row + ((size_t)t * BP + b) * 2 * kRowS + k);
+  block_sum<2 * kRowS>(r, smem);
+  for (int t = threadIdx.x; t < nb_col; t += kBlock)
+#pragma unroll
+    for (int k = 0; k < 2 * kColS; ++k) c[k] += __ldcg(col + ((size_t)t * BP + b) * 2 * kColS + k);
+  block_sum<2 * kColS>(c, smem);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < 2 * kRowS; ++k) tot[b * kCheckS + k] = r[k];
+#pragma unroll
+    for (int k = 0; k < 2 * kColS; ++k) tot[b * kCheckS + 2 * kRowS + k] = c[k];
+  }
 }
 
 // One thread per instance: termination, restart, primal weight, end of a
 // refinement round; the while condition clears when every instance is done.
 template <int BP>
-__global__ void __launch_bounds__(256) kb_control(BArgs<BP> a, int nb_row, int nb_col, int init) {
+__global__ void __launch_bounds__(64) kb_control(BArgs<BP> a, const double* tot, int init) {
   BGlobal* g = a.g;
   __shared__ int s_running;
-  __shared__ double smem[(256 / BP) * BP * 2 * kColS];
   if (threadIdx.x == 0) s_running = 0;
   __syncthreads();
-  double rs[2 * kRowS], cs[2 * kColS];
-  inst_final_sum<BP, 2 * kRowS>(preg(a.part, 1), nb_row, smem, rs);
-  inst_final_sum<BP, 2 * kColS>(preg(a.part, 2), nb_col, smem, cs);
   const int b = threadIdx.x;
   if (b < BP && !g->all_done) {
+    double rs[2 * kRowS], cs[2 * kColS];
+#pragma unroll
+    for (int k = 0; k < 2 * kRowS; ++k) rs[k] = tot[b * kCheckS + k];
+#pragma unroll
+    for (int k = 0; k < 2 * kColS; ++k) cs[k] = tot[b * kCheckS + 2 * kRowS + k];
     BInst& I = a.inst[b];
     I.restart_now = 0;
     I.refine = 0;
@@ -785,7 +1084,10 @@ __global__ void __launch_bounds__(256) kb_control(BArgs<BP> a, int nb_row, int n
         }
       }
     }
-    if (I.act) I.eta = fmin(I.eta, fp32_step_cap(I.omega));  // FP32 range (see fp32_step_cap)
+    if (I.act) {
+      I.eta = fmin(I.eta, fp32_step_cap(I.omega));  // FP32 range (see fp32_step_cap)
+      set_steps(I);
+    }
     if (!I.done) atomicAdd(&s_running, 1);
   }
   __syncthreads();
@@ -813,7 +1115,7 @@ __global__ void __launch_bounds__(kApplyRows * BP) kb_apply(BArgs<BP> a) {
   const double wsum = I.wsum;
   const double div = I.avg_div;
   const int cand_avg = I.cand_avg;
-  const float tau = (float)(I.eta / I.omega);
+  const float tau = I.tau;
   double sdx = 0.0, scp = 0.0, scd = 0.0;
   if (any) {
     // rows
@@ -956,55 +1258,106 @@ __global__ void __launch_bounds__(kApplyRows * BP) kb_apply(BArgs<BP> a) {
 
 // ---------------------------------------------------------------- setup kernels
 
-// Round-0 correction data per instance from the shared LP and the instance bounds.
+__global__ void kb_invert(const int32_t* __restrict__ perm, int32_t* __restrict__ inv, int n) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) inv[perm[t]] = t;
+}
+
+// Round-0 data of every instance.  The callers' bounds lie instance after instance
+// in the original order, the solver's vectors column after column in the internal
+// one: tiles of kTile original columns go through shared memory, so that both
+// sides are read and written in whole sectors.  A bound equal to the shared LP's
+// takes that one's scaled value (a division saved in all but the fixed columns).
+// The first pending primal step x' = proj(x - tau c) (K^T y = 0) and its
+// ||dx||^2 per block are formed on the way.
+constexpr int kTile = 32;
 template <int BP>
-__global__ void kb_setup(BArgs<BP> a, const double* __restrict__ lb, const double* __restrict__ ub,
-                         const int32_t* __restrict__ perm_col, const double* __restrict__ Dc,
-                         const double* __restrict__ c_s, const double* __restrict__ q_s,
-                         const double* __restrict__ l_s, const double* __restrict__ u_s) {
-  const int64_t Nn = (int64_t)a.n * BP, Nm = (int64_t)a.m * BP;
-  const int64_t N = Nn > Nm ? Nn : Nm;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(t % BP);
-    if (t < Nn) {
-      const int j = (int)(t / BP);
+__global__ void __launch_bounds__(kBThreads) kb_setup_cols(
+    BArgs<BP> a, const double* __restrict__ lb, const double* __restrict__ ub, const double* __restrict__ l0,
+    const double* __restrict__ u0, const int32_t* __restrict__ inv_col, const double* __restrict__ Dc,
+    const double* __restrict__ c_s, const double* __restrict__ l_s, const double* __restrict__ u_s) {
+  __shared__ double tl[kTile][BP + 1], tu[kTile][BP + 1];
+  const int b = threadIdx.x % BP;
+  const float tau = a.inst[b].tau;
+  double dx2 = 0.0;
+  for (int64_t o0 = (int64_t)blockIdx.x * kTile; o0 < a.n; o0 += (int64_t)gridDim.x * kTile) {
+    for (int t = threadIdx.x; t < kTile * BP; t += kBThreads) {
+      const int oo = t % kTile, bb = t / kTile;
+      if (o0 + oo < a.n && bb < a.B) {
+        tl[oo][bb] = lb[(size_t)bb * a.n + o0 + oo];
+        tu[oo][bb] = ub[(size_t)bb * a.n + o0 + oo];
+      }
+    }
+    __syncthreads();
+    for (int oo = threadIdx.x / BP; oo < kTile && o0 + oo < a.n; oo += kBThreads / BP) {
+      const int64_t o = o0 + oo;
+      const int j = inv_col[o];
       double lo = l_s[j], up = u_s[j];
       if (b < a.B) {
-        const int o = perm_col[j];
-        lo = lb[(size_t)b * a.n + o] / Dc[j];
-        up = ub[(size_t)b * a.n + o] / Dc[j];
+        const double l = tl[oo][b], u = tu[oo][b];
+        if (__double_as_longlong(l) != __double_as_longlong(l0[o])) lo = l / Dc[j];
+        if (__double_as_longlong(u) != __double_as_longlong(u0[o])) up = u / Dc[j];
       }
+      const size_t t = (size_t)j * BP + b;
+      const double c = c_s[j];
+      const float cf = (float)c, lf = (float)lo, uf = (float)up;
       a.lo[t] = lo;
       a.uo[t] = up;
       a.lh[t] = lo;
       a.uh[t] = up;
-      a.lf[t] = (float)lo;
-      a.uf[t] = (float)up;
-      a.ch[t] = c_s[j];
-      a.cf[t] = (float)c_s[j];
+      a.lf[t] = lf;
+      a.uf[t] = uf;
+      a.ch[t] = c;
+      a.cf[t] = cf;
       a.xst[t] = 0.0;
-      const float x0 = fminf(fmaxf(0.f, (float)lo), (float)up);
+      const float x0 = fminf(fmaxf(0.f, lf), uf);
+      const float x1 = fminf(fmaxf(x0 - tau * cf, lf), uf);
       a.x[0][t] = x0;
-      a.x[1][t] = x0;
+      a.x[1][t] = x1;
       a.xa[t] = x0;
       a.xbar[t] = 0.f;
       a.xbar64[t] = 0.0;
       a.KTy[0][t] = a.KTy[1][t] = 0.f;
+      if (__float_as_uint(x1) != __float_as_uint(x0)) {
+        const double d = to_f64(x1) - to_f64(x0);
+        dx2 += d * d;
+      }
     }
-    if (t < Nm) {
-      const int i = (int)(t / BP);
-      a.qh[t] = q_s[i];
-      a.qf[t] = (float)q_s[i];
-      const double yl = (i < a.m_eq) ? -INFINITY : 0.0;
-      a.ylh[t] = yl;
-      a.ylf[t] = (float)yl;
-      a.yst[t] = 0.0;
-      a.y[0][t] = a.y[1][t] = 0.f;
-      a.ya[t] = a.ybar[t] = 0.f;
-      a.ybar64[t] = 0.0;
-    }
+    __syncthreads();
   }
+  __shared__ double sm[kBThreads];
+  sm[threadIdx.x] = dx2;
+  __syncthreads();
+  if (threadIdx.x < BP) {
+    for (int k = 1; k < kBThreads / BP; ++k) dx2 += sm[threadIdx.x + k * BP];
+    a.part[(size_t)blockIdx.x * BP + threadIdx.x] = dx2;
+  }
+}
+
+template <int BP>
+__global__ void kb_setup_rows(BArgs<BP> a, const double* __restrict__ q_s) {
+  const int64_t N = (int64_t)a.m * BP;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (int)(t / BP);
+    const double q = q_s[i], yl = (i < a.m_eq) ? -INFINITY : 0.0;
+    a.qh[t] = q;
+    a.qf[t] = (float)q;
+    a.ylh[t] = yl;
+    a.ylf[t] = (float)yl;
+    a.yst[t] = 0.0;
+    a.y[0][t] = a.y[1][t] = 0.f;
+    a.ya[t] = a.ybar[t] = 0.f;
+    a.ybar64[t] = 0.0;
+  }
+}
+
+// ||x' - x||^2 of each instance from the blocks of kb_setup_cols.
+template <int BP>
+__global__ void __launch_bounds__(kBlock) kb_first_dx2(BArgs<BP> a, int nb) {
+  __shared__ double sm[kWarps];
+  double v[1] = {0.0};
+  for (int t = threadIdx.x; t < nb; t += kBlock) v[0] += __ldcg(a.part + (size_t)t * BP + blockIdx.x);
+  block_sum<1>(v, sm);
+  if (threadIdx.x == 0) a.inst[blockIdx.x].dx2 = v[0];
 }
 
 // K x for every slot (initial point of round 0).
@@ -1032,52 +1385,24 @@ __global__ void __launch_bounds__(kBThreads) kb_spmm(BArgs<BP> a) {
   }
 }
 
-// First pending primal step of round 0 (x' from x^0, K^T y = 0).
+// out[b][o] = D v[b] of internal element inv[o], through tiles as kb_setup_cols.
 template <int BP>
-__global__ void kb_first_primal(BArgs<BP> a) {
-  const int64_t Nn = (int64_t)a.n * BP;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < Nn;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(t % BP);
-    const BInst& I = a.inst[b];
-    const float tau = (float)(I.eta / I.omega);
-    const float x0 = a.x[0][t];
-    a.x[1][t] = fminf(fmaxf(x0 - tau * a.cf[t], a.lf[t]), a.uf[t]);
-  }
-}
-
-// ||x' - x||^2 per instance, deterministic (one block per instance).
-template <int BP>
-__global__ void kb_dx2(BArgs<BP> a) {
-  const int b = blockIdx.x;
-  double s = 0.0;
-  for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
-    const size_t idx = (size_t)j * BP + b;
-    const double d = (double)a.x[1][idx] - (double)a.x[0][idx];
-    s += d * d;
-  }
-  __shared__ double sm[kWarps];
-  double v[1] = {s};
-  block_sum<1>(v, sm);
-  if (threadIdx.x == 0) a.inst[b].dx2 = v[0];
-}
-
-template <int BP>
-__global__ void kb_output(BArgs<BP> a, const int32_t* __restrict__ perm_col,
-                          const int32_t* __restrict__ perm_row, const double* __restrict__ Dc,
-                          const double* __restrict__ Dr, double* x_out, double* y_out) {
-  const int64_t Nn = (int64_t)a.n * a.B, Nm = (int64_t)a.m * a.B;
-  const int64_t N = Nn > Nm ? Nn : Nm;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    if (x_out && t < Nn) {
-      const int b = (int)(t / a.n), j = (int)(t % a.n);
-      x_out[(size_t)b * a.n + perm_col[j]] = Dc[j] * a.xst[(size_t)j * BP + b];
+__global__ void __launch_bounds__(kBThreads) kb_output(const double* __restrict__ v, const double* __restrict__ D,
+                                                       const int32_t* __restrict__ inv, int64_t len, int B,
+                                                       double* __restrict__ out) {
+  __shared__ double tile[kTile][BP + 1];
+  const int b = threadIdx.x % BP;
+  for (int64_t o0 = (int64_t)blockIdx.x * kTile; o0 < len; o0 += (int64_t)gridDim.x * kTile) {
+    for (int oo = threadIdx.x / BP; oo < kTile && o0 + oo < len; oo += kBThreads / BP) {
+      const int j = inv[o0 + oo];
+      tile[oo][b] = D[j] * v[(size_t)j * BP + b];
     }
-    if (y_out && t < Nm) {
-      const int b = (int)(t / a.m), i = (int)(t % a.m);
-      y_out[(size_t)b * a.m + perm_row[i]] = Dr[i] * a.yst[(size_t)i * BP + b];
+    __syncthreads();
+    for (int t = threadIdx.x; t < kTile * B; t += kBThreads) {
+      const int oo = t % kTile, bb = t / kTile;
+      if (o0 + oo < len) out[(size_t)bb * len + o0 + oo] = tile[oo][bb];
     }
+    __syncthreads();
   }
 }
 
@@ -1097,6 +1422,7 @@ __global__ void kb_init_state(BInst* inst, BGlobal* g, int B, int BP, const doub
     memset(&I, 0, sizeof(I));
     I.eta = scalars[0];
     I.omega = scalars[1];
+    set_steps(I);
     I.act = b < B;
     I.done = b >= B;
     I.dp = I.dd = 1.0;
@@ -1119,11 +1445,12 @@ struct Batched {
   int32_t* done_host = nullptr;  // pinned copy of g->all_done (host-loop mode)
   BGlobal* g = nullptr;
   double* part = nullptr;
+  int32_t *inv_row = nullptr, *inv_col = nullptr;  // original -> internal
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
   int grid_rows = 0, grid_cols = 0, grid_kr = 0, grid_kc = 0, grid_apply = 0;
   int rw_dual = 4, rw_adj = 4;  // rows (columns) per warp of the sweeps
-  bool tuned = false;
+  bool tuned = false, inverted = false;
 };
 
 template <int BP>
@@ -1178,6 +1505,8 @@ int setup_batched(Workspace* w, Batched* bt, BArgs<BP>* out) {
   if (e == cudaSuccess) e = balloc(bt, &bt->inst, BP);
   if (e == cudaSuccess) e = balloc(bt, &bt->g, 1);
   if (e == cudaSuccess) e = balloc(bt, &bt->part, (size_t)3 * 8192 * 64 * 20);
+  if (e == cudaSuccess) e = balloc(bt, &bt->inv_row, w->m);
+  if (e == cudaSuccess) e = balloc(bt, &bt->inv_col, w->n);
   if (e != cudaSuccess) {
     g_err = std::string("batched allocation: ") + cudaGetErrorString(e);
     return PDHG_ERR_NOMEM;
@@ -1236,9 +1565,13 @@ void launch_body(const BArgs<BP>& a, Batched* bt, cudaStream_t s, int init) {
       launch_sweep_adjoint<BP>(a, bt->rw_adj, bt->grid_cols, s);
     }
   }
+  if (!init) kb_flush_x<BP><<<bt->grid_apply, 256, 0, s>>>(a);
   kb_kkt_row<BP><<<bt->grid_kr, kKktWarps * 32, 0, s>>>(a, init);
   kb_kkt_col<BP><<<bt->grid_kc, kKktWarps * 32, 0, s>>>(a, init);
-  kb_control<BP><<<1, 256, 0, s>>>(a, bt->grid_kr, bt->grid_kc, init);
+  // the attempts' region of the partials is free here
+  kb_check_sums<BP><<<BP, kBlock, 0, s>>>(a.g, preg(a.part, 1), bt->grid_kr, preg(a.part, 2), bt->grid_kc,
+                                          a.part);
+  kb_control<BP><<<1, 64, 0, s>>>(a, a.part, init);
   if (!init) kb_apply<BP><<<bt->grid_apply, kApplyRows * BP, 0, s>>>(a);
 }
 
@@ -1303,15 +1636,17 @@ void batched_start(Workspace* w, Batched* bt, const BArgs<BP>& a, int B, const d
   gin.n_real = B;
   kb_init_state<<<1, BP < 32 ? 32 : BP, 0, s>>>(bt->inst, bt->g, B, BP, w->scalars, gin);
   const int gv = std::min(w->num_sms * 8, 8192);
-  kb_setup<BP><<<gv, 256, 0, s>>>(a, l_b, u_b, w->perm_col, w->Dc, w->c_s, w->q_s, w->l_s, w->u_s);
+  const int gt = (int)std::min<int64_t>((w->n + kTile - 1) / kTile, gv);
+  kb_setup_cols<BP><<<gt, kBThreads, 0, s>>>(a, l_b, u_b, w->prob.l, w->prob.u, bt->inv_col, w->Dc, w->c_s, w->l_s,
+                                             w->u_s);
+  kb_setup_rows<BP><<<gv, 256, 0, s>>>(a, w->q_s);
+  kb_first_dx2<BP><<<BP, kBlock, 0, s>>>(a, gt);
   kb_spmm<BP><<<bt->grid_rows, kBThreads, 0, s>>>(a);
-  kb_first_primal<BP><<<gv, 256, 0, s>>>(a);
-  kb_dx2<BP><<<BP, kBlock, 0, s>>>(a);
   launch_body<BP>(a, bt, s, 1);  // initial KKT_w of every instance
 }
 
 // The batched autotuner: rows (columns) per warp R in {1, 2, 4} and the grid
-// (1 to 4 blocks per SM, capped by occupancy and by 8 rows per warp) of each
+// (1 to 8 blocks per SM, capped by occupancy and by one row group per warp) of each
 // sweep, timed with CUDA events on this matrix and batch width.  UCPDHG_TUNE_LOG=1
 // prints the table to stderr.
 template <int BP>
@@ -1345,7 +1680,8 @@ int autotune_batched(Workspace* w, Batched* bt, const BArgs<BP>& a, int B, const
             &occ, rw == 4 ? (const void*)kb_adjoint<BP, 4> : rw == 2 ? (const void*)kb_adjoint<BP, 2> : (const void*)kb_adjoint<BP, 1>,
             kBThreads, 0);
       occ = std::max(occ, 1);
-      const int need = (int)std::max<int64_t>(1, (len + 8 * kBWarps - 1) / (8 * kBWarps));
+      // at most one row group per warp
+      const int need = (int)std::max<int64_t>(1, (len + rw * kBWarps - 1) / (rw * kBWarps));
       for (int bps = 1; bps <= std::min(occ, 8); ++bps) {
         const int g = std::min(std::min(sms * bps, need), 8192);
         auto run = [&]() {
@@ -1400,6 +1736,16 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
     if (rc != PDHG_OK) return rc;
     bt->args = new BArgs<BP>(a);
   }
+  if (!bt->inverted) {
+    kb_invert<<<w->num_sms, 256, 0, s>>>(w->perm_row, bt->inv_row, (int)w->m);
+    kb_invert<<<w->num_sms, 256, 0, s>>>(w->perm_col, bt->inv_col, (int)w->n);
+    // a later call may use another stream
+    if (cudaStreamSynchronize(s) != cudaSuccess) {
+      g_err = std::string("batched setup: ") + cudaGetErrorString(cudaGetLastError());
+      return PDHG_ERR_CUDA;
+    }
+    bt->inverted = true;
+  }
   BArgs<BP> a = *(BArgs<BP>*)bt->args;
   a.B = B;
   a.in_graph = 0;
@@ -1438,8 +1784,13 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
       return PDHG_ERR_CUDA;
     }
   }
-  kb_output<BP><<<std::min(w->num_sms * 8, 8192), 256, 0, s>>>(a, w->perm_col, w->perm_row, w->Dc, w->Dr,
-                                                               x_out, y_out);
+  const int64_t gmax = std::min(w->num_sms * 8, 8192);
+  if (x_out)
+    kb_output<BP><<<(int)std::min<int64_t>((w->n + kTile - 1) / kTile, gmax), kBThreads, 0, s>>>(
+        a.xst, w->Dc, bt->inv_col, w->n, B, x_out);
+  if (y_out)
+    kb_output<BP><<<(int)std::min<int64_t>((w->m + kTile - 1) / kTile, gmax), kBThreads, 0, s>>>(
+        a.yst, w->Dr, bt->inv_row, w->m, B, y_out);
   cudaEventRecord(w->ev[1], s);
   if (cudaMemcpyAsync(bt->inst_host, bt->inst, sizeof(BInst) * BP, cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
@@ -1452,7 +1803,7 @@ int solve_batched_impl(Workspace* w, int B, const double* l_b, const double* u_b
   int64_t checks_max = 0;
   for (int b = 0; b < B; ++b) checks_max = std::max(checks_max, bt->inst_host[b].checks);
   const int passes = o.ruiz_iters + (o.pock_chambolle ? 1 : 0);
-  const int64_t launches = 5 + passes + 6 + 4 + (checks_max + 1) * (2 * kCheckEvery + 4) + 1;
+  const int64_t launches = 5 + passes + 5 + 4 + checks_max * (2 * kCheckEvery + 6) + 2;
   bool numeric = false;
   for (int b = 0; b < B; ++b) {
     const BInst& I = bt->inst_host[b];
