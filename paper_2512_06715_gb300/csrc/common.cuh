@@ -32,6 +32,7 @@ constexpr int kRunBits = 26;     // bits of a column index in the second word of
 // low bits of SellView::soff, one value per group of slices
 constexpr int kRunsNone = 0;     // explicit column indices
 constexpr int kRunsTwo = 1;      // every k-column is one or two runs
+constexpr int kRunsMixed = 3;    // most are, the others have split 0: take the indices
 constexpr int kRunsOne = 2;      // every k-column is one run
 constexpr int kTraceCheckCols = 12;  // values recorded per KKT check in the trace
 
@@ -46,18 +47,19 @@ struct SellView {
   const T* val;        // [nnz_pad]
   int32_t nslices;
   int32_t rows;        // logical rows (<= 32 * nslices)
-  // Column runs.  soff[s] is off[s] with, in its low bits, kRunsOne (kRunsTwo)
-  // where every k-column of the slice's group is one run (at most two runs) of
-  // consecutive column indices over the lanes; runs[off/32 + k] then replaces the
-  // 128 B of indices by 8 B: lanes below `split` gather x + lane, the others
-  // y + lane - split, with y in the low kRunBits bits of the second word and split
-  // above them.
+  // Column runs.  soff[s] is off[s] with, in its low bits, kRunsOne where every
+  // k-column of the slice's group is one run of consecutive column indices over the
+  // lanes, kRunsTwo where all are at most two and kRunsMixed where most are;
+  // runs[off/32 + k] then replaces the 128 B of indices by 8 B: lanes below `split`
+  // gather x + lane, the others y + lane - split, with y in the low kRunBits bits
+  // of the second word and split above them.  Split 0: this k-column has more runs.
   const int32_t* soff;  // [nslices + 1]
   const int2* runs;     // [nnz_pad / 32]
 };
 
+__device__ __forceinline__ int run_split(int2 r) { return (int)((unsigned)r.y >> kRunBits); }
 __device__ __forceinline__ int run_col(int2 r, int lane) {
-  const int split = (int)((unsigned)r.y >> kRunBits);
+  const int split = run_split(r);
   return lane < split ? r.x + lane : (r.y & ((1 << kRunBits) - 1)) + lane - split;
 }
 

@@ -45,26 +45,64 @@ __device__ __forceinline__ SliceSpan slice_span(int2 ob) {
   return {ob.x & ~(kSlice - 1), ((ob.y >> 5) - (ob.x >> 5)) / U, ob.x & (kSlice - 1)};
 }
 
+// Run words of the next 32 / U k-columns of each of the U slices: lane t holds the
+// one of slice t U / 32.  One coalesced load (issued an iteration ahead by the
+// per-attempt kernels) instead of a dependent one before every gather: entries and
+// gathers then leave together.  The 4 registers of the two iterations are there at
+// two slices per warp (6717-bus day, FP32, K x' 39.2 -> 36.9 us, K^T y' 25.0 ->
+// 22.8); at one slice and 40 registers they spill (45 -> 52 us), so U = 1 reads each
+// word where it is used.
+template <class T, int U>
+__device__ __forceinline__ int2 run_words(const SellView<T>& A, const SliceSpan& g, int k0, int lane) {
+  constexpr int W = 32 / U;
+  if (U == 1) return int2{};
+  const int k = k0 + lane % W;
+  return (g.mode != kRunsNone && k < g.w) ? __ldg(A.runs + (g.o >> 5) + (lane / W) * g.w + k)
+                                          : make_int2(0, (int)((unsigned)kSlice << kRunBits));
+}
+
+// E entries of each slice from k0 on; rw: the run words from k-column kw on.
 template <class T, int U, int E, int MODE, bool TWO, bool TAIL>
-__device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan& g, int k0, int lane,
-                                          const T* __restrict__ x1, const T* __restrict__ x2,
+__device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan& g, int2 rw, int kw, int k0,
+                                          int lane, const T* __restrict__ x1, const T* __restrict__ x2,
                                           T (&acc1)[U], T (&acc2)[U]) {
   int c[U][E];
   T v[U][E];
+  [[maybe_unused]] bool indices = false;
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const bool ok = !TAIL || k0 + e < g.w;
       const int slot = g.o + (u * g.w + k0 + e) * kSlice;
-      if (MODE == kRunsOne)
-        c[u][e] = ok ? __ldg(&A.runs[slot >> 5].x) + lane : 0;
-      else if (MODE == kRunsTwo)
-        c[u][e] = ok ? run_col(__ldg(A.runs + (slot >> 5)), lane) : 0;
-      else
+      if (MODE == kRunsNone) {
         c[u][e] = ok ? __ldg(A.col + slot + lane) : 0;
+      } else {
+        int2 r = make_int2(0, (int)((unsigned)kSlice << kRunBits));
+        if constexpr (U == 1) {
+          if (ok) r = __ldg(A.runs + (slot >> 5));
+        } else {
+          const int t = u * (32 / U) + k0 + e - kw;
+          r.x = __shfl_sync(0xffffffffu, rw.x, t);
+          if (MODE != kRunsOne) r.y = __shfl_sync(0xffffffffu, rw.y, t);
+        }
+        if (MODE == kRunsOne) {
+          c[u][e] = r.x + lane;
+        } else {
+          c[u][e] = run_col(r, lane);
+          if (MODE == kRunsMixed) indices |= run_split(r) == 0;
+        }
+      }
       v[u][e] = ok ? __ldg(A.val + slot + lane) : (T)0;
     }
+  // one branch for the chunk: a branch per k-column keeps the later loads behind it
+  if (MODE == kRunsMixed && indices) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (!TAIL || k0 + e < g.w) c[u][e] = __ldg(A.col + g.o + (u * g.w + k0 + e) * kSlice + lane);
+  }
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -76,33 +114,43 @@ __device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan&
 }
 
 template <class T, int U, int MODE, bool TWO>
-__device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceSpan& g, int k0, int lane,
+__device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceSpan& g, int2 rw, int lane,
                                               const T* __restrict__ x1, const T* __restrict__ x2,
                                               T (&acc1)[U], T (&acc2)[U]) {
   if constexpr (U == 1) {
-    if (g.w - k0 <= 2)
-      dot_chunk<T, U, 2, MODE, TWO, true>(A, g, k0, lane, x1, x2, acc1, acc2);
+    if (g.w <= 2)
+      dot_chunk<T, U, 2, MODE, TWO, true>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
     else
-      for (; k0 < g.w; k0 += 4) dot_chunk<T, U, 4, MODE, TWO, true>(A, g, k0, lane, x1, x2, acc1, acc2);
+      for (int k0 = 0; k0 < g.w; k0 += 4) dot_chunk<T, U, 4, MODE, TWO, true>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
   } else {
-    for (; k0 + 2 <= g.w; k0 += 2) dot_chunk<T, U, 2, MODE, TWO, false>(A, g, k0, lane, x1, x2, acc1, acc2);
-    if (k0 < g.w) dot_chunk<T, U, 1, MODE, TWO, false>(A, g, k0, lane, x1, x2, acc1, acc2);
+    constexpr int W = 32 / U;  // a multiple of the chunks
+    for (int kw = 0;;) {
+      const int end = min(g.w, kw + W);
+      int k0 = kw;
+      for (; k0 + 2 <= end; k0 += 2)
+        dot_chunk<T, U, 2, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+      if (k0 < end) dot_chunk<T, U, 1, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+      kw += W;
+      if (kw >= g.w) break;
+      rw = run_words<T, U>(A, g, kw, lane);
+    }
   }
 }
 
 template <class T, int U, bool TWO>
-__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int2 ob, int lane,
+__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, const SliceSpan& g, int2 rw, int lane,
                                              const T* __restrict__ x1, const T* __restrict__ x2,
                                              T (&acc1)[U], T (&acc2)[U]) {
-  const SliceSpan g = slice_span<U>(ob);
 #pragma unroll
   for (int u = 0; u < U; ++u) acc1[u] = acc2[u] = 0;
   if (g.mode == kRunsOne)
-    sell_dot_mode<T, U, kRunsOne, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsOne, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsTwo)
-    sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+  else if (g.mode == kRunsMixed)
+    sell_dot_mode<T, U, kRunsMixed, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else
-    sell_dot_mode<T, U, kRunsNone, TWO>(A, g, 0, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsNone, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
 }
 
 template <class T, int U, int MINB>
@@ -111,7 +159,9 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
-  int2 ob = slice_offsets<T, U>(a.K, gw * U);  // matrix only: before the previous kernel ends
+  // matrix only: before the previous kernel ends
+  int2 ob = slice_offsets<T, U>(a.K, gw * U), nb = U == 1 ? ob : slice_offsets<T, U>(a.K, (gw + nw) * U);
+  int2 rw = run_words<T, U>(a.K, slice_span<U>(ob), 0, lane);
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ DualScalars<T> sc;
@@ -130,7 +180,9 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   // throughput on this GPU is ~1/60 of FP32); the step rule is a heuristic
   T acc_dy2 = 0, acc_int = 0;
   for (int s0 = gw * U; s0 < a.K.nslices; s0 += nw * U) {
-    const int2 nb = slice_offsets<T, U>(a.K, s0 + nw * U);  // next group, one iteration ahead
+    // next group's run words, the offsets of the one after it
+    const int2 nrw = run_words<T, U>(a.K, slice_span<U>(nb), 0, lane);
+    const int2 nnb = slice_offsets<T, U>(a.K, s0 + (U == 1 ? 1 : 2) * nw * U);
     const int i0 = s0 * kSlice + lane;
     // row operands do not depend on the product: load them first so their
     // latency overlaps the matrix stream (vectors are allocated in whole groups)
@@ -150,11 +202,13 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
 #pragma unroll
       for (int u = 0; u < U; ++u) ko[u] = a.Kx[p][i0 + u * kSlice];
       T unused[U];
-      sell_dot_pre<T, U, false>(a.K, ob, lane, xn, xn, kx, unused);
+      sell_dot_pre<T, U, false>(a.K, slice_span<U>(ob), rw, lane, xn, xn, kx, unused);
     } else {
-      sell_dot_pre<T, U, true>(a.K, ob, lane, xn, xc, kx, ko);
+      sell_dot_pre<T, U, true>(a.K, slice_span<U>(ob), rw, lane, xn, xc, kx, ko);
     }
-    ob = nb;
+    ob = U == 1 ? nnb : nb;
+    nb = nnb;
+    rw = nrw;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = i0 + u * kSlice;
@@ -190,7 +244,9 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBlock) >> 5;
-  int2 ob = slice_offsets<T, U>(a.KT, gw * U);  // matrix only: before the previous kernel ends
+  // matrix only: before the previous kernel ends
+  int2 ob = slice_offsets<T, U>(a.KT, gw * U), nb = U == 1 ? ob : slice_offsets<T, U>(a.KT, (gw + nw) * U);
+  int2 rw = run_words<T, U>(a.KT, slice_span<U>(ob), 0, lane);
   grid_wait_prior();
   DevState* st = a.st;
   __shared__ AdjScalars<T> sc;
@@ -208,7 +264,8 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
   T* __restrict__ xn = a.x[1 - p];
   T acc_dx2 = 0;
   for (int s0 = gw * U; s0 < a.KT.nslices; s0 += nw * U) {
-    const int2 nb = slice_offsets<T, U>(a.KT, s0 + nw * U);  // one iteration ahead
+    const int2 nrw = run_words<T, U>(a.KT, slice_span<U>(nb), 0, lane);
+    const int2 nnb = slice_offsets<T, U>(a.KT, s0 + (U == 1 ? 1 : 2) * nw * U);
     const int j0 = s0 * kSlice + lane;
     T x0[U], cj[U], lj[U], uj[U], xb[U], g[U];
 #pragma unroll
@@ -222,12 +279,14 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
     }
     if (acc_last) {
       T unused[U];
-      sell_dot_pre<T, U, false>(a.KT, ob, lane, yc, yc, g, unused);
+      sell_dot_pre<T, U, false>(a.KT, slice_span<U>(ob), rw, lane, yc, yc, g, unused);
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u) g[u] = kty[j0 + u * kSlice];
     }
-    ob = nb;
+    ob = U == 1 ? nnb : nb;
+    nb = nnb;
+    rw = nrw;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = j0 + u * kSlice;
@@ -298,7 +357,7 @@ __device__ __forceinline__ void staged_dot(const SellView<T>& A, const SliceStag
       if (TWO) a2[0] += st.v[e] * __ldg(x2 + st.c[e]);
     }
   for (int k0 = kStage; k0 < st.g.w; k0 += 4)
-    dot_chunk<T, 1, 4, kRunsNone, TWO, true>(A, st.g, k0, lane, x1, x2, a1, a2);
+    dot_chunk<T, 1, 4, kRunsNone, TWO, true>(A, st.g, int2{}, 0, k0, lane, x1, x2, a1, a2);
   acc1 = a1[0];
   acc2 = a2[0];
 }
@@ -517,7 +576,8 @@ __global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __
     const int r = (s0 + u) * kSlice + lane;
     to[u] = perm && r < A.rows ? __ldg(perm + r) : r;
   }
-  sell_dot_pre<T, U, false>(A, slice_offsets<T, U>(A, s0), lane, x, x, acc, unused);
+  const SliceSpan g = slice_span<U>(slice_offsets<T, U>(A, s0));
+  sell_dot_pre<T, U, false>(A, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int r = (s0 + u) * kSlice + lane;

@@ -1,10 +1,13 @@
 // Internal layout (length-sorted orderings, sliced ELL) and the rescaling pass.
 //
-// Rows of K are reordered by decreasing length inside the equality block and
-// inside the inequality block, columns by decreasing column count, so that each
-// 32-row slice holds rows of (nearly) equal length and padding stays negligible
-// on the UC sparsity (rows of 2 to ~25 entries); rows (columns) of one length are
-// grouped so that a slice's gathers are contiguous (order_by_signature).  K and
+// Rows of K are reordered by (about) decreasing length inside the equality block
+// and inside the inequality block, columns by decreasing column count, so that each
+// 32-row slice holds rows of (nearly) equal length and padding stays small on the
+// UC sparsity (rows of 2 to ~25 entries); rows (columns) of one kind stay together
+// in time order so that a slice's gathers are contiguous (build_layout): 3 % padding
+// on the 6717-bus day, 1 % with strictly equal lengths, but all k-columns of K and
+// nearly all of K^T are then runs instead of 58 % of the entries, which took the
+// FP32 sweeps from 39.7 + 29.5 to 36.9 + 22.8 us.  K and
 // K^T are both kept in this layout; every vector the iterations touch lives in
 // the internal order, so no permutation is applied inside the PDHG loop.
 //
@@ -16,6 +19,8 @@
 #include <algorithm>
 #include <cstring>
 #include <numeric>
+#include <system_error>
+#include <thread>
 
 #include "internal.cuh"
 
@@ -30,51 +35,91 @@ inline uint64_t mix64(uint64_t z) {
   return z ^ (z >> 31);
 }
 
-// Internal order of a set of rows (columns): by decreasing length, equal
-// lengths grouped by signature in the order the signatures first occur, equal
-// signatures in their original order.  perm receives `count` ids from `first`;
-// members (optional) the size of each id's group.
-void order_by_signature(int64_t first, int64_t count, const std::vector<int32_t>& len,
-                        const std::vector<uint64_t>& sig, int32_t* perm, int32_t* members) {
-  if (count == 0) return;
-  // group ids by first occurrence (open addressing; lengths are part of the key)
+// Groups of equal keys of the ids first, first + 1, ..., numbered by first
+// occurrence (open addressing).
+struct Groups {
+  std::vector<int32_t> of;          // group of each id
+  std::vector<int32_t> rep;         // a member
+  std::vector<int32_t> size, most;  // members, longest length
+  std::vector<int64_t> total;       // entries
+};
+Groups group_by(int64_t first, int64_t count, const std::vector<int32_t>& len, const std::vector<uint64_t>& key) {
+  Groups g;
   size_t cap = 16;
   while (cap < (size_t)count * 2) cap <<= 1;
-  std::vector<int32_t> table(cap, -1), gid(count), glen;
-  std::vector<int64_t> gsize;
-  std::vector<int64_t> grep;  // a member of the group
+  std::vector<int32_t> table(cap, -1);
+  g.of.resize(count);
   for (int64_t t = 0; t < count; ++t) {
     const int64_t i = first + t;
-    size_t h = mix64(sig[i] + (uint64_t)len[i]) & (cap - 1);
-    for (;; h = (h + 1) & (cap - 1)) {
-      const int32_t g = table[h];
-      if (g < 0) {
-        table[h] = gid[t] = (int32_t)glen.size();
-        glen.push_back(len[i]);
-        gsize.push_back(1);
-        grep.push_back(i);
-        break;
-      }
-      if (glen[g] == len[i] && sig[grep[g]] == sig[i]) {
-        gid[t] = g;
-        ++gsize[g];
-        break;
+    size_t h = mix64(key[i]) & (cap - 1);
+    while (table[h] >= 0 && key[g.rep[table[h]]] != key[i]) h = (h + 1) & (cap - 1);
+    if (table[h] < 0) {
+      table[h] = (int32_t)g.rep.size();
+      g.rep.push_back((int32_t)i);
+      g.size.push_back(0);
+      g.most.push_back(0);
+      g.total.push_back(0);
+    }
+    const int32_t q = table[h];
+    g.of[t] = q;
+    ++g.size[q];
+    g.most[q] = std::max(g.most[q], len[i]);
+    g.total[q] += len[i];
+  }
+  return g;
+}
+
+// Internal order of a set of rows (columns): groups of equal keys by decreasing
+// longest length, equal lengths as they first occur, members in their original
+// order.  A group whose members differ so much in length that padding them to the
+// longest would cost more than a quarter of its entries is split by length.
+void order_by_key(int64_t first, int64_t count, const std::vector<int32_t>& len, std::vector<uint64_t>& key,
+                  int32_t* perm) {
+  if (count == 0) return;
+  Groups g = group_by(first, count, len, key);
+  bool split = false;
+  for (int64_t t = 0; t < count; ++t) {
+    const int32_t q = g.of[t];
+    if ((int64_t)g.most[q] * g.size[q] * 4 > g.total[q] * 5) {
+      key[first + t] = mix64(key[first + t] + (uint64_t)len[first + t] + 1);
+      split = true;
+    }
+  }
+  if (split) g = group_by(first, count, len, key);
+  std::vector<int32_t> order(g.rep.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return g.most[a] > g.most[b]; });
+  std::vector<int64_t> pos(g.rep.size());
+  int64_t at = 0;
+  for (int32_t q : order) {
+    pos[q] = at;
+    at += g.size[q];
+  }
+  for (int64_t t = 0; t < count; ++t) perm[pos[g.of[t]]++] = (int32_t)(first + t);
+}
+
+// The distance between one column and the next of its group that more than half
+// of such pairs have: the columns per period of a time-expanded model.  0: none.
+int64_t period_of(const Groups& g, int64_t n) {
+  std::vector<int32_t> last(g.rep.size(), -1);
+  int64_t cand = 0, votes = 0, pairs = 0, hits = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    std::fill(last.begin(), last.end(), -1);
+    for (int64_t j = 0; j < n; ++j) {
+      const int32_t prev = last[g.of[j]];
+      last[g.of[j]] = (int32_t)j;
+      if (prev < 0) continue;
+      const int64_t d = j - prev;
+      if (pass == 0) {  // majority vote
+        if (votes == 0) cand = d;
+        votes += d == cand ? 1 : -1;
+      } else {
+        ++pairs;
+        hits += d == cand;
       }
     }
   }
-  std::vector<int32_t> order(glen.size());
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return glen[a] > glen[b]; });
-  std::vector<int64_t> pos(glen.size());
-  int64_t at = 0;
-  for (int32_t g : order) {
-    pos[g] = at;
-    at += gsize[g];
-  }
-  for (int64_t t = 0; t < count; ++t) {
-    perm[pos[gid[t]]++] = (int32_t)(first + t);
-    if (members) members[t] = (int32_t)gsize[gid[t]];
-  }
+  return hits * 2 > pairs && pairs * 2 > n ? cand : 0;
 }
 
 // Offsets of the 32-row slices over the internal order.  Slices come in aligned
@@ -100,38 +145,92 @@ int64_t slice_offsets_of(const std::vector<int32_t>& len, const std::vector<int3
   return ng * kGroup;
 }
 
-// Column runs of a sliced-ELL matrix (see SellView::runs).
+void size_slots(const std::vector<int32_t>& off, std::vector<int32_t>* col, std::vector<int32_t>* src,
+                std::vector<int32_t>* soff, std::vector<int32_t>* runs) {
+  col->assign(off.back(), 0);
+  src->assign(off.back(), -1);
+  soff->assign(off.begin(), off.end());
+  runs->assign((size_t)off.back() / kSlice * 2, 0);
+}
+
+// Entries of the rows into their slots.  A row shorter than its slice sits at the
+// front or at the back of its slots, whichever continues more of the previous
+// row's columns (the horizon cuts minimum up time rows at their front, the columns
+// of the same variables at their back).
+template <class Col, class Src>
+void place_entries(int64_t rows, const std::vector<int32_t>& perm, const std::vector<int32_t>& len,
+                   const std::vector<int32_t>& off, Col&& col_of, Src&& src_of, std::vector<int32_t>* col,
+                   std::vector<int32_t>* src) {
+  for (int64_t i = 0; i < rows; ++i) {
+    const int64_t s = i / kSlice, lane = i % kSlice;
+    const int32_t o = perm[i], n = len[o], w = (off[s + 1] - off[s]) / kSlice;
+    int32_t front = 0;
+    if (n < w && i > 0) {
+      const int64_t q = (i - 1) / kSlice, p0 = off[q] + (i - 1) % kSlice;
+      const int32_t pw = (off[q + 1] - off[q]) / kSlice;
+      int hits[2] = {0, 0};
+      for (int at = 0; at < 2; ++at)
+        for (int32_t k = 0; k < n; ++k) {
+          const int32_t t = k + (at ? w - n : 0);
+          if (t < pw && (*src)[p0 + (int64_t)t * kSlice] >= 0 &&
+              (*col)[p0 + (int64_t)t * kSlice] + 1 == col_of(o, k))
+            ++hits[at];
+        }
+      if (hits[1] > hits[0]) front = w - n;
+    }
+    if (n < w && i + 1 < rows && front == 0) {
+      // the first of a run has only its successor to go by: the row after it, if longer
+      const int32_t on = perm[i + 1], nn = len[on];
+      if (nn > n && nn <= w) {
+        int hits[2] = {0, 0};
+        for (int at = 0; at < 2; ++at)
+          for (int32_t k = 0; k < n; ++k)
+            if (col_of(o, k) + 1 == col_of(on, k + (at ? nn - n : 0))) ++hits[at];
+        if (hits[1] > hits[0]) front = w - n;
+      }
+    }
+    for (int32_t k = 0; k < n; ++k) {
+      const int64_t slot = off[s] + (int64_t)(front + k) * kSlice + lane;
+      (*col)[slot] = col_of(o, k);
+      (*src)[slot] = src_of(o, k);
+    }
+  }
+}
+
+// Column runs of a sliced-ELL matrix (see SellView::runs).  Groups with more than a
+// quarter of their k-columns in more than two runs keep to the indices.
 void build_runs(const std::vector<int32_t>& off, const std::vector<int32_t>& col,
                 const std::vector<int32_t>& src, int64_t ncols, std::vector<int32_t>* soff,
                 std::vector<int32_t>* runs) {
   const int64_t ns = (int64_t)off.size() - 1;
-  soff->assign(off.begin(), off.end());
-  runs->assign((size_t)off[ns] / kSlice * 2, 0);
+  if (ncols >= ((int64_t)1 << kRunBits)) return;
   for (int64_t g = 0; g < ns; g += kGroup) {
     const int64_t o0 = off[g], o1 = off[g + kGroup];
-    int mode = ncols < ((int64_t)1 << kRunBits) ? kRunsOne : kRunsNone;
-    for (int64_t o = o0; o < o1 && mode != kRunsNone; o += kSlice) {
+    int64_t two = 0, more = 0;
+    for (int64_t o = o0; o < o1; o += kSlice) {
       int32_t prev = -1, start[2] = {0, 0}, split = kSlice, pieces = 0;
       for (int lane = 0; lane < kSlice; ++lane) {
         // a padding slot (value 0) continues the run it follows, inside the vector
         int32_t c = col[o + lane];
         if (src[o + lane] < 0) c = (lane > 0 && prev + 1 < ncols) ? prev + 1 : 0;
         if (lane == 0 || c != prev + 1) {
-          if (pieces == 2) {
-            mode = kRunsNone;
-            break;
-          }
-          if (pieces == 1) {
-            split = lane;
-            mode = kRunsTwo;
-          }
-          start[pieces++] = c;
+          if (pieces < 2) start[pieces] = c;
+          if (++pieces == 2) split = lane;
         }
         prev = c;
+      }
+      if (pieces == 2) ++two;
+      if (pieces > 2) {
+        ++more;
+        split = 0;  // the indices
       }
       (*runs)[o / kSlice * 2] = start[0];
       (*runs)[o / kSlice * 2 + 1] = (int32_t)(((uint32_t)split << kRunBits) | (uint32_t)start[1]);
     }
+    const int mode = more * 4 > (o1 - o0) / kSlice ? kRunsNone
+                     : more                        ? kRunsMixed
+                     : two                         ? kRunsTwo
+                                                   : kRunsOne;
     for (int s = 0; s < kGroup; ++s) (*soff)[g + s] |= mode;
   }
 }
@@ -155,13 +254,10 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
   // signatures of its rows and its place in them.  In a time-expanded model the
   // rows of one line (unit, bus) share a signature over all periods, and so do
   // its columns, so equal signatures kept in their original order run through
-  // time and row r + 1 gathers column c + 1 where row r gathers column c.  Rows
-  // that differ only in the unit they belong to (minimum up times: all values
-  // +-1) are told apart by the signature of one of their columns, the one with
-  // the most members: the others may be the few of the first or last periods.
+  // time and row r + 1 gathers column c + 1 where row r gathers column c.
   for (int64_t i = 0; i < m; ++i) {
     rlen[i] = (int32_t)(rp[i + 1] - rp[i]);
-    uint64_t h = 0;
+    uint64_t h = (uint64_t)rlen[i];
     for (int64_t e = rp[i]; e < rp[i + 1]; ++e) {
       uint64_t bits;
       std::memcpy(&bits, &val[e], sizeof(bits));
@@ -170,18 +266,44 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
     rsig[i] = mix64(h);
     for (int64_t e = rp[i]; e < rp[i + 1]; ++e) csig[col[e]] += mix64(rsig[i] + (uint64_t)(e - rp[i]));
   }
-  std::vector<int32_t> members(n);
-  L->perm_col.resize(n);
-  order_by_signature(0, n, clen, csig, L->perm_col.data(), members.data());
-  for (int64_t i = 0; i < m; ++i) {
-    int32_t best = -1;
-    for (int64_t e = rp[i]; e < rp[i + 1]; ++e)
-      if (best < 0 || members[col[e]] > members[best]) best = col[e];
-    if (best >= 0) rsig[i] = mix64(rsig[i] + csig[best]);
+  const Groups cg = group_by(0, n, clen, csig);
+  const int64_t period = period_of(cg, n);
+  if (period > 1) {
+    // Columns of one place in the period, rows of one kind at one place: the
+    // places of their first, last and last but one column and the end values.
+    // These do not change where the horizon cuts a row short (minimum up and down
+    // times), so such rows and the columns that lose them keep their places in
+    // the run of their unit, padded, instead of scattering over the lengths.
+    for (int64_t j = 0; j < n; ++j) csig[j] = (uint64_t)(j % period);
+    for (int64_t i = 0; i < m; ++i) {
+      const int64_t b = rp[i], e = rp[i + 1];
+      uint64_t h = e > b ? 1 : 0;
+      if (e > b) {
+        uint64_t v0, v1;
+        std::memcpy(&v0, &val[b], sizeof(v0));
+        std::memcpy(&v1, &val[e - 1], sizeof(v1));
+        h = mix64(h + (uint64_t)(col[b] % period)) + v0;
+        h = mix64(h + (uint64_t)(col[e - 1] % period)) + v1;
+        if (e - b > 1) h = mix64(h + (uint64_t)(col[e - 2] % period));
+      }
+      rsig[i] = mix64(h);
+    }
+  } else {
+    // Rows that differ only in the unit they belong to are told apart by the
+    // signature of the column with the most members
+    for (int64_t i = 0; i < m; ++i) {
+      int32_t best = -1;
+      for (int64_t e = rp[i]; e < rp[i + 1]; ++e)
+        if (best < 0 || cg.size[cg.of[col[e]]] > cg.size[cg.of[best]]) best = col[e];
+      if (best >= 0) rsig[i] = mix64(rsig[i] + csig[best]);
+    }
+    for (int64_t j = 0; j < n; ++j) csig[j] = mix64(csig[j] + (uint64_t)clen[j]);
   }
   L->perm_row.resize(m);
-  order_by_signature(0, m_eq, rlen, rsig, L->perm_row.data(), nullptr);
-  order_by_signature(m_eq, m - m_eq, rlen, rsig, L->perm_row.data() + m_eq, nullptr);
+  order_by_key(0, m_eq, rlen, rsig, L->perm_row.data());
+  order_by_key(m_eq, m - m_eq, rlen, rsig, L->perm_row.data() + m_eq);
+  L->perm_col.resize(n);
+  order_by_key(0, n, clen, csig, L->perm_col.data());
   std::vector<int32_t> inv_row(m), inv_col(n);
   for (int64_t i = 0; i < m; ++i) inv_row[L->perm_row[i]] = (int32_t)i;
   for (int64_t j = 0; j < n; ++j) inv_col[L->perm_col[j]] = (int32_t)j;
@@ -192,23 +314,6 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
     *err = "padded nnz of K exceeds 2^31";
     return PDHG_ERR_UNSUPPORTED;
   }
-  int64_t tot = L->k_off[ks];
-  L->k_col.assign(tot, 0);
-  L->k_src.assign(tot, -1);
-  for (int64_t s = 0; s < ks; ++s) {
-    for (int lane = 0; lane < kSlice; ++lane) {
-      int64_t i = s * kSlice + lane;
-      if (i >= m) continue;
-      int32_t o = L->perm_row[i];
-      for (int32_t k = 0; k < rlen[o]; ++k) {
-        int64_t e = rp[o] + k;
-        int64_t slot = L->k_off[s] + (int64_t)k * kSlice + lane;
-        L->k_col[slot] = inv_col[col[e]];
-        L->k_src[slot] = (int32_t)e;
-      }
-    }
-  }
-
   // ---- K^T in sliced ELL over internal columns (entries by ascending row) ----
   std::vector<int64_t> cptr(n + 1, 0);
   for (int64_t j = 0; j < n; ++j) cptr[j + 1] = cptr[j] + clen[j];
@@ -227,23 +332,28 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
     *err = "padded nnz of K^T exceeds 2^31";
     return PDHG_ERR_UNSUPPORTED;
   }
-  tot = L->t_off[ts];
-  L->t_col.assign(tot, 0);
-  L->t_src.assign(tot, -1);
-  for (int64_t s = 0; s < ts; ++s) {
-    for (int lane = 0; lane < kSlice; ++lane) {
-      int64_t j = s * kSlice + lane;
-      if (j >= n) continue;
-      int32_t o = L->perm_col[j];
-      for (int64_t k = 0; k < clen[o]; ++k) {
-        int64_t slot = L->t_off[s] + k * kSlice + lane;
-        L->t_col[slot] = inv_row[crow[cptr[o] + k]];
-        L->t_src[slot] = csrc[cptr[o] + k];
-      }
+  size_slots(L->k_off, &L->k_col, &L->k_src, &L->k_soff, &L->k_runs);
+  size_slots(L->t_off, &L->t_col, &L->t_src, &L->t_soff, &L->t_runs);
+  // the two matrices side by side; nothing here allocates or throws
+  const auto fill_k = [&]() noexcept {
+    place_entries(
+        m, L->perm_row, rlen, L->k_off, [&](int64_t o, int32_t k) { return inv_col[col[rp[o] + k]]; },
+        [&](int64_t o, int32_t k) { return (int32_t)(rp[o] + k); }, &L->k_col, &L->k_src);
+    build_runs(L->k_off, L->k_col, L->k_src, n, &L->k_soff, &L->k_runs);
+  };
+  std::thread other;
+  if (col.size() > (1u << 18)) {  // below, starting a thread costs what it saves
+    try {
+      other = std::thread(fill_k);
+    } catch (const std::system_error&) {
     }
   }
-  build_runs(L->k_off, L->k_col, L->k_src, n, &L->k_soff, &L->k_runs);
+  if (!other.joinable()) fill_k();
+  place_entries(
+      n, L->perm_col, clen, L->t_off, [&](int64_t o, int32_t k) { return inv_row[crow[cptr[o] + k]]; },
+      [&](int64_t o, int32_t k) { return csrc[cptr[o] + k]; }, &L->t_col, &L->t_src);
   build_runs(L->t_off, L->t_col, L->t_src, m, &L->t_soff, &L->t_runs);
+  if (other.joinable()) other.join();
   return PDHG_OK;
 }
 
