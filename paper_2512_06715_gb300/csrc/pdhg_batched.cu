@@ -101,7 +101,6 @@ struct BGlobal {
   double infeas_eps;  // certificate tolerance of the infeasibility test (0: off)
   int32_t fold_every;  // a refinement round also ends after this many checks (0: off)
   int32_t n_real, all_done;
-  uint32_t counter, counter2;
 };
 
 template <int BP>
@@ -128,6 +127,7 @@ struct BArgs {
   BInst* inst;
   BGlobal* g;
   double* part;               // per-block partials
+  uint32_t* tier;             // arrivals of grid_inst_sum: the groups, each group's blocks (0 between kernels)
   volatile int32_t* cancel;
   unsigned long long cond;
   int32_t in_graph;
@@ -254,17 +254,45 @@ __device__ __forceinline__ void inst_final_sum(const double* part, int nblocks, 
   __syncthreads();
 }
 
-// Last-block detection shared by the kernels that finish with per-instance sums.
-__device__ __forceinline__ bool last_block(uint32_t* counter) {
+// True in the last of `count` blocks to arrive at *counter.
+__device__ __forceinline__ bool last_arrival(uint32_t* counter, unsigned count) {
   __shared__ int last;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    unsigned t = atomicAdd(counter, 1u);
-    last = (t == gridDim.x - 1);
+    last = atomicAdd(counter, 1u) == count - 1;
+    if (last) *counter = 0;  // everyone has arrived: ready for the next kernel
   }
   __syncthreads();
   return last != 0;
+}
+
+// Per-instance sums over the grid of what block_inst_sum left in part[block]: true
+// in one block, whose threads t < BP then hold them.  One block adding up the whole
+// grid is bound by its FP64 pipe (two lanes a clock: 34 ns per block of 64 x 2
+// values, 5 us of the 33 us of K x' for 64 node LPs of 200 buses at 152 blocks, and
+// it kept the sweeps from more blocks), so the last of every kTier blocks adds up
+// those, on its own SM, and the last of these the groups'.  Fixed order.
+// Now 20.0 us at 304 blocks, K^T y' 25.5 -> 16.6; 9 node LPs of 24 buses 17.5 -> 13.2 ms
+// for 512 attempts.
+constexpr int kTier = 16;
+constexpr int kTierCount = 1 + (kMaxBlocks + kTier - 1) / kTier;
+constexpr size_t kTierSums = (size_t)kMaxBlocks * 64 * 3;  // of `part`, behind the blocks' own
+template <int BP, int NV>
+__device__ __forceinline__ bool grid_inst_sum(double* part, uint32_t* tier, double* smem, double (&tot)[NV]) {
+  static_assert(BP * NV <= 64 * 3, "fits before kTierSums");
+  const unsigned grp = blockIdx.x / kTier, groups = (gridDim.x + kTier - 1) / kTier;
+  const unsigned cnt = min((unsigned)kTier, gridDim.x - grp * kTier);
+  if (!last_arrival(tier + 1 + grp, cnt)) return false;
+  inst_final_sum<BP, NV>(part + (size_t)grp * kTier * BP * NV, cnt, smem, tot);
+  if (groups == 1) return true;
+  double* sums = part + kTierSums;
+  if (threadIdx.x < BP)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sums[((size_t)grp * BP + threadIdx.x) * NV + k] = tot[k];
+  if (!last_arrival(tier, groups)) return false;
+  inst_final_sum<BP, NV>(sums, groups, smem, tot);
+  return true;
 }
 
 // ---------------------------------------------------------------- attempt kernels
@@ -306,7 +334,7 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
   // Where a lane's instances agree on what they do and on their buffers (always
   // with one instance per lane; with two until a step of one is rejected) every
   // access is one of the lane's pair; else they go one by one.  64 node LPs of 6049
-  // buses x 48 periods: 615 us in pairs (1.25 ms with K^T y' before, 1.07 now), of
+  // buses x 48 periods: 576 us in pairs (1.25 ms with K^T y' one by one, 1.03 now), of
   // 455 us for the vectors alone at the copy bandwidth.
   const int nq = (a.m + RW - 1) / RW;
   auto sweep = [&](auto paired) {
@@ -408,14 +436,14 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
     v[h][1] = (double)a_int[h];
   }
   block_inst_sum<BP, 2, kBWarps>(v, smem, a.part);
-  if (last_block(&g->counter)) {
-    double tot[2], down = 0.0, up = 0.0;
+  double tot[2];
+  if (grid_inst_sum<BP, 2>(a.part, a.tier, smem, tot)) {
+    double down = 0.0, up = 0.0;
     if (threadIdx.x < BP) {  // does not depend on the sums
       const int64_t k = a.inst[threadIdx.x].k_total + 2;
       down = 1.0 - step_power(k, g->red_exp);
       up = 1.0 + step_power(k, g->grow_exp);
     }
-    inst_final_sum<BP, 2>(a.part, gridDim.x, smem, tot);
     if (threadIdx.x < BP) {
       const int b = threadIdx.x;
       BInst& I = a.inst[b];
@@ -445,7 +473,6 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
         I.sigma = (float)(eta_next * omega);
       }
     }
-    if (threadIdx.x == 0) g->counter = 0;
   }
 }
 
@@ -576,14 +603,12 @@ __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
 #pragma unroll
   for (int h = 0; h < H; ++h) v[h][0] = (double)a_dx2[h];
   block_inst_sum<BP, 1, kBWarps>(v, smem, a.part);
-  if (last_block(&g->counter)) {
-    double tot[1];
-    inst_final_sum<BP, 1>(a.part, gridDim.x, smem, tot);
+  double tot[1];
+  if (grid_inst_sum<BP, 1>(a.part, a.tier, smem, tot)) {
     if (threadIdx.x < BP) {
       const int b = threadIdx.x;
       if (a.inst[b].act) a.inst[b].dx2 = tot[0];
     }
-    if (threadIdx.x == 0) g->counter = 0;
   }
 }
 
@@ -1227,9 +1252,8 @@ __global__ void __launch_bounds__(kApplyRows * BP) kb_apply(BArgs<BP> a) {
     out[1] = s1;
     out[2] = s2;
   }
-  if (last_block(&g->counter2)) {
-    double tot[3];
-    inst_final_sum<BP, 3>(a.part, gridDim.x, smem, tot);
+  double tot[3];
+  if (grid_inst_sum<BP, 3>(a.part, a.tier, smem, tot)) {
     if (threadIdx.x < BP) {
       BInst& J = a.inst[threadIdx.x];
       if (J.restart_now || J.refine || J.finalize) {
@@ -1252,7 +1276,6 @@ __global__ void __launch_bounds__(kApplyRows * BP) kb_apply(BArgs<BP> a) {
       J.refine = 0;
       J.finalize = 0;
     }
-    if (threadIdx.x == 0) g->counter2 = 0;
   }
 }
 
@@ -1406,16 +1429,16 @@ __global__ void __launch_bounds__(kBThreads) kb_output(const double* __restrict_
   }
 }
 
-__global__ void kb_init_state(BInst* inst, BGlobal* g, int B, int BP, const double* scalars,
+__global__ void kb_init_state(BInst* inst, BGlobal* g, uint32_t* tier, int B, int BP, const double* scalars,
                               BGlobal gin) {
   const int b = threadIdx.x;
+  for (int t = b; t < kTierCount; t += blockDim.x) tier[t] = 0;
   if (b == 0) {
     *g = gin;
     g->t_start = globaltimer_ns();
     g->qnorm = scalars[2];
     g->cnorm = scalars[3];
     g->all_done = 0;
-    g->counter = g->counter2 = 0;
   }
   if (b < BP) {
     BInst I;
@@ -1445,6 +1468,7 @@ struct Batched {
   int32_t* done_host = nullptr;  // pinned copy of g->all_done (host-loop mode)
   BGlobal* g = nullptr;
   double* part = nullptr;
+  uint32_t* tier = nullptr;
   int32_t *inv_row = nullptr, *inv_col = nullptr;  // original -> internal
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1505,6 +1529,7 @@ int setup_batched(Workspace* w, Batched* bt, BArgs<BP>* out) {
   if (e == cudaSuccess) e = balloc(bt, &bt->inst, BP);
   if (e == cudaSuccess) e = balloc(bt, &bt->g, 1);
   if (e == cudaSuccess) e = balloc(bt, &bt->part, (size_t)3 * 8192 * 64 * 20);
+  if (e == cudaSuccess) e = balloc(bt, &bt->tier, kTierCount);
   if (e == cudaSuccess) e = balloc(bt, &bt->inv_row, w->m);
   if (e == cudaSuccess) e = balloc(bt, &bt->inv_col, w->n);
   if (e != cudaSuccess) {
@@ -1532,6 +1557,7 @@ int setup_batched(Workspace* w, Batched* bt, BArgs<BP>* out) {
   a.inst = bt->inst;
   a.g = bt->g;
   a.part = bt->part;
+  a.tier = bt->tier;
   a.cancel = w->opts.cancel_flag;
   *out = a;
   const int sms = w->num_sms;
@@ -1634,7 +1660,7 @@ void batched_start(Workspace* w, Batched* bt, const BArgs<BP>& a, int B, const d
   gin.infeas_eps = o.infeas_tol > 0.0 ? std::max(o.infeas_tol, kFp32RayTol) : 0.0;  // FP32 iterates
   gin.fold_every = o.ir_fold_checks;
   gin.n_real = B;
-  kb_init_state<<<1, BP < 32 ? 32 : BP, 0, s>>>(bt->inst, bt->g, B, BP, w->scalars, gin);
+  kb_init_state<<<1, BP < 32 ? 32 : BP, 0, s>>>(bt->inst, bt->g, bt->tier, B, BP, w->scalars, gin);
   const int gv = std::min(w->num_sms * 8, 8192);
   const int gt = (int)std::min<int64_t>((w->n + kTile - 1) / kTile, gv);
   kb_setup_cols<BP><<<gt, kBThreads, 0, s>>>(a, l_b, u_b, w->prob.l, w->prob.u, bt->inv_col, w->Dc, w->c_s, w->l_s,
