@@ -211,6 +211,20 @@ __device__ __forceinline__ bool finite_bits(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
 
+// max as fmax gives it (the other operand where one is NaN) in integer
+// instructions: an FP64 compare holds the FP64 pipe (two lanes a clock) for 16 clocks
+__device__ __forceinline__ bool is_nan_bits(double v) {
+  return (unsigned long long)(__double_as_longlong(v) & 0x7fffffffffffffffLL) > 0x7ff0000000000000ULL;
+}
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double max_of(double v, double w) {
+  return is_nan_bits(w) || (!is_nan_bits(v) && order_key(v) >= order_key(w)) ? v : w;
+}
+__device__ __forceinline__ float max_of(float v, float w) { return max(v, w); }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
