@@ -27,8 +27,12 @@ namespace ucpdhg {
 // What bounds these sweeps is not DRAM but the instructions and dependent round
 // trips per 32 rows (the time per row is the same for a matrix that stays in L2),
 // so a warp takes U slices whose entries and operand rows lie at fixed distances:
-// loads without predicates or address arithmetic of their own, U E entries and
-// 4 U (5 U) operands in flight before the dependent gathers.
+// loads without predicates or address arithmetic of their own, U E entries, their
+// gathers and 4 U (5 U) operands in flight together.  Warps in flight count as much:
+// chunks of E = 4 at U = 2 spill at 64 registers (44.5 us for K x' of the 6717-bus
+// day) and lose a quarter of the warps at 80 (44.9).  With column runs and the order
+// of build_layout, FP32, 6717-bus 96-period day: K x' 49.3 -> 36.9 us, K^T y' 36.5 ->
+// 22.8 us; FP64 107 -> 83 and 61 -> 51 us, where the FP64 pipe is the bound.
 //
 // soff[s0] and soff[s0 + U] (clamped past the end, giving empty slices).  The
 // per-attempt kernels load the NEXT group's offsets one iteration ahead, so this
