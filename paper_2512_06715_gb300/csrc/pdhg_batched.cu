@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(kKktWarps * 32) kb_kkt_row(BArgs<BP> a, int in
     store_inst<H, double>(a.Kzc, idx, d0, on);
     store_inst<H, double>(a.Kza, idx, d1, on);
     if (init) store_inst<H, double>(a.Kxa, idx, d0, on);
-    bool live = false;
+    bool live = !finite_bits(qo);  // seen in q y alone (as in the single-instance check)
 #pragma unroll
     for (int h = 0; h < H; ++h) {
       double r0 = on[h] ? qr[h] - d0[h] : 0.0, r1 = on[h] ? qr[h] - d1[h] : 0.0;

@@ -164,8 +164,10 @@ __global__ void __launch_bounds__(kBlock) k_kkt_row(IterArgs<T> a, int init) {
       }
     }
     // dual side: nothing to add where the row has never had a dual since the
-    // last restart
-    const bool live = non_zero(yo) || non_zero(yb) || non_zero(yb64) || non_zero(ya);
+    // last restart.  A NaN or an infinity in q counts as one: pos_part and the
+    // projection of y drop it, so q y is the only sum that shows it to k_control.
+    const bool live =
+        non_zero(yo) || non_zero(yb) || non_zero(yb64) || non_zero(ya) || !finite_bits(qo);
     if (__any_sync(0xffffffffu, live)) {
       if (pw != 0.0) {
         yb = yb + pwT * yo;
