@@ -295,6 +295,14 @@ int pdhg_rescale_noalloc(const pdhg_problem *prob, int32_t ruiz_iters, int32_t p
 
 /* ---- diagnostics (kernel-level tests and measurement) -------------------- */
 
+/* Value slots that a workspace's layout of an LP takes for K and for K^T,
+ * padding included (a workspace holds 20 bytes per slot of either, and a slot
+ * count of 2^31 or more is refused by pdhg_workspace_create with
+ * PDHG_ERR_UNSUPPORTED, here too).  The CSR of `pdhg_problem` in host memory:
+ * row_ptr [m+1], col and val [row_ptr[m]].  Host work only. */
+int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64_t *row_ptr, const int32_t *col,
+                      const double *val, int64_t *slots_k, int64_t *slots_kt);
+
 /* Load the values and run the rescaling of a solve without iterating. */
 int pdhg_prepare(void *ws, void *stream);
 

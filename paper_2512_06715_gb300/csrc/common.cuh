@@ -27,13 +27,14 @@ constexpr int kRsSlices = 32;        // slices per chunk of the row-staged kerne
 // infeasibility direction; FP32 iterations therefore test rays at
 // max(infeas_tol, kFp32RayTol).
 constexpr double kFp32RayTol = 1e-6;
-constexpr int kGroup = 4;        // slices per aligned group of one width
+constexpr int kGroup = 4;        // slices per aligned group, of one width unless kRunsOwn
 constexpr int kRunBits = 26;     // bits of a column index in the second word of a column run
 // low bits of SellView::soff, one value per group of slices
 constexpr int kRunsNone = 0;     // explicit column indices
 constexpr int kRunsTwo = 1;      // every k-column is one or two runs
 constexpr int kRunsMixed = 3;    // most are, the others have split 0: take the indices
 constexpr int kRunsOne = 2;      // every k-column is one run
+constexpr int kRunsOwn = 4;      // slices of their own widths, explicit column indices
 constexpr int kTraceCheckCols = 12;  // values recorded per KKT check in the trace
 
 // Sliced ELL with 32-row slices over the internal (length-sorted) row order.
@@ -53,8 +54,10 @@ struct SellView {
   // runs[off/32 + k] then replaces the 128 B of indices by 8 B: lanes below `split`
   // gather x + lane, the others y + lane - split, with y in the low kRunBits bits
   // of the second word and split above them.  Split 0: this k-column has more runs.
+  // kRunsOwn: the group's slices differ in width (a row far longer than the rest).
   const int32_t* soff;  // [nslices + 1]
   const int2* runs;     // [nnz_pad / 32]
+  int32_t own;          // some groups are kRunsOwn
 };
 
 __device__ __forceinline__ int run_split(int2 r) { return (int)((unsigned)r.y >> kRunBits); }

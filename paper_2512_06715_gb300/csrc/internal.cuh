@@ -24,8 +24,9 @@ struct DevSell {
   int32_t nchunks2 = 0;
   int32_t* soff = nullptr;  // column runs (SellView)
   int32_t* runs = nullptr;
-  SellView<double> v64() const { return {off, col, val64, nslices, rows, soff, (const int2*)runs}; }
-  SellView<float> v32() const { return {off, col, val32, nslices, rows, soff, (const int2*)runs}; }
+  int32_t own = 0;  // some groups of slices have no common width
+  SellView<double> v64() const { return {off, col, val64, nslices, rows, soff, (const int2*)runs, own}; }
+  SellView<float> v32() const { return {off, col, val32, nslices, rows, soff, (const int2*)runs, own}; }
 };
 
 // Iterate buffers of one precision.
@@ -50,11 +51,16 @@ struct HostLayout {
   std::vector<int32_t> k_off, k_col, k_src;
   std::vector<int32_t> t_off, t_col, t_src;
   std::vector<int32_t> k_soff, k_runs, t_soff, t_runs;  // column runs (SellView)
+  int32_t k_own = 0, t_own = 0;                         // SellView::own
 };
 
 int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& row_ptr,
                  const std::vector<int32_t>& col, const std::vector<double>& val, HostLayout* out,
                  std::string* err);
+// Value slots (padding included) of K and of K^T in that layout.
+int count_slots(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& row_ptr,
+                const std::vector<int32_t>& col, const std::vector<double>& val, int64_t* slots_k, int64_t* slots_kt,
+                std::string* err);
 
 // Per-round initialisation of the device state.
 struct RoundInit {

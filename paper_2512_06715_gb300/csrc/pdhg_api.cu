@@ -728,9 +728,11 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   w->K.nslices = (int32_t)(L.k_off.size() - 1);
   w->K.rows = (int32_t)w->m;
   w->K.nnz_pad = L.k_col.size();
+  w->K.own = L.k_own;
   w->KT.nslices = (int32_t)(L.t_off.size() - 1);
   w->KT.rows = (int32_t)w->n;
   w->KT.nnz_pad = L.t_col.size();
+  w->KT.own = L.t_own;
   std::vector<int32_t> kch, tch;
   if (build_chunks(L.k_off, &kch, kStageEntries, 1 << 30) && build_chunks(L.t_off, &tch, kStageEntries, 1 << 30)) {
     w->K.nchunks = (int32_t)kch.size() - 1;
@@ -811,6 +813,24 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   if (cudaDeviceSynchronize() != cudaSuccess) return bail(fail(PDHG_ERR_CUDA, "setup failed"));
   *out = w;
   return PDHG_OK;
+}
+
+extern "C" int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64_t* row_ptr, const int32_t* col,
+                                 const double* val, int64_t* slots_k, int64_t* slots_kt) {
+  g_err.clear();
+  if (!row_ptr || !slots_k || !slots_kt) return fail(PDHG_ERR_INVALID_ARG, "NULL argument");
+  if (n < 1 || m < 1 || m_eq < 0 || m_eq > m || n >= ((int64_t)1 << 31) - 64 || m >= ((int64_t)1 << 31) - 64)
+    return fail(PDHG_ERR_INVALID_ARG, "problem sizes: need 1 <= n, m < 2^31 and 0 <= m_eq <= m");
+  const std::vector<int64_t> rp(row_ptr, row_ptr + m + 1);
+  const int64_t nnz = rp[m];
+  if (rp[0] != 0 || nnz < 0 || nnz >= ((int64_t)1 << 31) || (nnz > 0 && (!col || !val)))
+    return fail(PDHG_ERR_INVALID_ARG, "row_ptr inconsistent");
+  for (int64_t i = 0; i < m; ++i)
+    if (rp[i + 1] < rp[i]) return fail(PDHG_ERR_INVALID_ARG, "row_ptr not monotone");
+  std::string err;
+  const int rc = count_slots(n, m, m_eq, rp, std::vector<int32_t>(col, col + nnz),
+                             std::vector<double>(val, val + nnz), slots_k, slots_kt, &err);
+  return rc == PDHG_OK ? rc : fail(rc, err);
 }
 
 static void drop_graphs(Workspace* w) {

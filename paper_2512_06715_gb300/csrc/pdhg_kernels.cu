@@ -19,8 +19,8 @@
 namespace ucpdhg {
 
 // Row dot products of U consecutive slices (U = 1, or 2 or 4 slices of one group:
-// one width w) with x1 and, if TWO, with x2 in the same matrix pass; lane = row
-// within each slice.  The columns of a slice come from its runs (8 B per 32
+// one width w unless kRunsOwn) with x1 and, if TWO, with x2 in the same matrix pass;
+// lane = row within each slice.  The columns of a slice come from its runs (8 B per 32
 // entries: the gather is then one or two contiguous pieces and needs no index
 // load of its own) or, where it has none, from the explicit indices.
 //
@@ -141,8 +141,32 @@ __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceS
   }
 }
 
+// Slices of their own widths (groups with a row far longer than the rest), one after
+// the other, eight unpredicated entries in flight: such a row is a serial chain of its
+// warp (K x of the 4224-bus, 18-period day with a row of 20000 entries: 1.74 ms; 2.5 ms
+// with predicated chunks of four, 6.4 ms where the row widens its whole group).  Only
+// compiled into the kernels for matrices with such groups (OWN): in the others it
+// would cost 1 % (FP32 K x' of the 6717-bus day 36.9 -> 37.2 us, its FP64 solve 73.6 ->
+// 74.4 ms).
 template <class T, int U, bool TWO>
-__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, const SliceSpan& g, int2 rw, int lane,
+__device__ __forceinline__ void sell_dot_own(const SellView<T>& A, int s0, int lane, const T* __restrict__ x1,
+                                             const T* __restrict__ x2, T (&acc1)[U], T (&acc2)[U]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const SliceSpan g = slice_span<1>(slice_offsets<T, 1>(A, s0 + u));
+    T a1[1] = {0}, a2[1] = {0};
+    int k0 = 0;
+    for (; k0 + 8 <= g.w; k0 += 8)
+      dot_chunk<T, 1, 8, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+    for (; k0 < g.w; ++k0) dot_chunk<T, 1, 1, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+    acc1[u] = a1[0];
+    acc2[u] = a2[0];
+  }
+}
+
+// s0: the first of the U slices, g: their span.
+template <class T, int U, bool TWO, bool OWN>
+__device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int s0, const SliceSpan& g, int2 rw, int lane,
                                              const T* __restrict__ x1, const T* __restrict__ x2,
                                              T (&acc1)[U], T (&acc2)[U]) {
 #pragma unroll
@@ -153,11 +177,13 @@ __device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, const SliceSp
     sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsMixed)
     sell_dot_mode<T, U, kRunsMixed, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+  else if (OWN && g.mode == kRunsOwn)
+    sell_dot_own<T, U, TWO>(A, s0, lane, x1, x2, acc1, acc2);
   else
     sell_dot_mode<T, U, kRunsNone, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
 }
 
-template <class T, int U, int MINB>
+template <class T, int U, int MINB, bool OWN = false>
 __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   grid_launch_dependents();
   const int lane = threadIdx.x & 31;
@@ -206,9 +232,9 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
 #pragma unroll
       for (int u = 0; u < U; ++u) ko[u] = a.Kx[p][i0 + u * kSlice];
       T unused[U];
-      sell_dot_pre<T, U, false>(a.K, slice_span<U>(ob), rw, lane, xn, xn, kx, unused);
+      sell_dot_pre<T, U, false, OWN>(a.K, s0, slice_span<U>(ob), rw, lane, xn, xn, kx, unused);
     } else {
-      sell_dot_pre<T, U, true>(a.K, slice_span<U>(ob), rw, lane, xn, xc, kx, ko);
+      sell_dot_pre<T, U, true, OWN>(a.K, s0, slice_span<U>(ob), rw, lane, xn, xc, kx, ko);
     }
     ob = U == 1 ? nnb : nb;
     nb = nnb;
@@ -251,7 +277,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_dual(IterArgs<T> a) {
   }
 }
 
-template <class T, int U, int MINB>
+template <class T, int U, int MINB, bool OWN = false>
 __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
   grid_launch_dependents();
   const int lane = threadIdx.x & 31;
@@ -292,7 +318,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_adjoint(IterArgs<T> a) {
     }
     if (acc_last) {
       T unused[U];
-      sell_dot_pre<T, U, false>(a.KT, slice_span<U>(ob), rw, lane, yc, yc, g, unused);
+      sell_dot_pre<T, U, false, OWN>(a.KT, s0, slice_span<U>(ob), rw, lane, yc, yc, g, unused);
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u) g[u] = kty[j0 + u * kSlice];
@@ -576,7 +602,7 @@ __global__ void k_init_vectors(IterArgs<T> a) {
 // (pdhg_apply_K: the unscrambling, and for FP32 the widening, in the same pass).
 // Two slices per warp, one pass over the matrix without a loop: a sweep this
 // short is all latency.
-template <class T, int U>
+template <class T, int U, bool OWN>
 __global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __restrict__ x, T* __restrict__ y,
                                                       const int32_t* __restrict__ perm, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
@@ -590,7 +616,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __
     to[u] = perm && r < A.rows ? __ldg(perm + r) : r;
   }
   const SliceSpan g = slice_span<U>(slice_offsets<T, U>(A, s0));
-  sell_dot_pre<T, U, false>(A, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
+  sell_dot_pre<T, U, false, OWN>(A, s0, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int r = (s0 + u) * kSlice + lane;
@@ -683,7 +709,8 @@ template <class T>
 static void spmv_any(const SellView<T>& A, const T* x, T* y, const int32_t* perm, double* out, cudaStream_t s) {
   const int64_t warps = (A.nslices + 1) / 2;
   const unsigned grid = (unsigned)((warps + kWarps - 1) / kWarps);
-  k_spmv_into<T, 2><<<grid < 1 ? 1 : grid, kBlock, 0, s>>>(A, x, y, perm, out);
+  const auto kernel = A.own ? k_spmv_into<T, 2, true> : k_spmv_into<T, 2, false>;
+  kernel<<<grid < 1 ? 1 : grid, kBlock, 0, s>>>(A, x, y, perm, out);
 }
 
 template <class T>
@@ -749,10 +776,12 @@ static void launch_iter(void (*k)(IterArgs<T>), const IterArgs<T>& a, int grid, 
 
 template <class T>
 void launch_dual(const IterArgs<T>& a, int grid, cudaStream_t s, int unroll) {
+  constexpr int B = MinBlocks<T, 2>::value;
+  static_assert(B == MinBlocks<T, 4>::value, "variants 2 and 4 share it");
   switch (unroll) {
     case 0: launch_iter<T>(k_dual_pipe<T, MinBlocksPipe<T>::value>, a, grid, s); break;
-    case 2: launch_iter<T>(k_dual<T, 2, MinBlocks<T, 2>::value>, a, grid, s); break;
-    case 4: launch_iter<T>(k_dual<T, 4, MinBlocks<T, 4>::value>, a, grid, s); break;
+    case 2: launch_iter<T>(a.K.own ? k_dual<T, 2, B, true> : k_dual<T, 2, B>, a, grid, s); break;
+    case 4: launch_iter<T>(a.K.own ? k_dual<T, 4, B, true> : k_dual<T, 4, B>, a, grid, s); break;
     case 8: launch_iter<T>(k_dual<T, 1, 8>, a, grid, s); break;
     case 9: launch_iter<T>(k_dual_pipe<T, 8>, a, grid, s); break;
     case 16: launch_dual_staged<T>(a, grid, s, 1); break;
@@ -767,10 +796,11 @@ void launch_dual(const IterArgs<T>& a, int grid, cudaStream_t s, int unroll) {
 
 template <class T>
 void launch_adjoint(const IterArgs<T>& a, int grid, cudaStream_t s, int unroll) {
+  constexpr int B = MinBlocks<T, 2>::value;
   switch (unroll) {
     case 0: launch_iter<T>(k_adjoint_pipe<T, MinBlocksPipe<T>::value>, a, grid, s); break;
-    case 2: launch_iter<T>(k_adjoint<T, 2, MinBlocks<T, 2>::value>, a, grid, s); break;
-    case 4: launch_iter<T>(k_adjoint<T, 4, MinBlocks<T, 4>::value>, a, grid, s); break;
+    case 2: launch_iter<T>(a.KT.own ? k_adjoint<T, 2, B, true> : k_adjoint<T, 2, B>, a, grid, s); break;
+    case 4: launch_iter<T>(a.KT.own ? k_adjoint<T, 4, B, true> : k_adjoint<T, 4, B>, a, grid, s); break;
     case 8: launch_iter<T>(k_adjoint<T, 1, 8>, a, grid, s); break;
     case 9: launch_iter<T>(k_adjoint_pipe<T, 8>, a, grid, s); break;
     case 16: launch_adjoint_staged<T>(a, grid, s, 1); break;

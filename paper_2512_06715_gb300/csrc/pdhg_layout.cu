@@ -124,20 +124,35 @@ int64_t period_of(const Groups& g, int64_t n) {
 
 // Offsets of the 32-row slices over the internal order.  Slices come in aligned
 // groups of kGroup of one width, so that a warp sweeping a group (or half of one)
-// finds its entries at fixed distances.  Returns the number of slices (a multiple
-// of kGroup), -1 if the entries exceed 2^31.
-int64_t slice_offsets_of(const std::vector<int32_t>& len, const std::vector<int32_t>& perm,
+// finds its entries at fixed distances.  A group whose slices keep their own widths
+// (own, or where the common one would add more than a quarter to its slots and more
+// than kOwnPadding k-columns: a row far longer than its neighbours, such as a budget
+// or reserve row, would pad 128 rows instead of 32) is swept slice by slice: 40000
+// columns and one full row take 1.4 instead of 5.2 million slots.  The second
+// condition leaves rows of up to 42 entries in groups of one width whatever their
+// neighbours (all of the scheduling LPs here: 28 at most).  Returns the number of slices (a multiple of kGroup), -1 if the
+// entries exceed 2^31.
+constexpr int64_t kOwnPadding = 128;
+int64_t slice_offsets_of(const std::vector<int32_t>& len, const std::vector<int32_t>& perm, bool own,
                          std::vector<int32_t>* off) {
   const int64_t rows = (int64_t)perm.size();
   const int64_t ng = (rows + kSlice * kGroup - 1) / (kSlice * kGroup);
   off->assign(ng * kGroup + 1, 0);
   int64_t tot = 0;
   for (int64_t g = 0; g < ng; ++g) {
-    int32_t w = 0;
-    const int64_t end = std::min(rows, (g + 1) * kSlice * kGroup);
-    for (int64_t i = g * kSlice * kGroup; i < end; ++i) w = std::max(w, len[perm[i]]);
+    int32_t w[kGroup], most = 0;
+    int64_t sum = 0;
     for (int s = 0; s < kGroup; ++s) {
-      tot += (int64_t)w * kSlice;
+      const int64_t first = (g * kGroup + s) * kSlice;
+      w[s] = 0;
+      for (int64_t i = first; i < std::min(rows, first + kSlice); ++i) w[s] = std::max(w[s], len[perm[i]]);
+      most = std::max(most, w[s]);
+      sum += w[s];
+    }
+    const int64_t pad = (int64_t)most * kGroup - sum;
+    const bool one = !own && (pad * 4 <= sum || pad <= kOwnPadding);
+    for (int s = 0; s < kGroup; ++s) {
+      tot += (int64_t)(one ? most : w[s]) * kSlice;
       if (tot >= (int64_t)1 << 31) return -1;
       (*off)[g * kGroup + s + 1] = (int32_t)tot;
     }
@@ -145,12 +160,21 @@ int64_t slice_offsets_of(const std::vector<int32_t>& len, const std::vector<int3
   return ng * kGroup;
 }
 
-void size_slots(const std::vector<int32_t>& off, std::vector<int32_t>* col, std::vector<int32_t>* src,
+// Returns whether some groups keep a width per slice.
+bool size_slots(const std::vector<int32_t>& off, std::vector<int32_t>* col, std::vector<int32_t>* src,
                 std::vector<int32_t>* soff, std::vector<int32_t>* runs) {
   col->assign(off.back(), 0);
   src->assign(off.back(), -1);
-  soff->assign(off.begin(), off.end());
   runs->assign((size_t)off.back() / kSlice * 2, 0);
+  soff->assign(off.begin(), off.end());
+  bool any = false;
+  for (size_t g = 0; g + kGroup < off.size(); g += kGroup) {
+    bool own = false;
+    for (int s = 1; s < kGroup; ++s) own = own || off[g + s + 1] - off[g + s] != off[g + 1] - off[g];
+    for (int s = 0; own && s < kGroup; ++s) (*soff)[g + s] |= kRunsOwn;
+    any = any || own;
+  }
+  return any;
 }
 
 // Entries of the rows into their slots.  A row shorter than its slice sits at the
@@ -206,6 +230,7 @@ void build_runs(const std::vector<int32_t>& off, const std::vector<int32_t>& col
   if (ncols >= ((int64_t)1 << kRunBits)) return;
   for (int64_t g = 0; g < ns; g += kGroup) {
     const int64_t o0 = off[g], o1 = off[g + kGroup];
+    if (((*soff)[g] & (kSlice - 1)) == kRunsOwn) continue;
     int64_t two = 0, more = 0;
     for (int64_t o = o0; o < o1; o += kSlice) {
       int32_t prev = -1, start[2] = {0, 0}, split = kSlice, pieces = 0;
@@ -235,12 +260,14 @@ void build_runs(const std::vector<int32_t>& off, const std::vector<int32_t>& col
   }
 }
 
-}  // namespace
-
-int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& rp,
+// The internal order of rows and columns and the slices' offsets; rlen and clen
+// receive the lengths.
+int order_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& rp,
                  const std::vector<int32_t>& col, const std::vector<double>& val, HostLayout* L,
-                 std::string* err) {
-  std::vector<int32_t> rlen(m), clen(n, 0);
+                 std::vector<int32_t>* rlen_out, std::vector<int32_t>* clen_out, std::string* err) {
+  std::vector<int32_t>&rlen = *rlen_out, &clen = *clen_out;
+  rlen.assign(m, 0);
+  clen.assign(n, 0);
   std::vector<uint64_t> rsig(m), csig(n, 0);
   for (size_t e = 0; e < col.size(); ++e) {
     if (col[e] < 0 || col[e] >= n) {
@@ -304,16 +331,50 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
   order_by_key(m_eq, m - m_eq, rlen, rsig, L->perm_row.data() + m_eq);
   L->perm_col.resize(n);
   order_by_key(0, n, clen, csig, L->perm_col.data());
+  if (slice_offsets_of(rlen, L->perm_row, false, &L->k_off) >= 0 &&
+      slice_offsets_of(clen, L->perm_col, false, &L->t_off) >= 0)
+    return PDHG_OK;
+  // The order above pads rows of one kind to one length and slices to groups.  What
+  // only fits below 2^31 slots without that is ordered by length alone.
+  const auto by_length = [](std::vector<int32_t>* perm, int64_t first, int64_t last, const std::vector<int32_t>& len) {
+    std::iota(perm->begin() + first, perm->begin() + last, (int32_t)first);
+    std::stable_sort(perm->begin() + first, perm->begin() + last,
+                     [&](int32_t a, int32_t b) { return len[a] > len[b]; });
+  };
+  by_length(&L->perm_row, 0, m_eq, rlen);
+  by_length(&L->perm_row, m_eq, m, rlen);
+  by_length(&L->perm_col, 0, n, clen);
+  const char* over = slice_offsets_of(rlen, L->perm_row, true, &L->k_off) < 0   ? "K"
+                     : slice_offsets_of(clen, L->perm_col, true, &L->t_off) < 0 ? "K^T"
+                                                                                : nullptr;
+  if (!over) return PDHG_OK;
+  *err = std::string("padded nnz of ") + over + " exceeds 2^31";
+  return PDHG_ERR_UNSUPPORTED;
+}
+
+}  // namespace
+
+int count_slots(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& rp, const std::vector<int32_t>& col,
+                const std::vector<double>& val, int64_t* slots_k, int64_t* slots_kt, std::string* err) {
+  HostLayout L;
+  std::vector<int32_t> rlen, clen;
+  const int rc = order_layout(n, m, m_eq, rp, col, val, &L, &rlen, &clen, err);
+  if (rc != PDHG_OK) return rc;
+  *slots_k = L.k_off.back();
+  *slots_kt = L.t_off.back();
+  return PDHG_OK;
+}
+
+int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& rp,
+                 const std::vector<int32_t>& col, const std::vector<double>& val, HostLayout* L,
+                 std::string* err) {
+  std::vector<int32_t> rlen, clen;
+  const int rc = order_layout(n, m, m_eq, rp, col, val, L, &rlen, &clen, err);
+  if (rc != PDHG_OK) return rc;
   std::vector<int32_t> inv_row(m), inv_col(n);
   for (int64_t i = 0; i < m; ++i) inv_row[L->perm_row[i]] = (int32_t)i;
   for (int64_t j = 0; j < n; ++j) inv_col[L->perm_col[j]] = (int32_t)j;
 
-  // ---- K in sliced ELL over internal rows ----
-  const int64_t ks = slice_offsets_of(rlen, L->perm_row, &L->k_off);
-  if (ks < 0) {
-    *err = "padded nnz of K exceeds 2^31";
-    return PDHG_ERR_UNSUPPORTED;
-  }
   // ---- K^T in sliced ELL over internal columns (entries by ascending row) ----
   std::vector<int64_t> cptr(n + 1, 0);
   for (int64_t j = 0; j < n; ++j) cptr[j + 1] = cptr[j] + clen[j];
@@ -327,13 +388,8 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
         csrc[pos] = (int32_t)e;
       }
   }
-  const int64_t ts = slice_offsets_of(clen, L->perm_col, &L->t_off);
-  if (ts < 0) {
-    *err = "padded nnz of K^T exceeds 2^31";
-    return PDHG_ERR_UNSUPPORTED;
-  }
-  size_slots(L->k_off, &L->k_col, &L->k_src, &L->k_soff, &L->k_runs);
-  size_slots(L->t_off, &L->t_col, &L->t_src, &L->t_soff, &L->t_runs);
+  L->k_own = size_slots(L->k_off, &L->k_col, &L->k_src, &L->k_soff, &L->k_runs);
+  L->t_own = size_slots(L->t_off, &L->t_col, &L->t_src, &L->t_soff, &L->t_runs);
   // the two matrices side by side; nothing here allocates or throws
   const auto fill_k = [&]() noexcept {
     place_entries(

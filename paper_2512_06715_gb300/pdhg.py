@@ -88,6 +88,8 @@ _SIGS = {
     "pdhg_backward": ([C.c_void_p, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p], C.c_int),
     "pdhg_last_error": ([], C.c_char_p),
     "pdhg_polish": ([C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(pdhg_polish_result), C.c_void_p], C.c_int),
+    "pdhg_layout_slots": ([C.c_int64, C.c_int64, C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p,
+                           C.POINTER(C.c_int64), C.POINTER(C.c_int64)], C.c_int),
     "pdhg_prepare": ([C.c_void_p, C.c_void_p], C.c_int),
     "pdhg_get_scaling": ([C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p], C.c_int),
     "pdhg_apply_K": ([C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p], C.c_int),
@@ -283,6 +285,16 @@ class Workspace:
         _check(lib().pdhg_time_kernels(self.ws, precision, reps, C.byref(md), C.byref(ma), C.byref(bd),
                                        C.byref(ba), _stream_ptr(stream)), "pdhg_time_kernels")
         return dict(ms_dual=md.value, ms_adj=ma.value, bytes_dual=bd.value, bytes_adj=ba.value)
+
+
+def layout_slots(row_ptr, col, val, n: int, m_eq: int) -> tuple[int, int]:
+    """Value slots of K and K^T, padding included, that a workspace of this CSR would
+    hold (host arrays, no GPU work)."""
+    row_ptr, col, val = np.asarray(row_ptr, np.int64), np.asarray(col, np.int32), np.asarray(val, np.float64)
+    k, kt = C.c_int64(), C.c_int64()
+    _check(lib().pdhg_layout_slots(n, len(row_ptr) - 1, m_eq, row_ptr.ctypes.data, col.ctypes.data, val.ctypes.data,
+                                   C.byref(k), C.byref(kt)), "pdhg_layout_slots")
+    return k.value, kt.value
 
 
 def header_symbols() -> list[str]:
