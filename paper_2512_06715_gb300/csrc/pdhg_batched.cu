@@ -200,16 +200,18 @@ __device__ __forceinline__ void load_par(float* const (&v)[2], const int (&par)[
 
 __host__ __device__ __forceinline__ double* preg(double* p, int r) { return p + (size_t)r * 8192 * 64 * 20; }
 
-// Per-instance block reduction of NV values held by each lane for its
-// instances b = H lane + h; result written to part[block][b][k] by threads
-// b < BP.  smem: [warps][BP][NV].
-template <int BP, int NV, int WARPS>
-__device__ __forceinline__ void block_inst_sum(const double (&v)[BP / 32][NV], double* smem, double* out) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+// Per-instance block reduction of NV values held by each lane for its instances
+// b = first + step h: put_inst leaves them in smem [warps][BP][NV], sum_inst writes
+// the sums to part[block][b][k] by threads b < BP.
+template <int BP, int NV>
+__device__ __forceinline__ void put_inst(const double (&v)[BP / 32][NV], double* smem, int first, int step) {
 #pragma unroll
   for (int h = 0; h < BP / 32; ++h)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) smem[(wid * BP + lane * (BP / 32) + h) * NV + k] = v[h][k];
+    for (int k = 0; k < NV; ++k) smem[((threadIdx.x >> 5) * BP + first + step * h) * NV + k] = v[h][k];
+}
+template <int BP, int NV, int WARPS>
+__device__ __forceinline__ void sum_inst(const double* smem, double* out) {
   __syncthreads();
   if (threadIdx.x < BP) {
     const int b = threadIdx.x;
@@ -318,34 +320,46 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBThreads + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBThreads) >> 5;
-  float a_dy2[H], a_int[H], sigma[H], pw[H];
-  int par[H];
-  bool on[H], upd[H];
+  struct Lane {  // of the instances b = first + step h
+    float sigma[H], pw[H];
+    int par[H];
+    bool on[H], upd[H];
+  };
+  auto lane_state = [&](int first, int step) {
+    Lane s;
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    const int b = H * lane + h;
-    a_dy2[h] = a_int[h] = 0.f;
-    sigma[h] = s_sigma[b];
-    pw[h] = s_pw[b];
-    par[h] = s_par[b];
-    on[h] = s_act[b];
-    upd[h] = on[h] && pw[h] != 0.f;
-  }
-  // Where a lane's instances agree on what they do and on their buffers (always
-  // with one instance per lane; with two until a step of one is rejected) every
-  // access is one of the lane's pair; else they go one by one.  64 node LPs of 6049
-  // buses x 48 periods: 576 us in pairs (1.25 ms with K^T y' one by one, 1.03 now), of
-  // 455 us for the vectors alone at the copy bandwidth.
+    for (int h = 0; h < H; ++h) {
+      const int b = first + step * h;
+      s.sigma[h] = s_sigma[b];
+      s.pw[h] = s_pw[b];
+      s.par[h] = s_par[b];
+      s.on[h] = s_act[b];
+      s.upd[h] = s.on[h] && s.pw[h] != 0.f;
+    }
+    return s;
+  };
+  __shared__ double smem[kBWarps * BP * 2];
+  // Where all lanes' instances agree in pairs on what they do and on their buffers
+  // (always with one instance per lane; with two until a step of one is rejected, one
+  // ends, or B is odd) every access is one of a lane's pair (b = 2 lane + h); else
+  // each instance's are its own, a warp's contiguous (b = lane + 32 h).  64 node LPs of
+  // 6049 buses x 48 periods, K x' and K^T y': 545 and 448 us in pairs, 624 and 537 us one
+  // by one (708 and 612 us one by one with b = 2 lane + h), of 455 us for the vectors
+  // of K x' alone at the copy bandwidth.
   const int nq = (a.m + RW - 1) / RW;
-  auto sweep = [&](auto paired) {
+  auto sweep = [&](auto paired, const Lane& me) {
     constexpr int S = decltype(paired)::value ? H : 1;  // instances per access
     constexpr int N = H / S;                            // accesses per lane
+    const int at = S * lane;                            // access g: instances at + 32 g ...
+    float a_dy2[H], a_int[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) a_dy2[h] = a_int[h] = 0.f;
     const float *xg[N], *kxr[N], *yr[N];
     float *kxw[N], *yw[N];
 #pragma unroll
     for (int g = 0; g < N; ++g) {
-      const int p = par[g * S];
-      xg[g] = on[g * S] ? a.x[1 - p] + H * lane + g * S : nullptr;
+      const int p = me.par[g * S];
+      xg[g] = me.on[g * S] ? a.x[1 - p] + at + 32 * g : nullptr;
       kxr[g] = a.Kx[p];
       yr[g] = a.y[p];
       kxw[g] = a.Kx[1 - p];
@@ -369,12 +383,12 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
           for (int t = 0; t < S; ++t)
             ko[r][g][t] = yo[r][g][t] = qv[r][g][t] = lo[r][g][t] = yb[r][g][t] = acc[r][g][t] = 0.f;
           if (i < a.m && xg[g]) {
-            const size_t idx = (size_t)i * BP + H * lane + g * S;
+            const size_t idx = (size_t)i * BP + at + 32 * g;
             load_inst<S>(kxr[g], idx, ko[r][g]);
             load_inst<S>(yr[g], idx, yo[r][g]);
             load_inst<S>(a.qf, idx, qv[r][g]);
             if (i >= a.m_eq) load_inst<S>(a.ylf, idx, lo[r][g]);
-            if (upd[g * S]) load_inst<S>(a.ybar, idx, yb[r][g]);
+            if (me.upd[g * S]) load_inst<S>(a.ybar, idx, yb[r][g]);
           }
         }
       // entry k of the group's rows: RW adjacent slots (16 B aligned:
@@ -402,40 +416,42 @@ __global__ void __launch_bounds__(kBThreads) kb_dual(BArgs<BP> a) {
 #pragma unroll
         for (int g = 0; g < N; ++g) {
           if (!xg[g]) continue;
-          const size_t idx = (size_t)i * BP + H * lane + g * S;
+          const size_t idx = (size_t)i * BP + at + 32 * g;
           float vn[S], bn[S];
 #pragma unroll
           for (int t = 0; t < S; ++t) {
             const int h = g * S + t;
             float z = qv[r][g][t] - 2.f * acc[r][g][t];
             z = z + ko[r][g][t];
-            float v = yo[r][g][t] + sigma[h] * z;
+            float v = yo[r][g][t] + me.sigma[h] * z;
             if (i >= a.m_eq) v = fmaxf(v, lo[r][g][t]);
             vn[t] = v;
-            bn[t] = yb[r][g][t] + pw[h] * yo[r][g][t];
+            bn[t] = yb[r][g][t] + me.pw[h] * yo[r][g][t];
             const float dy = v - yo[r][g][t], dk = acc[r][g][t] - ko[r][g][t];
             a_dy2[h] += dy * dy;
             a_int[h] += dy * dk;
           }
           store_inst<S>(kxw[g], idx, acc[r][g]);
           store_inst<S>(yw[g], idx, vn);
-          if (upd[g * S]) store_inst<S>(a.ybar, idx, bn);
+          if (me.upd[g * S]) store_inst<S>(a.ybar, idx, bn);
         }
       }
     }
-  };
-  if (__all_sync(0xffffffffu, H == 1 || (par[0] == par[H - 1] && on[0] == on[H - 1] && upd[0] == upd[H - 1])))
-    sweep(std::true_type{});
-  else
-    sweep(std::false_type{});
-  __shared__ double smem[kBWarps * BP * 2];
-  double v[H][2];
+    double v[H][2];
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    v[h][0] = (double)a_dy2[h];
-    v[h][1] = (double)a_int[h];
-  }
-  block_inst_sum<BP, 2, kBWarps>(v, smem, a.part);
+    for (int h = 0; h < H; ++h) {
+      v[h][0] = (double)a_dy2[h];
+      v[h][1] = (double)a_int[h];
+    }
+    put_inst<BP, 2>(v, smem, at, S == H ? 1 : 32);
+  };
+  const Lane me = lane_state(H * lane, 1);
+  if (__all_sync(0xffffffffu,
+                 H == 1 || (me.par[0] == me.par[H - 1] && me.on[0] == me.on[H - 1] && me.upd[0] == me.upd[H - 1])))
+    sweep(std::true_type{}, me);
+  else
+    sweep(std::false_type{}, lane_state(lane, 32));
+  sum_inst<BP, 2, kBWarps>(smem, a.part);
   double tot[2];
   if (grid_inst_sum<BP, 2>(a.part, a.tier, smem, tot)) {
     double down = 0.0, up = 0.0;
@@ -498,30 +514,40 @@ __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * kBThreads + threadIdx.x) >> 5;
   const int nw = (gridDim.x * kBThreads) >> 5;
-  float a_dx2[H], tau[H], wl[H];
-  int par[H];
-  bool on[H], got[H], upd[H];  // active; new K^T y this attempt; the x-average moves
+  struct Lane {  // as in kb_dual
+    float tau[H], wl[H];
+    int par[H];
+    bool on[H], got[H], upd[H];  // active; new K^T y this attempt; the x-average moves
+  };
+  auto lane_state = [&](int first, int step) {
+    Lane s;
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    const int b = H * lane + h;
-    a_dx2[h] = 0.f;
-    tau[h] = s_tau[b];
-    wl[h] = s_wl[b];
-    par[h] = s_par[b];
-    on[h] = s_act[b];
-    got[h] = s_acc[b];
-    upd[h] = got[h] && wl[h] != 0.f;
-  }
+    for (int h = 0; h < H; ++h) {
+      const int b = first + step * h;
+      s.tau[h] = s_tau[b];
+      s.wl[h] = s_wl[b];
+      s.par[h] = s_par[b];
+      s.on[h] = s_act[b];
+      s.got[h] = s_acc[b];
+      s.upd[h] = s.got[h] && s.wl[h] != 0.f;
+    }
+    return s;
+  };
+  __shared__ double smem[kBWarps * BP];
   const int nq = (a.n + RW - 1) / RW;
-  auto sweep = [&](auto paired) {  // as in kb_dual
+  auto sweep = [&](auto paired, const Lane& me) {  // as in kb_dual
     constexpr int S = decltype(paired)::value ? H : 1;
     constexpr int N = H / S;
+    const int at = S * lane;
+    float a_dx2[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) a_dx2[h] = 0.f;
     const float *yg[N], *xr[N];
     float *kty[N], *xw[N];
 #pragma unroll
     for (int g = 0; g < N; ++g) {
-      const int p = par[g * S];
-      yg[g] = got[g * S] ? a.y[p] + H * lane + g * S : nullptr;
+      const int p = me.par[g * S];
+      yg[g] = me.got[g * S] ? a.y[p] + at + 32 * g : nullptr;
       xr[g] = a.x[p];
       xw[g] = a.x[1 - p];
       kty[g] = a.KTy[p];
@@ -541,14 +567,14 @@ __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
 #pragma unroll
           for (int t = 0; t < S; ++t)
             x0[r][g][t] = cv[r][g][t] = lv[r][g][t] = uv[r][g][t] = xb[r][g][t] = acc[r][g][t] = 0.f;
-          if (j < a.n && on[g * S]) {
-            const size_t idx = (size_t)j * BP + H * lane + g * S;
+          if (j < a.n && me.on[g * S]) {
+            const size_t idx = (size_t)j * BP + at + 32 * g;
             load_inst<S>(xr[g], idx, x0[r][g]);
             load_inst<S>(a.cf, idx, cv[r][g]);
             load_inst<S>(a.lf, idx, lv[r][g]);
             load_inst<S>(a.uf, idx, uv[r][g]);
             if (!yg[g]) load_inst<S>(kty[g], idx, acc[r][g]);  // the old K^T y
-            if (upd[g * S]) load_inst<S>(a.xbar, idx, xb[r][g]);
+            if (me.upd[g * S]) load_inst<S>(a.xbar, idx, xb[r][g]);
           }
         }
 #pragma unroll 2
@@ -573,36 +599,37 @@ __global__ void __launch_bounds__(kBThreads) kb_adjoint(BArgs<BP> a) {
         if (j >= a.n) continue;
 #pragma unroll
         for (int g = 0; g < N; ++g) {
-          if (!on[g * S]) continue;
-          const size_t idx = (size_t)j * BP + H * lane + g * S;
+          if (!me.on[g * S]) continue;
+          const size_t idx = (size_t)j * BP + at + 32 * g;
           float vn[S], bn[S];
 #pragma unroll
           for (int t = 0; t < S; ++t) {
             const int h = g * S + t;
-            bn[t] = xb[r][g][t] + wl[h] * x0[r][g][t];
-            float v = x0[r][g][t] - tau[h] * (cv[r][g][t] - acc[r][g][t]);
+            bn[t] = xb[r][g][t] + me.wl[h] * x0[r][g][t];
+            float v = x0[r][g][t] - me.tau[h] * (cv[r][g][t] - acc[r][g][t]);
             v = fminf(fmaxf(v, lv[r][g][t]), uv[r][g][t]);
             vn[t] = v;
             const float d = v - x0[r][g][t];
             a_dx2[h] += d * d;
           }
           if (yg[g]) store_inst<S>(kty[g], idx, acc[r][g]);
-          if (upd[g * S]) store_inst<S>(a.xbar, idx, bn);
+          if (me.upd[g * S]) store_inst<S>(a.xbar, idx, bn);
           store_inst<S>(xw[g], idx, vn);
         }
       }
     }
-  };
-  if (__all_sync(0xffffffffu, H == 1 || (par[0] == par[H - 1] && on[0] == on[H - 1] && got[0] == got[H - 1] &&
-                                         upd[0] == upd[H - 1])))
-    sweep(std::true_type{});
-  else
-    sweep(std::false_type{});
-  __shared__ double smem[kBWarps * BP];
-  double v[H][1];
+    double v[H][1];
 #pragma unroll
-  for (int h = 0; h < H; ++h) v[h][0] = (double)a_dx2[h];
-  block_inst_sum<BP, 1, kBWarps>(v, smem, a.part);
+    for (int h = 0; h < H; ++h) v[h][0] = (double)a_dx2[h];
+    put_inst<BP, 1>(v, smem, at, S == H ? 1 : 32);
+  };
+  const Lane me = lane_state(H * lane, 1);
+  if (H == 1 || __all_sync(0xffffffffu, me.par[0] == me.par[H - 1] && me.on[0] == me.on[H - 1] &&
+                                            me.got[0] == me.got[H - 1] && me.upd[0] == me.upd[H - 1]))
+    sweep(std::true_type{}, me);
+  else
+    sweep(std::false_type{}, lane_state(lane, 32));
+  sum_inst<BP, 1, kBWarps>(smem, a.part);
   double tot[1];
   if (grid_inst_sum<BP, 1>(a.part, a.tier, smem, tot)) {
     if (threadIdx.x < BP) {
@@ -812,7 +839,8 @@ __global__ void __launch_bounds__(kKktWarps * 32) kb_kkt_row(BArgs<BP> a, int in
     acc[h][kRowS + 1] *= idp2[h];
   }
   __shared__ double smem[kKktWarps * BP * 2 * kRowS];
-  block_inst_sum<BP, 2 * kRowS, kKktWarps>(acc, smem, preg(a.part, 1));
+  put_inst<BP, 2 * kRowS>(acc, smem, H * lane, 1);
+  sum_inst<BP, 2 * kRowS, kKktWarps>(smem, preg(a.part, 1));
 }
 
 template <int BP>
@@ -924,7 +952,8 @@ __global__ void __launch_bounds__(kKktWarps * 32) kb_kkt_col(BArgs<BP> a, int in
       acc[h][c * kColS + 3] *= idd[h];
     }
   __shared__ double smem[kKktWarps * BP * 2 * kColS];
-  block_inst_sum<BP, 2 * kColS, kKktWarps>(acc, smem, preg(a.part, 2));
+  put_inst<BP, 2 * kColS>(acc, smem, H * lane, 1);
+  sum_inst<BP, 2 * kColS, kKktWarps>(smem, preg(a.part, 2));
 }
 
 // Fixed-order totals of the check's partials, one block per instance (one block
