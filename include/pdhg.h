@@ -303,6 +303,14 @@ int pdhg_rescale_noalloc(const pdhg_problem *prob, int32_t ruiz_iters, int32_t p
 int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64_t *row_ptr, const int32_t *col,
                       const double *val, int64_t *slots_k, int64_t *slots_kt);
 
+/* Failures that the host makes up, to test how a workspace goes on after them.
+ *   PDHG_INJECT_RESIDENT_REFUSED, value 1: launches of the resident attempts (see
+ *   pdhg_opts.autotune) fail as if the driver refused them; 0: they are tried
+ *   again by workspaces that have not met a refusal (a workspace that has keeps
+ *   to the separate kernels). */
+#define PDHG_INJECT_RESIDENT_REFUSED 1
+int pdhg_inject(void *ws, int32_t what, int32_t value);
+
 /* Load the values and run the rescaling of a solve without iterating. */
 int pdhg_prepare(void *ws, void *stream);
 

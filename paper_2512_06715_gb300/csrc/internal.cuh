@@ -103,6 +103,7 @@ struct Tune {
 // each slice's entries lie in its block's shared memory.
 struct ResidentPlan {
   bool done = false, on = false, cluster = false;
+  bool refused = false;  // the driver would not launch it: the separate kernels from then on
   int grid = 0, warps = 0;
   size_t smem = 0;
   int32_t kcap = 0, tcap = 0, rcap = 0, ccap = 0;
@@ -145,6 +146,7 @@ struct Workspace {
   int grid_k = 0, grid_kt = 0, grid_vec = 0;
   Tune tune[2];  // [0] FP64, [1] FP32
   ResidentPlan resident[2];
+  bool inject_refusal = false;  // pdhg_inject
   std::vector<int32_t> koff_h, toff_h;  // slice offsets of K and K^T
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
@@ -205,7 +207,7 @@ template <class T>
 bool plan_resident(const std::vector<int32_t>& koff, const std::vector<int32_t>& toff, int sms,
                    ResidentPlan* pl, std::vector<int32_t>* kloc, std::vector<int32_t>* tloc);
 template <class T>
-void launch_resident(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_t s);
+cudaError_t launch_resident(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_t s);
 // chunks of consecutive slices with at most max_entries entries and max_slices
 // slices each; false if a single slice is larger
 bool build_chunks(const std::vector<int32_t>& off, std::vector<int32_t>* chunks, int max_entries,

@@ -177,18 +177,30 @@ static void run_adjoint(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
   launch_adjoint<T>(a, t.grid_adj, s, t.unroll_adj);
 }
 
-// The 64 attempts between two checks.
+// The 64 attempts between two checks; an error only if the resident launch is
+// refused (nothing has run then).
 template <class T>
-static void run_attempts(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
+static cudaError_t run_attempts(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
   const ResidentPlan& pl = w->resident[sizeof(T) == 8 ? 0 : 1];
-  if (pl.on) {
-    launch_resident<T>(a, pl, s);
-    return;
-  }
+  if (pl.on) return w->inject_refusal ? cudaErrorNotSupported : launch_resident<T>(a, pl, s);
   for (int k = 0; k < kCheckEvery; ++k) {
     run_dual<T>(w, a, s);
     run_adjoint<T>(w, a, s);
   }
+  return cudaSuccess;
+}
+
+// The driver refused the resident launch: the separate kernels take over, for good
+// (as overlap_refused), with launch shapes that have yet to be timed.
+template <class T>
+static void refuse_resident(Workspace* w) {
+  ResidentPlan& pl = w->resident[sizeof(T) == 8 ? 0 : 1];
+  Tune& t = w->tune[sizeof(T) == 8 ? 0 : 1];
+  cudaGetLastError();
+  g_err.clear();
+  pl.on = false;
+  pl.refused = true;
+  if (t.untimed) t.done = t.untimed = false;
 }
 
 // Decides once per precision whether the attempts run resident: the LP fits, and
@@ -197,7 +209,8 @@ template <class T>
 static int setup_resident(Workspace* w) {
   ResidentPlan& pl = w->resident[sizeof(T) == 8 ? 0 : 1];
   const pdhg_opts& o = w->opts;
-  const bool wanted = o.autotune && o.kernel_variant < 0 && o.kernel_grid == 0 && !o.launch_overlap;
+  const bool wanted =
+      !pl.refused && o.autotune && o.kernel_variant < 0 && o.kernel_grid == 0 && !o.launch_overlap;
   Tune& t = w->tune[sizeof(T) == 8 ? 0 : 1];
   if (!wanted) {
     pl.on = false;
@@ -320,20 +333,13 @@ static int autotune(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
 template <class T>
 static int build_graph_once(Workspace* w);
 
-// The solve graph; built with the resident attempts or with programmatic
-// dependent launches of the per-attempt kernels when enabled, and once more
-// without them if the driver refuses that graph.
+// The solve graph; built with programmatic dependent launches of the per-attempt
+// kernels when enabled, and once more without them if the driver refuses that graph.
 template <class T>
 static int build_graph(Workspace* w) {
   const int pi = sizeof(T) == 8 ? 0 : 1;
   if (w->graph_exec[pi]) return PDHG_OK;
   int rc = build_graph_once<T>(w);
-  if (rc != PDHG_OK && w->resident[pi].on) {
-    cudaGetLastError();
-    w->resident[pi].on = false;
-    g_err.clear();
-    rc = build_graph_once<T>(w);
-  }
   if (rc != PDHG_OK && w->opts.launch_overlap && !w->overlap_refused) {
     cudaGetLastError();
     w->overlap_refused = true;
@@ -343,13 +349,13 @@ static int build_graph(Workspace* w) {
   return rc;
 }
 
+// The graph's while loop over the attempts and the check, captured into its body.
 template <class T>
-static int build_graph_once(Workspace* w) {
+static cudaError_t capture_body(Workspace* w, cudaGraph_t g) {
   const int pi = sizeof(T) == 8 ? 0 : 1;
-  cudaGraph_t g = nullptr;
-  CK(cudaGraphCreate(&g, 0));
   cudaGraphConditionalHandle h;
-  CK(cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault));
+  cudaError_t e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) return e;
   // cudaGraphNodeParams has no default constructor: zeroed storage instead
   alignas(cudaGraphNodeParams) unsigned char cp_raw[sizeof(cudaGraphNodeParams)];
   std::memset(cp_raw, 0, sizeof(cp_raw));
@@ -359,26 +365,31 @@ static int build_graph_once(Workspace* w) {
   cp.conditional.type = cudaGraphCondTypeWhile;
   cp.conditional.size = 1;
   cudaGraphNode_t node;
-  CK(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp));
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  CK(cudaStreamBeginCaptureToGraph(w->cap_stream, body, nullptr, nullptr, 0,
-                                   cudaStreamCaptureModeThreadLocal));
+  if ((e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp)) != cudaSuccess) return e;
+  e = cudaStreamBeginCaptureToGraph(w->cap_stream, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                    cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
   IterArgs<T> a = make_args<T>(w);
   a.in_graph = 1;
   a.cond = (unsigned long long)h;
-  run_attempts<T>(w, a, w->cap_stream);
+  const cudaError_t launched = run_attempts<T>(w, a, w->cap_stream);
   launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->resident[pi].on, w->cap_stream);
   cudaGraph_t captured = nullptr;
-  cudaError_t e = cudaStreamEndCapture(w->cap_stream, &captured);
-  if (e != cudaSuccess) {
-    cudaGraphDestroy(g);
-    return fail(PDHG_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-  }
+  e = cudaStreamEndCapture(w->cap_stream, &captured);
+  return launched != cudaSuccess ? launched : e;
+}
+
+template <class T>
+static int build_graph_once(Workspace* w) {
+  const int pi = sizeof(T) == 8 ? 0 : 1;
+  cudaGraph_t g = nullptr;
+  CK(cudaGraphCreate(&g, 0));
+  cudaError_t e = capture_body<T>(w, g);
   cudaGraphExec_t ex = nullptr;
-  e = cudaGraphInstantiate(&ex, g, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
   if (e != cudaSuccess) {
     cudaGraphDestroy(g);
-    return fail(PDHG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    return fail(PDHG_ERR_CUDA, std::string("solve graph: ") + cudaGetErrorString(e));
   }
   w->graph[pi] = g;
   w->graph_exec[pi] = ex;
@@ -444,6 +455,7 @@ template <class T>
 static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* res,
                       cudaStream_t s) {
   const bool mixed = sizeof(T) == 4;
+  const int pi = mixed ? 1 : 0;
   int rc;
   if (mixed) {
     if ((rc = alloc_bufs(w, &w->b32)) != PDHG_OK) return rc;
@@ -531,13 +543,17 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
       ri.grow_exp = o.step_growth_exp;
       ri.infeas_eps = (mixed && o.infeas_tol > 0.0) ? std::max(o.infeas_tol, kFp32RayTol) : o.infeas_tol;
       ri.fold_every = o.ir_fold_checks;
-      if (r == 0 && !w->tune[mixed ? 1 : 0].done) {
-        launch_state_init(w->st, ri, w->scalars, s);
-        launch_init_iterates<T>(a, 0, s);
-        launch_adjoint<T>(a, w->grid_kt, s, 1);
-        if ((rc = autotune<T>(w, a, s)) != PDHG_OK) return rc;
+      for (;;) {
+        if (r == 0 && !w->tune[pi].done) {
+          launch_state_init(w->st, ri, w->scalars, s);
+          launch_init_iterates<T>(a, 0, s);
+          launch_adjoint<T>(a, w->grid_kt, s, 1);
+          if ((rc = autotune<T>(w, a, s)) != PDHG_OK) return rc;
+        }
+        if (o.host_loop || (rc = build_graph<T>(w)) == PDHG_OK) break;
+        if (!w->resident[pi].on) return rc;
+        refuse_resident<T>(w);
       }
-      if (!o.host_loop && (rc = build_graph<T>(w)) != PDHG_OK) return rc;
       launch_state_init(w->st, ri, w->scalars, s);
       launch_init_iterates<T>(a, 0, s);
       run_adjoint<T>(w, a, s);
@@ -548,14 +564,17 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
       // Same kernels as the graph body, launched from the host; the done flag
       // is read after every check (one host wait per 64 attempts).
       for (;;) {
-        run_attempts<T>(w, a, s);
-        launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->resident[mixed ? 1 : 0].on, s);
+        if (run_attempts<T>(w, a, s) != cudaSuccess) {
+          refuse_resident<T>(w);
+          CK(run_attempts<T>(w, a, s));
+        }
+        launch_check<T>(a, w->grid_k, w->grid_kt, 0, w->resident[pi].on, s);
         CK(cudaMemcpyAsync(w->st_host, w->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (w->st_host->done) break;
       }
     } else {
-      CK(cudaGraphLaunch(w->graph_exec[mixed ? 1 : 0], s));
+      CK(cudaGraphLaunch(w->graph_exec[pi], s));
     }
     launch_accumulate<T>(a, w->x_star, w->y_star, 0, s);
     CK(cudaMemcpyAsync(w->st_host, w->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
@@ -568,7 +587,7 @@ static int solve_impl(Workspace* w, double* x_out, double* y_out, pdhg_result* r
     accepted += h.accepted;
     restarts += h.restarts;
     checks += h.checks;
-    launches += h.checks * ((w->resident[mixed ? 1 : 0].on ? 1 : 2 * kCheckEvery + (mixed ? 1 : 0)) + 4) + 1;
+    launches += h.checks * ((w->resident[pi].on ? 1 : 2 * kCheckEvery + (mixed ? 1 : 0)) + 4) + 1;
     rounds = r;
     status = h.status;
     if (h.status != 0) break;  // optimal or a limit
@@ -859,6 +878,16 @@ extern "C" int pdhg_set_opts(void* ws, const pdhg_opts* opts) {
   drop_graphs(w);  // graphs bake the cancel and trace pointers in
   release_batched(w);
   return ensure_trace(w);
+}
+
+extern "C" int pdhg_inject(void* ws, int32_t what, int32_t value) {
+  g_err.clear();
+  if (!ws) return fail(PDHG_ERR_INVALID_ARG, "workspace is NULL");
+  Workspace* w = (Workspace*)ws;
+  if (what != PDHG_INJECT_RESIDENT_REFUSED) return fail(PDHG_ERR_INVALID_ARG, "unknown injection");
+  w->inject_refusal = value != 0;
+  drop_graphs(w);
+  return PDHG_OK;
 }
 
 extern "C" int pdhg_solve(void* ws, double* x_out, double* y_out, pdhg_result* res, void* stream) {

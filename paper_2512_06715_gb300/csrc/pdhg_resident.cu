@@ -561,18 +561,16 @@ bool plan_resident(const std::vector<int32_t>& koff, const std::vector<int32_t>&
 }
 
 template <class T>
-void launch_resident(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_t s) {
-  if (pl.cluster)
-    pl.warps == 32 ? res_launch<T, true, 32>(a, pl, s) : res_launch<T, true, 16>(a, pl, s);
-  else
-    pl.warps == 32 ? res_launch<T, false, 32>(a, pl, s) : res_launch<T, false, 16>(a, pl, s);
+cudaError_t launch_resident(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_t s) {
+  if (pl.cluster) return pl.warps == 32 ? res_launch<T, true, 32>(a, pl, s) : res_launch<T, true, 16>(a, pl, s);
+  return pl.warps == 32 ? res_launch<T, false, 32>(a, pl, s) : res_launch<T, false, 16>(a, pl, s);
 }
 
 template bool plan_resident<float>(const std::vector<int32_t>&, const std::vector<int32_t>&, int, ResidentPlan*,
                                    std::vector<int32_t>*, std::vector<int32_t>*);
 template bool plan_resident<double>(const std::vector<int32_t>&, const std::vector<int32_t>&, int, ResidentPlan*,
                                     std::vector<int32_t>*, std::vector<int32_t>*);
-template void launch_resident<float>(const IterArgs<float>&, const ResidentPlan&, cudaStream_t);
-template void launch_resident<double>(const IterArgs<double>&, const ResidentPlan&, cudaStream_t);
+template cudaError_t launch_resident<float>(const IterArgs<float>&, const ResidentPlan&, cudaStream_t);
+template cudaError_t launch_resident<double>(const IterArgs<double>&, const ResidentPlan&, cudaStream_t);
 
 }  // namespace ucpdhg

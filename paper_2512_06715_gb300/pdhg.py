@@ -17,6 +17,7 @@ ERRORS = {-1: "INVALID_ARG", -2: "CUDA", -3: "NUMERIC", -4: "TIMEOUT", -5: "UNSU
 STATUS = {0: "round", 1: "optimal", 2: "iteration_limit", 3: "time_limit", 4: "cancelled", 5: "numeric",
           6: "primal_infeasible", 7: "dual_infeasible"}
 PREC_FP64, PREC_MIXED = 0, 1
+INJECT_RESIDENT_REFUSED = 1
 
 
 class pdhg_problem(C.Structure):
@@ -90,6 +91,7 @@ _SIGS = {
     "pdhg_polish": ([C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(pdhg_polish_result), C.c_void_p], C.c_int),
     "pdhg_layout_slots": ([C.c_int64, C.c_int64, C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p,
                            C.POINTER(C.c_int64), C.POINTER(C.c_int64)], C.c_int),
+    "pdhg_inject": ([C.c_void_p, C.c_int32, C.c_int32], C.c_int),
     "pdhg_prepare": ([C.c_void_p, C.c_void_p], C.c_int),
     "pdhg_get_scaling": ([C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p], C.c_int),
     "pdhg_apply_K": ([C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p], C.c_int),
@@ -244,6 +246,10 @@ class Workspace:
         if d["status_name"] == "not_square":
             return None, None, d
         return x, y, d
+
+    def inject(self, what: int, value: int):
+        """A failure made up on the host (pdhg_inject)."""
+        _check(lib().pdhg_inject(self.ws, what, value), "pdhg_inject")
 
     def prepare(self, stream=None):
         _check(lib().pdhg_prepare(self.ws, _stream_ptr(stream)), "pdhg_prepare")
