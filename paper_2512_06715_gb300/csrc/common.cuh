@@ -40,7 +40,7 @@ constexpr int kTraceCheckCols = 12;  // values recorded per KKT check in the tra
 // Sliced ELL with 32-row slices over the internal (length-sorted) row order.
 // Entry k of row r = 32 s + lane sits at off[s] + 32 k + lane, so the warp
 // owning a slice reads each k-column with one coalesced 128 B / 256 B access.
-// Padding entries carry col = 0 and value 0.
+// Padding entries carry col = 0 and value -0.0, entries of the LP never -0.0.
 template <class T>
 struct SellView {
   const int32_t* off;  // [nslices + 1] element offsets (multiples of 32)
@@ -210,6 +210,11 @@ __device__ __forceinline__ bool non_zero(double v) {
   return ((unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v)) != 0;
 }
 __device__ __forceinline__ bool non_zero(float v) { return __float_as_uint(v) << 1 != 0; }
+// the value of a padding slot (SellView)
+__device__ __forceinline__ bool is_padding(double v) {
+  return (unsigned)__double2hiint(v) == 0x80000000u && __double2loint(v) == 0;
+}
+__device__ __forceinline__ bool is_padding(float v) { return __float_as_uint(v) == 0x80000000u; }
 __device__ __forceinline__ bool finite_bits(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }

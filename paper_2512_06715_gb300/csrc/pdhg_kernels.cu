@@ -65,8 +65,11 @@ __device__ __forceinline__ int2 run_words(const SellView<T>& A, const SliceSpan&
                                           : make_int2(0, (int)((unsigned)kSlice << kRunBits));
 }
 
-// E entries of each slice from k0 on; rw: the run words from k-column kw on.
-template <class T, int U, int E, int MODE, bool TWO, bool TAIL>
+// E entries of each slice from k0 on; rw: the run words from k-column kw on.  SKIP
+// leaves out padding slots, which gather what their neighbours' run leads to: times
+// their zero value that adds nothing to a sum unless it is infinite or a NaN, which
+// the caller's vector of a product may be.
+template <class T, int U, int E, int MODE, bool TWO, bool TAIL, bool SKIP = false>
 __device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan& g, int2 rw, int kw, int k0,
                                           int lane, const T* __restrict__ x1, const T* __restrict__ x2,
                                           T (&acc1)[U], T (&acc2)[U]) {
@@ -111,29 +114,30 @@ __device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan&
   for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int e = 0; e < E; ++e)
-      if (!TAIL || k0 + e < g.w) {
+      if ((!TAIL || k0 + e < g.w) && !(SKIP && is_padding(v[u][e]))) {
         acc1[u] += v[u][e] * __ldg(x1 + c[u][e]);
         if (TWO) acc2[u] += v[u][e] * __ldg(x2 + c[u][e]);
       }
 }
 
-template <class T, int U, int MODE, bool TWO>
+template <class T, int U, int MODE, bool TWO, bool SKIP>
 __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceSpan& g, int2 rw, int lane,
                                               const T* __restrict__ x1, const T* __restrict__ x2,
                                               T (&acc1)[U], T (&acc2)[U]) {
   if constexpr (U == 1) {
     if (g.w <= 2)
-      dot_chunk<T, U, 2, MODE, TWO, true>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
+      dot_chunk<T, U, 2, MODE, TWO, true, SKIP>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
     else
-      for (int k0 = 0; k0 < g.w; k0 += 4) dot_chunk<T, U, 4, MODE, TWO, true>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
+      for (int k0 = 0; k0 < g.w; k0 += 4)
+        dot_chunk<T, U, 4, MODE, TWO, true, SKIP>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
   } else {
     constexpr int W = 32 / U;  // a multiple of the chunks
     for (int kw = 0;;) {
       const int end = min(g.w, kw + W);
       int k0 = kw;
       for (; k0 + 2 <= end; k0 += 2)
-        dot_chunk<T, U, 2, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
-      if (k0 < end) dot_chunk<T, U, 1, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+        dot_chunk<T, U, 2, MODE, TWO, false, SKIP>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+      if (k0 < end) dot_chunk<T, U, 1, MODE, TWO, false, SKIP>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
       kw += W;
       if (kw >= g.w) break;
       rw = run_words<T, U>(A, g, kw, lane);
@@ -148,7 +152,7 @@ __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceS
 // compiled into the kernels for matrices with such groups (OWN): in the others it
 // would cost 1 % (FP32 K x' of the 6717-bus day 36.9 -> 37.2 us, its FP64 solve 73.6 ->
 // 74.4 ms).
-template <class T, int U, bool TWO>
+template <class T, int U, bool TWO, bool SKIP>
 __device__ __forceinline__ void sell_dot_own(const SellView<T>& A, int s0, int lane, const T* __restrict__ x1,
                                              const T* __restrict__ x2, T (&acc1)[U], T (&acc2)[U]) {
 #pragma unroll
@@ -157,30 +161,31 @@ __device__ __forceinline__ void sell_dot_own(const SellView<T>& A, int s0, int l
     T a1[1] = {0}, a2[1] = {0};
     int k0 = 0;
     for (; k0 + 8 <= g.w; k0 += 8)
-      dot_chunk<T, 1, 8, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
-    for (; k0 < g.w; ++k0) dot_chunk<T, 1, 1, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+      dot_chunk<T, 1, 8, kRunsNone, TWO, false, SKIP>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+    for (; k0 < g.w; ++k0)
+      dot_chunk<T, 1, 1, kRunsNone, TWO, false, SKIP>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
     acc1[u] = a1[0];
     acc2[u] = a2[0];
   }
 }
 
 // s0: the first of the U slices, g: their span.
-template <class T, int U, bool TWO, bool OWN>
+template <class T, int U, bool TWO, bool OWN, bool SKIP = false>
 __device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int s0, const SliceSpan& g, int2 rw, int lane,
                                              const T* __restrict__ x1, const T* __restrict__ x2,
                                              T (&acc1)[U], T (&acc2)[U]) {
 #pragma unroll
   for (int u = 0; u < U; ++u) acc1[u] = acc2[u] = 0;
   if (g.mode == kRunsOne)
-    sell_dot_mode<T, U, kRunsOne, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsOne, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsTwo)
-    sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsTwo, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsMixed)
-    sell_dot_mode<T, U, kRunsMixed, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsMixed, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (OWN && g.mode == kRunsOwn)
-    sell_dot_own<T, U, TWO>(A, s0, lane, x1, x2, acc1, acc2);
+    sell_dot_own<T, U, TWO, SKIP>(A, s0, lane, x1, x2, acc1, acc2);
   else
-    sell_dot_mode<T, U, kRunsNone, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsNone, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
 }
 
 template <class T, int U, int MINB, bool OWN = false>
@@ -616,7 +621,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __
     to[u] = perm && r < A.rows ? __ldg(perm + r) : r;
   }
   const SliceSpan g = slice_span<U>(slice_offsets<T, U>(A, s0));
-  sell_dot_pre<T, U, false, OWN>(A, s0, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
+  sell_dot_pre<T, U, false, OWN, true>(A, s0, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int r = (s0 + u) * kSlice + lane;

@@ -442,7 +442,8 @@ __global__ void k_load_vals(const int32_t* __restrict__ ksrc, const int32_t* __r
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nk + nt;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t e = t < nk ? ksrc[t] : tsrc[t - nk];
-    (t < nk ? kval : tval - nk)[t] = (e >= 0) ? csr[e] : 0.0;
+    const double v = e >= 0 ? csr[e] : 0.0;
+    (t < nk ? kval : tval - nk)[t] = e < 0 ? -0.0 : non_zero(v) ? v : 0.0;
   }
 }
 
