@@ -307,8 +307,13 @@ int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64_t *row_ptr
  *   PDHG_INJECT_RESIDENT_REFUSED, value 1: launches of the resident attempts (see
  *   pdhg_opts.autotune) fail as if the driver refused them; 0: they are tried
  *   again by workspaces that have not met a refusal (a workspace that has keeps
- *   to the separate kernels). */
+ *   to the separate kernels).
+ *   PDHG_INJECT_WAIT_POLLS, value >= 0: polls after which a block of the resident
+ *   attempts gives up waiting for the others (0: at once; the solve then ends with
+ *   PDHG_ERR_TIMEOUT); negative: the default, about a second's worth.  LPs of up to
+ *   16 blocks wait in a hardware barrier instead. */
 #define PDHG_INJECT_RESIDENT_REFUSED 1
+#define PDHG_INJECT_WAIT_POLLS 2
 int pdhg_inject(void *ws, int32_t what, int32_t value);
 
 /* Load the values and run the rescaling of a solve without iterating. */

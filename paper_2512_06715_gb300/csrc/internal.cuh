@@ -101,7 +101,9 @@ struct Tune {
 
 // 64 attempts in one launch (pdhg_resident.cu): blocks, shared memory, and where
 // each slice's entries lie in its block's shared memory.
+constexpr int kResWait = 1 << 21;  // polls before a block gives up (a second or so)
 struct ResidentPlan {
+  int polls = kResWait;
   bool done = false, on = false, cluster = false;
   bool refused = false;  // the driver would not launch it: the separate kernels from then on
   int grid = 0, warps = 0;

@@ -884,8 +884,12 @@ extern "C" int pdhg_inject(void* ws, int32_t what, int32_t value) {
   g_err.clear();
   if (!ws) return fail(PDHG_ERR_INVALID_ARG, "workspace is NULL");
   Workspace* w = (Workspace*)ws;
-  if (what != PDHG_INJECT_RESIDENT_REFUSED) return fail(PDHG_ERR_INVALID_ARG, "unknown injection");
-  w->inject_refusal = value != 0;
+  if (what == PDHG_INJECT_RESIDENT_REFUSED)
+    w->inject_refusal = value != 0;
+  else if (what == PDHG_INJECT_WAIT_POLLS)
+    w->resident[0].polls = w->resident[1].polls = value < 0 ? kResWait : value;
+  else
+    return fail(PDHG_ERR_INVALID_ARG, "unknown injection");
   drop_graphs(w);
   return PDHG_OK;
 }

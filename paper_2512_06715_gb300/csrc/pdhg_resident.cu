@@ -27,13 +27,13 @@ constexpr int kResCluster = 16;
 constexpr int kResBlocks = 160;  // most blocks of a cooperative launch (GB300: 152 SMs)
 constexpr int kResStates = 7;                  // vectors kept per row and per column
 constexpr size_t kResSmem = 223 * 1024;  // dynamic shared memory a block may take (227 KB less the static)
-constexpr int kResWait = 1 << 21;         // polls before a block gives up (a second or so)
 
 struct ResArgs {
   const int32_t* kloc;  // entry offset of each slice of K in its block's shared memory
   const int32_t* tloc;
   int32_t kcap, tcap;  // entries per block
   int32_t rcap, ccap;  // rows and columns per block
+  int32_t polls;       // of grid_barrier before a block gives up
 };
 
 __device__ __forceinline__ void cluster_barrier() {
@@ -45,10 +45,10 @@ __device__ __forceinline__ void cluster_barrier() {
 // arrivals.  False if it gave up.  A counter that all poll beats words with a tag
 // per block that all collect (17.2 against 20.0 us per attempt at 152 blocks:
 // 152 x 152 polled words cost more than the second round trip for the sums).
-__device__ __forceinline__ bool grid_barrier(uint32_t* counter, unsigned target) {
+__device__ __forceinline__ bool grid_barrier(uint32_t* counter, unsigned target, int polls) {
   __threadfence();
   atomicAdd(counter, 1u);
-  for (int it = 0; it < kResWait; ++it) {
+  for (int it = 0; it < polls; ++it) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
     if (v >= target) {
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_resident(IterArgs<T> a, ResAr
         if (lane == 0) step_factors(rs_, st);
         if constexpr (!CLUSTER) {
           // the block's y' is ordered before by the barrier in the block sum
-          if (lane == 0) ok = grid_barrier(&a.st->bar, target);
+          if (lane == 0) ok = grid_barrier(&a.st->bar, target, r.polls);
           __syncwarp();
           sum_parts<2, T>(gpart, G, lane, tot);
         }
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_resident(IterArgs<T> a, ResAr
             if (lane == 0) {
               __stcg(gpart + 4 * b + 2, acc[0]);
               target += (unsigned)G;
-              if (!grid_barrier(&a.st->bar, target)) abort_s = 1;
+              if (!grid_barrier(&a.st->bar, target, r.polls)) abort_s = 1;
             }
           }
           __syncthreads();
@@ -491,7 +491,7 @@ cudaError_t res_launch(const IterArgs<T>& a, const ResidentPlan& pl, cudaStream_
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const ResArgs r = {pl.kloc, pl.tloc, pl.kcap, pl.tcap, pl.rcap, pl.ccap};
+  const ResArgs r = {pl.kloc, pl.tloc, pl.kcap, pl.tcap, pl.rcap, pl.ccap, pl.polls};
   return cudaLaunchKernelEx(&cfg, k_resident<T, CLUSTER, WARPS>, a, r);
 }
 

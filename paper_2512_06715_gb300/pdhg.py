@@ -17,7 +17,7 @@ ERRORS = {-1: "INVALID_ARG", -2: "CUDA", -3: "NUMERIC", -4: "TIMEOUT", -5: "UNSU
 STATUS = {0: "round", 1: "optimal", 2: "iteration_limit", 3: "time_limit", 4: "cancelled", 5: "numeric",
           6: "primal_infeasible", 7: "dual_infeasible"}
 PREC_FP64, PREC_MIXED = 0, 1
-INJECT_RESIDENT_REFUSED = 1
+INJECT_RESIDENT_REFUSED, INJECT_WAIT_POLLS = 1, 2
 
 
 class pdhg_problem(C.Structure):
