@@ -58,6 +58,8 @@ struct SellView {
   const int32_t* soff;  // [nslices + 1]
   const int2* runs;     // [nnz_pad / 32]
   int32_t own;          // some groups are kRunsOwn
+  int32_t widest;       // entries per row of the widest slice
+  int32_t slots;        // nnz_pad
 };
 
 __device__ __forceinline__ int run_split(int2 r) { return (int)((unsigned)r.y >> kRunBits); }
@@ -218,6 +220,8 @@ __device__ __forceinline__ bool is_padding(float v) { return __float_as_uint(v) 
 __device__ __forceinline__ bool finite_bits(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
+
+__device__ __forceinline__ bool finite_bits(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
 
 // max as fmax gives it (the other operand where one is NaN) in integer
 // instructions: an FP64 compare holds the FP64 pipe (two lanes a clock) for 16 clocks

@@ -24,9 +24,16 @@ struct DevSell {
   int32_t nchunks2 = 0;
   int32_t* soff = nullptr;  // column runs (SellView)
   int32_t* runs = nullptr;
-  int32_t own = 0;  // some groups of slices have no common width
-  SellView<double> v64() const { return {off, col, val64, nslices, rows, soff, (const int2*)runs, own}; }
-  SellView<float> v32() const { return {off, col, val32, nslices, rows, soff, (const int2*)runs, own}; }
+  int32_t own = 0;     // some groups of slices have no common width
+  int32_t widest = 0;  // entries per row of the widest slice
+  SellView<double> v64() const { return view(val64); }
+  SellView<float> v32() const { return view(val32); }
+
+ private:
+  template <class T>
+  SellView<T> view(const T* val) const {
+    return {off, col, val, nslices, rows, soff, (const int2*)runs, own, widest, (int32_t)nnz_pad};
+  }
 };
 
 // Iterate buffers of one precision.
@@ -51,7 +58,7 @@ struct HostLayout {
   std::vector<int32_t> k_off, k_col, k_src;
   std::vector<int32_t> t_off, t_col, t_src;
   std::vector<int32_t> k_soff, k_runs, t_soff, t_runs;  // column runs (SellView)
-  int32_t k_own = 0, t_own = 0;                         // SellView::own
+  int32_t k_own = 0, t_own = 0, k_wide = 0, t_wide = 0;  // SellView::own, widest
 };
 
 int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>& row_ptr,

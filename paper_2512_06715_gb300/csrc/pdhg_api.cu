@@ -748,10 +748,12 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   w->K.rows = (int32_t)w->m;
   w->K.nnz_pad = L.k_col.size();
   w->K.own = L.k_own;
+  w->K.widest = L.k_wide;
   w->KT.nslices = (int32_t)(L.t_off.size() - 1);
   w->KT.rows = (int32_t)w->n;
   w->KT.nnz_pad = L.t_col.size();
   w->KT.own = L.t_own;
+  w->KT.widest = L.t_wide;
   std::vector<int32_t> kch, tch;
   if (build_chunks(L.k_off, &kch, kStageEntries, 1 << 30) && build_chunks(L.t_off, &tch, kStageEntries, 1 << 30)) {
     w->K.nchunks = (int32_t)kch.size() - 1;

@@ -65,11 +65,8 @@ __device__ __forceinline__ int2 run_words(const SellView<T>& A, const SliceSpan&
                                           : make_int2(0, (int)((unsigned)kSlice << kRunBits));
 }
 
-// E entries of each slice from k0 on; rw: the run words from k-column kw on.  SKIP
-// leaves out padding slots, which gather what their neighbours' run leads to: times
-// their zero value that adds nothing to a sum unless it is infinite or a NaN, which
-// the caller's vector of a product may be.
-template <class T, int U, int E, int MODE, bool TWO, bool TAIL, bool SKIP = false>
+// E entries of each slice from k0 on; rw: the run words from k-column kw on.
+template <class T, int U, int E, int MODE, bool TWO, bool TAIL>
 __device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan& g, int2 rw, int kw, int k0,
                                           int lane, const T* __restrict__ x1, const T* __restrict__ x2,
                                           T (&acc1)[U], T (&acc2)[U]) {
@@ -114,30 +111,30 @@ __device__ __forceinline__ void dot_chunk(const SellView<T>& A, const SliceSpan&
   for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int e = 0; e < E; ++e)
-      if ((!TAIL || k0 + e < g.w) && !(SKIP && is_padding(v[u][e]))) {
+      if (!TAIL || k0 + e < g.w) {
         acc1[u] += v[u][e] * __ldg(x1 + c[u][e]);
         if (TWO) acc2[u] += v[u][e] * __ldg(x2 + c[u][e]);
       }
 }
 
-template <class T, int U, int MODE, bool TWO, bool SKIP>
+template <class T, int U, int MODE, bool TWO>
 __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceSpan& g, int2 rw, int lane,
                                               const T* __restrict__ x1, const T* __restrict__ x2,
                                               T (&acc1)[U], T (&acc2)[U]) {
   if constexpr (U == 1) {
     if (g.w <= 2)
-      dot_chunk<T, U, 2, MODE, TWO, true, SKIP>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
+      dot_chunk<T, U, 2, MODE, TWO, true>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
     else
       for (int k0 = 0; k0 < g.w; k0 += 4)
-        dot_chunk<T, U, 4, MODE, TWO, true, SKIP>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
+        dot_chunk<T, U, 4, MODE, TWO, true>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
   } else {
     constexpr int W = 32 / U;  // a multiple of the chunks
     for (int kw = 0;;) {
       const int end = min(g.w, kw + W);
       int k0 = kw;
       for (; k0 + 2 <= end; k0 += 2)
-        dot_chunk<T, U, 2, MODE, TWO, false, SKIP>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
-      if (k0 < end) dot_chunk<T, U, 1, MODE, TWO, false, SKIP>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+        dot_chunk<T, U, 2, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
+      if (k0 < end) dot_chunk<T, U, 1, MODE, TWO, false>(A, g, rw, kw, k0, lane, x1, x2, acc1, acc2);
       kw += W;
       if (kw >= g.w) break;
       rw = run_words<T, U>(A, g, kw, lane);
@@ -152,7 +149,7 @@ __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceS
 // compiled into the kernels for matrices with such groups (OWN): in the others it
 // would cost 1 % (FP32 K x' of the 6717-bus day 36.9 -> 37.2 us, its FP64 solve 73.6 ->
 // 74.4 ms).
-template <class T, int U, bool TWO, bool SKIP>
+template <class T, int U, bool TWO>
 __device__ __forceinline__ void sell_dot_own(const SellView<T>& A, int s0, int lane, const T* __restrict__ x1,
                                              const T* __restrict__ x2, T (&acc1)[U], T (&acc2)[U]) {
 #pragma unroll
@@ -161,31 +158,31 @@ __device__ __forceinline__ void sell_dot_own(const SellView<T>& A, int s0, int l
     T a1[1] = {0}, a2[1] = {0};
     int k0 = 0;
     for (; k0 + 8 <= g.w; k0 += 8)
-      dot_chunk<T, 1, 8, kRunsNone, TWO, false, SKIP>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+      dot_chunk<T, 1, 8, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
     for (; k0 < g.w; ++k0)
-      dot_chunk<T, 1, 1, kRunsNone, TWO, false, SKIP>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+      dot_chunk<T, 1, 1, kRunsNone, TWO, false>(A, g, int2{}, 0, k0, lane, x1, x2, a1, a2);
     acc1[u] = a1[0];
     acc2[u] = a2[0];
   }
 }
 
 // s0: the first of the U slices, g: their span.
-template <class T, int U, bool TWO, bool OWN, bool SKIP = false>
+template <class T, int U, bool TWO, bool OWN>
 __device__ __forceinline__ void sell_dot_pre(const SellView<T>& A, int s0, const SliceSpan& g, int2 rw, int lane,
                                              const T* __restrict__ x1, const T* __restrict__ x2,
                                              T (&acc1)[U], T (&acc2)[U]) {
 #pragma unroll
   for (int u = 0; u < U; ++u) acc1[u] = acc2[u] = 0;
   if (g.mode == kRunsOne)
-    sell_dot_mode<T, U, kRunsOne, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsOne, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsTwo)
-    sell_dot_mode<T, U, kRunsTwo, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsTwo, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (g.mode == kRunsMixed)
-    sell_dot_mode<T, U, kRunsMixed, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsMixed, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
   else if (OWN && g.mode == kRunsOwn)
-    sell_dot_own<T, U, TWO, SKIP>(A, s0, lane, x1, x2, acc1, acc2);
+    sell_dot_own<T, U, TWO>(A, s0, lane, x1, x2, acc1, acc2);
   else
-    sell_dot_mode<T, U, kRunsNone, TWO, SKIP>(A, g, rw, lane, x1, x2, acc1, acc2);
+    sell_dot_mode<T, U, kRunsNone, TWO>(A, g, rw, lane, x1, x2, acc1, acc2);
 }
 
 template <class T, int U, int MINB, bool OWN = false>
@@ -603,13 +600,26 @@ __global__ void k_init_vectors(IterArgs<T> a) {
   }
 }
 
+// Product of one row without its padding slots.  They gather what their neighbours'
+// run leads to: times their zero that adds nothing to a sum unless it is infinite or a
+// NaN, as entries of a caller's vector may be.
+template <class T>
+__device__ __noinline__ T dot_entries(const T* val, const int32_t* col, int w, const T* x) {
+  T acc = 0;
+  for (int k = 0; k < w; ++k)
+    if (!is_padding(val[k * kSlice])) acc += val[k * kSlice] * x[col[k * kSlice]];
+  return acc;
+}
+
 // y = A x, or with perm the FP64 result in another order, out[perm[r]] = (A x)_r
-// (pdhg_apply_K: the unscrambling, and for FP32 the widening, in the same pass).
-// Two slices per warp, one pass over the matrix without a loop: a sweep this
-// short is all latency.
-template <class T, int U, bool OWN>
-__global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __restrict__ x, T* __restrict__ y,
-                                                      const int32_t* __restrict__ perm, double* __restrict__ out) {
+// (pdhg_apply_K: the unscrambling, and for FP32 the widening, in the same pass).  U
+// slices per warp, one pass over the matrix without a loop: a sweep this short is all
+// latency.  LONG (U = 1): sixteen unpredicated entries in flight from the explicit
+// indices, and the registers for them (three blocks per SM instead of five or more).
+template <class T, int U, bool LONG>
+__global__ void __launch_bounds__(kBlock, LONG ? 3 : U == 1 ? 8 : sizeof(T) == 4 ? 6 : 5)
+    k_spmv_into(SellView<T> A, const T* __restrict__ x, T* __restrict__ y, const int32_t* __restrict__ perm,
+                double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int s0 = ((blockIdx.x * kBlock + threadIdx.x) >> 5) * U;
   if (s0 >= A.nslices) return;
@@ -621,15 +631,26 @@ __global__ void __launch_bounds__(kBlock) k_spmv_into(SellView<T> A, const T* __
     to[u] = perm && r < A.rows ? __ldg(perm + r) : r;
   }
   const SliceSpan g = slice_span<U>(slice_offsets<T, U>(A, s0));
-  sell_dot_pre<T, U, false, OWN, true>(A, s0, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
+  if constexpr (LONG) {
+    acc[0] = 0;
+    int k0 = 0;
+    for (; k0 + 16 <= g.w; k0 += 16)
+      dot_chunk<T, 1, 16, kRunsNone, false, false>(A, g, int2{}, 0, k0, lane, x, x, acc, unused);
+    for (; k0 < g.w; k0 += 4)
+      dot_chunk<T, 1, 4, kRunsNone, false, true>(A, g, int2{}, 0, k0, lane, x, x, acc, unused);
+  } else {
+    sell_dot_pre<T, U, false, false>(A, s0, g, run_words<T, U>(A, g, 0, lane), lane, x, x, acc, unused);
+  }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int r = (s0 + u) * kSlice + lane;
     if (r < A.rows) {
+      const int o = g.o + u * g.w * kSlice + lane;
+      const T v = finite_bits(acc[u]) ? acc[u] : dot_entries<T>(A.val + o, A.col + o, g.w, x);
       if (perm)
-        out[to[u]] = (double)acc[u];
+        out[to[u]] = (double)v;
       else
-        y[r] = acc[u];
+        y[r] = v;
     }
   }
 }
@@ -710,12 +731,26 @@ static int vgrid(int64_t n) {
   return (int)(g < 1 ? 1 : g);
 }
 
+template <class T, int U, bool LONG>
+static void spmv_slices(const SellView<T>& A, const T* x, T* y, const int32_t* perm, double* out, cudaStream_t s) {
+  const int64_t warps = (A.nslices + U - 1) / U;
+  const unsigned grid = (unsigned)((warps + kWarps - 1) / kWarps);
+  k_spmv_into<T, U, LONG><<<grid < 1 ? 1 : grid, kBlock, 0, s>>>(A, x, y, perm, out);
+}
+
+// A slice is a serial chain of its warp, 0.27 us per entry of its rows in steps of two
+// at two slices a warp.  That outlasts the rest where the widest slice has more than
+// 1/65536 of the slots (LONG): K x of a transport LP (1600 rows of 700 and 900 entries)
+// 276 -> 117 us, of 20000 x 20000 with 200 entries a row 84 -> 47 us.  Elsewhere LONG
+// loses warps and the runs' short index reads: the 6717-bus day 68 -> 100 us.
 template <class T>
 static void spmv_any(const SellView<T>& A, const T* x, T* y, const int32_t* perm, double* out, cudaStream_t s) {
-  const int64_t warps = (A.nslices + 1) / 2;
-  const unsigned grid = (unsigned)((warps + kWarps - 1) / kWarps);
-  const auto kernel = A.own ? k_spmv_into<T, 2, true> : k_spmv_into<T, 2, false>;
-  kernel<<<grid < 1 ? 1 : grid, kBlock, 0, s>>>(A, x, y, perm, out);
+  if (A.widest >= 32 && (int64_t)A.widest * 65536 > (int64_t)A.slots)
+    spmv_slices<T, 1, true>(A, x, y, perm, out, s);
+  else if (A.own)
+    spmv_slices<T, 1, false>(A, x, y, perm, out, s);
+  else
+    spmv_slices<T, 2, false>(A, x, y, perm, out, s);
 }
 
 template <class T>

@@ -388,6 +388,13 @@ int build_layout(int64_t n, int64_t m, int64_t m_eq, const std::vector<int64_t>&
         csrc[pos] = (int32_t)e;
       }
   }
+  const auto widest = [](const std::vector<int32_t>& off) {
+    int32_t w = 0;
+    for (size_t t = 0; t + 1 < off.size(); ++t) w = std::max(w, (off[t + 1] - off[t]) / kSlice);
+    return w;
+  };
+  L->k_wide = widest(L->k_off);
+  L->t_wide = widest(L->t_off);
   L->k_own = size_slots(L->k_off, &L->k_col, &L->k_src, &L->k_soff, &L->k_runs);
   L->t_own = size_slots(L->t_off, &L->t_col, &L->t_src, &L->t_soff, &L->t_runs);
   // the two matrices side by side; nothing here allocates or throws

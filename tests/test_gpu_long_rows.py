@@ -74,3 +74,25 @@ def test_products(precision, tol):
         got = ws.apply_K(torch.as_tensor(v), transpose=transpose, precision=precision).cpu().numpy()
         assert (np.abs(got - A @ v) <= 64 * tol * (abs(A) @ np.abs(v) + 1e-300)).all()
     ws.close()
+
+
+def test_products_of_many_short_rows_and_a_longer_one():
+    """1.4 million rows of three entries and one of 60: a group with a width per slice in
+    a matrix too large for its widest slice to matter."""
+    from paper_2512_06715_gb300.pdhg import Workspace
+    m, n, w = 1_400_000, 1_000_000, 60
+    rng = np.random.default_rng(5)
+    col = np.concatenate([np.sort(rng.choice(n, w, replace=False)),
+                          (rng.integers(0, n - 3, m)[:, None] + np.arange(3)).ravel()]).astype(np.int32)
+    row_ptr = np.concatenate([[0], w + 3 * np.arange(m + 1)]).astype(np.int64)
+    val = rng.standard_normal(len(col))
+    ws = Workspace(row_ptr, col, val, np.ones(n), np.zeros(n), np.ones(n), np.zeros(m + 1), 0)
+    ws.prepare()
+    dr, dc = (d.cpu().numpy() for d in ws.scaling())
+    K = sp.diags(dr) @ sp.csr_matrix((val, col, row_ptr), shape=(m + 1, n)) @ sp.diags(dc)
+    for precision, tol in ((0, 1e-14), (1, 1e-6)):
+        for A, transpose in ((K, False), (K.T.tocsr(), True)):
+            v = rng.standard_normal(A.shape[1])
+            got = ws.apply_K(torch.as_tensor(v), transpose=transpose, precision=precision).cpu().numpy()
+            assert (np.abs(got - A @ v) <= 64 * tol * (abs(A) @ np.abs(v) + 1e-300)).all()
+    ws.close()
