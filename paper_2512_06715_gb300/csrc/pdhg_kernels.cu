@@ -124,7 +124,14 @@ __device__ __forceinline__ void sell_dot_mode(const SellView<T>& A, const SliceS
   if constexpr (U == 1) {
     if (g.w <= 2)
       dot_chunk<T, U, 2, MODE, TWO, true>(A, g, rw, 0, 0, lane, x1, x2, acc1, acc2);
-    else
+    else if (MODE == kRunsNone) {
+      // rows without runs may be long: eight unpredicated entries in flight (100000
+      // rows of 40 random entries, FP32: K^T y' 22.4 -> 19.3 us, K x' 37.1 -> 35.7)
+      int k0 = 0;
+      for (; k0 + 8 <= g.w; k0 += 8)
+        dot_chunk<T, U, 8, MODE, TWO, false>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
+      for (; k0 < g.w; k0 += 4) dot_chunk<T, U, 4, MODE, TWO, true>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
+    } else
       for (int k0 = 0; k0 < g.w; k0 += 4)
         dot_chunk<T, U, 4, MODE, TWO, true>(A, g, rw, 0, k0, lane, x1, x2, acc1, acc2);
   } else {
