@@ -404,7 +404,10 @@ __device__ __forceinline__ void staged_dot(const SellView<T>& A, const SliceStag
       a1[0] += st.v[e] * __ldg(x1 + st.c[e]);
       if (TWO) a2[0] += st.v[e] * __ldg(x2 + st.c[e]);
     }
-  for (int k0 = kStage; k0 < st.g.w; k0 += 4)
+  int k0 = kStage;
+  for (; k0 + 8 <= st.g.w; k0 += 8)
+    dot_chunk<T, 1, 8, kRunsNone, TWO, false>(A, st.g, int2{}, 0, k0, lane, x1, x2, a1, a2);
+  for (; k0 < st.g.w; k0 += 4)
     dot_chunk<T, 1, 4, kRunsNone, TWO, true>(A, st.g, int2{}, 0, k0, lane, x1, x2, a1, a2);
   acc1 = a1[0];
   acc2 = a2[0];
