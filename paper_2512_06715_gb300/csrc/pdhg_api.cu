@@ -268,7 +268,10 @@ static int autotune(Workspace* w, const IterArgs<T>& a, cudaStream_t s) {
   const bool staged = w->K.nchunks > 0 && w->KT.nchunks > 0 && staged_setup() == 0;
   const bool rowstaged = w->K.nchunks2 > 0 && w->KT.nchunks2 > 0 && rowstaged_setup() == 0;
   const bool ring = ring_setup() == 0;
-  const int unrolls[12] = {1, 2, 4, 0, 8, 9, 16, 17, 18, 19, 20, 21};
+  // Two slices first: a later candidate has to be 2 % faster, and one slice in FP64 ties
+  // with it (6717-bus day, 84.3 us both) but repeats less well in a solve (73.2 to 74.7
+  // ms from one workspace to the next against 73.4 to 73.5)
+  const int unrolls[12] = {2, 1, 4, 0, 8, 9, 16, 17, 18, 19, 20, 21};
   // grids beyond one resident wave let blocks that finish early take the
   // remaining slices (the sweeps' slices are spread round-robin over warps)
   const int bps[7] = {2, 3, 4, 6, 8, 12, 16};
