@@ -191,11 +191,12 @@ typedef struct pdhg_result {
 /* Fill *o with the defaults listed above. */
 int pdhg_opts_default(pdhg_opts *o);
 
-/* Create a workspace for `prob`.  Copies the sparsity structure to the host
- * once to build the internal row/column orderings and sliced-ELL layouts,
- * then allocates every device buffer a solve needs.  Values (val, c, l, u, q)
- * are read at each solve, so they may change between solves; the structure
- * and the pointers must stay valid and unchanged for the workspace's life.
+/* Create a workspace for `prob`.  Copies the CSR arrays (val too, which only
+ * guides the orderings) to the host once to build the internal row/column
+ * orderings and sliced-ELL layouts, then allocates every device buffer a solve
+ * needs.  Values (val, c, l, u, q) are read at each solve, so they may change
+ * between solves; the structure and the pointers must stay valid and unchanged
+ * for the workspace's life.
  * `opts` may be NULL (defaults).  Synchronises `stream`. */
 int pdhg_workspace_create(const pdhg_problem *prob, const pdhg_opts *opts, void **ws, void *stream);
 
@@ -327,7 +328,9 @@ int pdhg_get_scaling(void *ws, double *Dr, double *Dc, void *stream);
  * in [m], out [n]) with the rescaled matrix in the workspace's sliced-ELL
  * layout, original index order, device FP64 vectors.  precision selects the
  * FP64 or the FP32 copy of the values (FP32 rounds `in` to float first and
- * accumulates in FP32). */
+ * accumulates in FP32).  The FP32 copy is there after pdhg_prepare and after
+ * mixed-precision and batched solves; an FP64 solve leaves it out of date and
+ * PDHG_PREC_MIXED is refused until one of those. */
 int pdhg_apply_K(void *ws, int32_t transpose, int32_t precision, const double *in, double *out,
                  void *stream);
 

@@ -237,12 +237,6 @@ __device__ __forceinline__ double max_of(double v, double w) {
 }
 __device__ __forceinline__ float max_of(float v, float w) { return max(v, w); }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Warp totals of NV values: while values are left to split, each step hands half
 // of a lane's values to its partner and adds the other half, so 16 values take 16
 // additions instead of 80.  out[k] receives the total of v[k].
