@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <new>
 #include <string>
 
 #include "internal.cuh"
@@ -681,9 +682,9 @@ extern "C" int pdhg_opts_default(pdhg_opts* o) {
   return PDHG_OK;
 }
 
-extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* opts, void** out,
-                                     void* stream) {
-  g_err.clear();
+// *made: the workspace under construction, for the caller to release if this throws.
+static int create_workspace(const pdhg_problem* prob, const pdhg_opts* opts, void** out, void* stream,
+                            Workspace** made) {
   if (!out) return fail(PDHG_ERR_INVALID_ARG, "ws out-pointer is NULL");
   *out = nullptr;
   if (!prob) return fail(PDHG_ERR_INVALID_ARG, "problem is NULL");
@@ -703,7 +704,7 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   int rc = validate_opts(&o);
   if (rc != PDHG_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  Workspace* w = new Workspace();
+  Workspace* w = *made = new Workspace();
   w->prob = *prob;
   w->opts = o;
   w->n = prob->n;
@@ -711,6 +712,7 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   w->m_eq = prob->m_eq;
   w->nnz = prob->nnz;
   auto bail = [&](int code) {
+    *made = nullptr;
     release(w);
     delete w;
     return code;
@@ -839,8 +841,23 @@ extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* 
   return PDHG_OK;
 }
 
+extern "C" int pdhg_workspace_create(const pdhg_problem* prob, const pdhg_opts* opts, void** out,
+                                     void* stream) {
+  g_err.clear();
+  Workspace* made = nullptr;
+  try {
+    return create_workspace(prob, opts, out, stream, &made);
+  } catch (const std::bad_alloc&) {
+    if (made) {
+      release(made);
+      delete made;
+    }
+    return fail(PDHG_ERR_NOMEM, "host allocation failed");
+  }
+}
+
 extern "C" int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64_t* row_ptr, const int32_t* col,
-                                 const double* val, int64_t* slots_k, int64_t* slots_kt) {
+                                 const double* val, int64_t* slots_k, int64_t* slots_kt) try {
   g_err.clear();
   if (!row_ptr || !slots_k || !slots_kt) return fail(PDHG_ERR_INVALID_ARG, "NULL argument");
   if (n < 1 || m < 1 || m_eq < 0 || m_eq > m || n >= ((int64_t)1 << 31) - 64 || m >= ((int64_t)1 << 31) - 64)
@@ -855,6 +872,8 @@ extern "C" int pdhg_layout_slots(int64_t n, int64_t m, int64_t m_eq, const int64
   const int rc = count_slots(n, m, m_eq, rp, std::vector<int32_t>(col, col + nnz),
                              std::vector<double>(val, val + nnz), slots_k, slots_kt, &err);
   return rc == PDHG_OK ? rc : fail(rc, err);
+} catch (const std::bad_alloc&) {
+  return fail(PDHG_ERR_NOMEM, "host allocation failed");
 }
 
 static void drop_graphs(Workspace* w) {

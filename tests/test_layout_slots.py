@@ -54,3 +54,27 @@ def test_a_row_of_17_million_entries():
     col = np.concatenate([np.arange(n, dtype=np.int32), np.array([3, 5, 3, 7], np.int32)])
     k, _ = layout_slots(row_ptr, col, np.ones(n + 4), n, 0)
     assert k <= 32 * n + 4096
+
+
+def test_a_failed_host_allocation_is_an_error_code():
+    """In a process whose address space is nearly used up: an exception must not leave
+    the C entry."""
+    import subprocess
+    import sys
+    code = """
+import resource
+import numpy as np
+from paper_2512_06715_gb300.pdhg import PDHGError, layout_slots
+n = 4_000_000
+row_ptr, col, val = np.array([0, n], np.int64), np.arange(n, dtype=np.int32), np.ones(n)
+layout_slots(row_ptr[:1].repeat(2), col, val, n, 0)  # loads the library
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (60 << 20),) * 2)
+try:
+    layout_slots(row_ptr, col, val, n, 0)
+except PDHGError as e:
+    assert "NOMEM" in str(e), e
+else:
+    raise SystemExit("no error")
+"""
+    assert subprocess.run([sys.executable, "-c", code], timeout=120).returncode == 0
